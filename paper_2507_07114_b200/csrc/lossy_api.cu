@@ -8,7 +8,9 @@
 
 #include <mutex>
 #include <new>
+#include <type_traits>
 
+#include "lossy_diag.cuh"
 #include "lossy_gather.cuh"
 #include "lossy_phase_tma.cuh"
 
@@ -690,6 +692,34 @@ int run_phase(lossy_ctx* ctx, const Params& P, float* norms, double* sumsq, cuda
   return LOSSY_OK;
 }
 
+// One block per SM, of as many warps as their tables and slots leave room for; fewer blocks when there are not as many
+// chunks as warps.
+template <class RT, bool ELIDE, class M>
+cudaError_t launch_pairwise(lossy_ctx* ctx, const PairwiseArgs& A, cudaStream_t s) {
+  auto kern = drift_pairwise_kernel<RT, ELIDE, M>;
+  const uint32_t wb = pair_warp_bytes(A.W, sizeof(typename RT::raw));
+  const uint32_t room = (uint32_t)ctx->smem_optin;
+  uint32_t warps = room / wb;
+  if (warps > (uint32_t)PairShape<M>::kMaxWarps) warps = PairShape<M>::kMaxWarps;
+  if (warps == 0) return cudaErrorInvalidConfiguration;
+  static bool opted_in[kMaxDevices];   // per kernel instantiation and device: raise the dynamic shared memory limit once
+  {
+    std::lock_guard<std::mutex> lock(g_setup_mu);
+    if (ctx->device >= kMaxDevices || !opted_in[ctx->device]) {
+      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room);
+      if (e != cudaSuccess) return e;
+      if (ctx->device < kMaxDevices) opted_in[ctx->device] = true;
+    }
+  }
+  const uint64_t chunks = (uint64_t)A.segs * A.chunks_per_seg;
+  // (a small bucket spreads its chunks over the SMs rather than filling a few of them)
+  if (chunks < (uint64_t)ctx->num_sms * warps) warps = (uint32_t)((chunks + ctx->num_sms - 1) / ctx->num_sms);
+  uint64_t blocks = (chunks + warps - 1) / warps;
+  if (blocks > (uint64_t)ctx->num_sms) blocks = ctx->num_sms;
+  kern<<<(uint32_t)blocks, warps * 32u, warps * wb, s>>>(A);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
 extern "C" {
@@ -787,12 +817,21 @@ int lossy_packet_sqnorms(lossy_ctx* ctx, const void* const* grads, float* out, v
   A.W = ctx->cfg.W;
   A.P = ctx->cfg.packet_elems;
   A.K = (uint32_t)ctx->K;
-  uint64_t blocks = ((uint64_t)A.W * A.K + 7) / 8;
-  const uint64_t cap = (uint64_t)ctx->num_sms * 8;
+  // pieces of at most one chunk: kSqLoads of them per warp at a time (one vector each), else one piece per warp
+  const bool many = A.P <= (uint32_t)kChunk;
+  const uint64_t tasks = many ? ((uint64_t)A.K + kSqLoads - 1) / kSqLoads : A.K;
+  uint64_t blocks = (tasks + 7) / 8;
+  const uint64_t cap = ((uint64_t)ctx->num_sms * 8 + A.W - 1) / A.W;
   if (blocks > cap) blocks = cap;
+  const dim3 grid((uint32_t)blocks, A.W);
   cudaStream_t s = (cudaStream_t)stream;
-  if (ctx->cfg.grad_dtype == LOSSY_BF16) packet_sqnorms_kernel<BF16><<<(uint32_t)blocks, 256, 0, s>>>(A);
-  else packet_sqnorms_kernel<F32><<<(uint32_t)blocks, 256, 0, s>>>(A);
+  if (ctx->cfg.grad_dtype == LOSSY_BF16) {
+    if (many) packet_sqnorms_kernel<BF16, true><<<grid, 256, 0, s>>>(A);
+    else packet_sqnorms_kernel<BF16, false><<<grid, 256, 0, s>>>(A);
+  } else {
+    if (many) packet_sqnorms_kernel<F32, true><<<grid, 256, 0, s>>>(A);
+    else packet_sqnorms_kernel<F32, false><<<grid, 256, 0, s>>>(A);
+  }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail_cuda(ctx, "packet norm launch", e);
   ctx->launches++;
@@ -995,24 +1034,26 @@ int drift_pairwise(lossy_ctx* ctx, const void* const* replicas, double* d2, void
   A.d2 = d2;
   A.n = ctx->cfg.n;
   A.W = ctx->cfg.W;
-  A.nblk = (ctx->cfg.W + 3) / 4;
-  if (ctx->cfg.flags & LOSSY_REPLICA_SKIP_OWNER) {
-    A.elide = 1u;
-    A.P = ctx->cfg.packet_elems;
-    A.pps = ctx->pps;
-    A.k0 = (uint32_t)ctx->cfg.shard_packet0;
-    for (uint32_t i = 0; i < ctx->cfg.W; ++i) A.rep_skip[i] = own_elems(ctx, i);
+  const lossy_config& c = ctx->cfg;
+  A.segs = 1;
+  A.seg_len = c.n;
+  if (c.flags & LOSSY_REPLICA_SKIP_OWNER) {
+    A.seg_len = (uint64_t)ctx->pps * c.packet_elems;
+    A.seg_off = c.shard_packet0 * c.packet_elems;
+    A.seg0 = (uint32_t)(c.shard_packet0 / ctx->pps);
+    A.segs = (uint32_t)((c.shard_packet0 + ctx->K - 1) / ctx->pps) - A.seg0 + 1u;
+    for (uint32_t i = 0; i < c.W; ++i) A.rep_skip[i] = own_elems(ctx, i);
   }
-  const uint32_t pairs = A.nblk * (A.nblk + 1) / 2;
-  const uint64_t nvec = (A.n + 7) / 8;
-  uint64_t bx = (nvec + 255) / 256;
-  const uint64_t cap = (uint64_t)ctx->num_sms * 4;
-  if (bx > cap) bx = cap;
-  const dim3 grid((uint32_t)bx, pairs);
+  const uint64_t longest = A.seg_len < c.n ? A.seg_len : c.n;
+  A.chunks_per_seg = (uint32_t)((longest + kChunk - 1) / kChunk);
   cudaStream_t s = (cudaStream_t)stream;
-  if (ctx->cfg.replica_dtype == LOSSY_BF16) drift_pairwise_kernel<BF16><<<grid, 256, 0, s>>>(A);
-  else drift_pairwise_kernel<F32><<<grid, 256, 0, s>>>(A);
-  cudaError_t e = cudaGetLastError();
+  const bool bf16 = c.replica_dtype == LOSSY_BF16, small = c.W <= 32u;
+  auto pick = [&](auto elide) {
+    constexpr bool E = decltype(elide)::value;
+    return bf16 ? (small ? launch_pairwise<BF16, E, uint32_t>(ctx, A, s) : launch_pairwise<BF16, E, uint64_t>(ctx, A, s))
+                : (small ? launch_pairwise<F32, E, uint32_t>(ctx, A, s) : launch_pairwise<F32, E, uint64_t>(ctx, A, s));
+  };
+  const cudaError_t e = c.flags & LOSSY_REPLICA_SKIP_OWNER ? pick(std::true_type{}) : pick(std::false_type{});
   if (e != cudaSuccess) return fail_cuda(ctx, "pairwise drift launch", e);
   ctx->launches++;
   return LOSSY_OK;

@@ -271,13 +271,13 @@ __device__ __forceinline__ float warp_sum(float x) {
   return x;
 }
 
-// Warp totals of N (4 or 8) per-lane values at once. Each exchange (lane distance 16, 8, ...) halves the
+// Warp totals of N (2, 4 or 8) per-lane values at once. Each exchange (lane distance 16, 8, ...) halves the
 // values a lane carries: the lanes whose bit is set keep the upper half and hand over the lower half. The
 // one value left is then summed over the remaining lane bits, so every lane ends with the warp total of
-// value number lane / (32 / N), in N + 1 (N = 8) or N + 2 (N = 4) shuffles instead of 5 N.
+// value number lane / (32 / N), in N + 1 (N = 8), N + 2 (N = 4) or N + 3 (N = 2) shuffles instead of 5 N.
 template <int N>
 __device__ __forceinline__ float warp_sum_multi(float (&v)[N], int lane) {
-  static_assert(N == 4 || N == 8, "4 or 8 values");
+  static_assert(N == 2 || N == 4 || N == 8, "2, 4 or 8 values");
   constexpr unsigned kFull = 0xFFFFFFFFu;
   int o = 16;
 #pragma unroll

@@ -60,3 +60,54 @@ def test_pair_constant_of_the_theorem_at_scale():
                 continue
             want = sigma2 * ((n - own[i] - own[k]) * 2 * p / (1 - p * p) + (own[i] + own[k]) * p / (1 - p))
             assert abs(got[i, k] / want - 1) < 0.03, (i, k, got[i, k] / want)
+
+
+def _against_fp64(W, n, P, dtype, copies, elided=False):
+    """drift_pairwise of the given full copies (elided: without each owner's shard) next to the same differences in fp64."""
+    flags = L.LOSSY_REPLICA_SKIP_OWNER if elided else 0
+    ctx = L.lossy_init(W=W, n=n, packet_elems=P, p_grad=0.1, p_param=0.1, seed=1, grad_dtype=dtype, replica_dtype=dtype,
+                       optimizer="sgd", lr=0.1, flags=flags)
+    K = -(-n // P)
+    pps = -(-K // W)
+    owner = torch.arange(n, device="cuda") // (pps * P)
+    held = [c[owner != i] if elided else c for i, c in enumerate(copies)]
+    d2 = torch.zeros(W * W, dtype=torch.float64, device="cuda")
+    L.drift_pairwise(ctx, [h if h.numel() else torch.zeros(8, dtype=dtype, device="cuda") for h in held], d2)
+    torch.cuda.synchronize()
+    L.lossy_destroy(ctx)
+    R = torch.stack(copies).double()
+    want = torch.zeros(W, W, dtype=torch.float64, device="cuda")
+    for i in range(W):
+        for k in range(W):
+            sq = (R[i] - R[k]) ** 2
+            want[i, k] = (sq[(owner != i) & (owner != k)] if elided else sq).sum()
+    return d2.view(W, W), want
+
+
+@pytest.mark.parametrize("W,n,P", [(1, 100, 8), (2, 256 * 9 + 3, 64), (3, 45, 8), (16, 100_003, 736), (46, 9000, 128), (64, 30_011, 512)])
+@pytest.mark.parametrize("late", [0.0, 0.2, 0.7, 1.0])
+@pytest.mark.parametrize("elided", [False, True])
+def test_pairwise_for_any_share_of_differing_copies(W, n, P, late, elided):
+    """From all copies equal to all distinct, also where the copy compared first is in the minority. A pair's fp32 partial
+    sums have 8 terms per lane and five tree levels: each rounds by at most 2^-24, so 13 * 2^-24 < 1e-6."""
+    torch.manual_seed(W)
+    for dtype in (torch.bfloat16, torch.float32):
+        base = torch.randn(n, device="cuda") * 0.02
+        miss = (torch.rand(W, -(-n // P), device="cuda") < late).repeat_interleave(P, 1)[:, :n]
+        copies = [(base + 1e-3 * torch.randn(n, device="cuda") * miss[i]).to(dtype) for i in range(W)]
+        got, want = _against_fp64(W, n, P, dtype, copies, elided)
+        assert torch.all(got[want == 0] == 0)
+        assert torch.all((got - want).abs() <= 1e-6 * want)
+
+
+def test_pairwise_keeps_infinities_and_nan():
+    """Equal infinities differ by NaN, also on the diagonal, as the differences themselves say."""
+    W, n, P = 6, 3000, 256
+    base = torch.randn(n, device="cuda")
+    copies = [base.clone() for _ in range(W)]
+    copies[0][17] = copies[1][17] = float("inf")
+    copies[2][2999] = float("nan")
+    copies[3][300] = float("-inf")
+    got, want = _against_fp64(W, n, P, torch.float32, copies)
+    assert torch.equal(got.isnan(), want.isnan()) and torch.equal(got.isinf(), want.isinf())
+    assert want.isnan().any() and torch.equal(got[want == 0], want[want == 0])

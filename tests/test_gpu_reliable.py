@@ -53,3 +53,22 @@ def test_importance_classes_by_gradient_norm(case, mode):
     assert_same(to_np(gpu.master), orc.master, "master bits")
     L.lossy_set_reliable(gpu.ctx, None)
     L.lossy_device_status(gpu.ctx)
+
+
+@pytest.mark.parametrize("P", [8, 128, 248, 256, 264, 1024, 1032, 2048, 2056])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_packet_norms_at_the_edges_of_chunks_and_batches(P, dtype):
+    """One to four vectors per lane, pieces shorter than a chunk, a count of pieces that is no multiple of four, a short
+    last piece; fp32 sums of at most 9 * 8 terms per lane and five tree levels: 77 * 2^-24 < 5e-6."""
+    W, n = 3, 5 * P + 3
+    K = 6
+    ctx = L.lossy_init(W=W, n=n, packet_elems=P, p_grad=0.1, p_param=0.1, seed=1, grad_dtype=dtype, replica_dtype=dtype,
+                       optimizer="sgd", lr=0.1)
+    torch.manual_seed(P)
+    g = [torch.randn(n, device="cuda").to(dtype) for _ in range(W)]
+    sq = torch.full((W * K,), -1.0, device="cuda")
+    L.lossy_packet_sqnorms(ctx, g, sq)
+    torch.cuda.synchronize()
+    L.lossy_destroy(ctx)
+    want = torch.stack([torch.nn.functional.pad(x.double() ** 2, (0, K * P - n)).view(K, P).sum(1) for x in g]).view(-1)
+    assert torch.all((sq.double() - want).abs() <= 5e-6 * want)
