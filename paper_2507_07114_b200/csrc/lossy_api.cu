@@ -287,21 +287,27 @@ int try_tma(lossy_ctx* ctx, const Params& P, bool drift, cudaStream_t s, uint32_
 
 // ---- gather pipeline (packets shorter than a tile) ------------------------------------------
 // barriers, the ring of tile masks, stage headers; the drift sums per compute warp, the wire ring and the stages follow
-constexpr uint32_t kGatherSmemFixed = kGatherBarBytes + kGatherRing * sizeof(TileMasks) + kGatherMaxStages * sizeof(StageHdr);
+template <bool ANY> constexpr uint32_t kGatherSmemFixed =
+    kGatherBarBytes + kGatherRing * sizeof(TileMasks<ANY ? kAnySub : kMaxSub>) + kGatherMaxStages * sizeof(StageHdr);
 
 // rd: the stale copies are read outside the compute warps (twin geometry: by the replica warps, one replica each;
 // wide geometry: by drift warps of their own)
-template <int CW>
+template <int CW, bool ANY>
 bool gather_geometry(const lossy_ctx* ctx, bool rd, TmaGeom& G) {
   constexpr uint32_t kTile = GatherShape<CW>::kTile;
   const lossy_config& c = ctx->cfg;
   const uint64_t kfull = c.n / c.packet_elems;               // packets that are complete
   if (kfull == 0 || kfull >= (1ull << 31)) return false;
-  // whole packets per tile: powers of two from 128 elements that divide the tile, at most kMaxSub of them
+  // !ANY: packets that divide the tile (powers of two), kMaxSub of them at most. ANY: all others, short or long, laid
+  // over the tiles as they come (multiples of 8 elements), from 128 elements (a compute warp's 128 elements then lie in
+  // at most two packets) and as long as a tile touches at most kAnySub of them.
   const uint32_t P = c.packet_elems;
-  if (P >= kTile || (P & (P - 1u)) != 0 || P < 128u || kTile / P > (uint32_t)kMaxSub) return false;
+  if (P < 128u || P >= (1u << 15) || ANY != (kTile % P != 0) || (!ANY && P >= kTile)) return false;
+  const uint32_t touched = ANY ? (P - 8u + kTile - 1u) / P + 1u : kTile / P;
+  if (touched > (uint32_t)(ANY ? kAnySub : kMaxSub)) return false;
   memset(&G, 0, sizeof G);
-  G.packets_per_tile = kTile / P;
+  G.packets_per_tile = touched;
+  G.magic = (uint32_t)(((1ull << 32) + P - 1u) / P);
   G.full_packets = (uint32_t)kfull;
   const uint32_t gb = c.grad_dtype == LOSSY_BF16 ? 2 : 4, rb = c.replica_dtype == LOSSY_BF16 ? 2 : 4;
   G.grad_slots = c.W < 8u ? c.W : 8u;
@@ -321,19 +327,19 @@ bool gather_geometry(const lossy_ctx* ctx, bool rd, TmaGeom& G) {
   }
   const uint32_t budget = (227u * 1024u) / GatherShape<CW>::kCtasPerSm - 1024u;
   const uint32_t avail = (uint32_t)ctx->smem_optin < budget ? (uint32_t)ctx->smem_optin : budget;
-  if (avail < kGatherSmemFixed + G.state_bytes + 2 * G.stage_bytes) return false;
-  G.stages = (avail - kGatherSmemFixed - G.state_bytes) / G.stage_bytes;
+  if (avail < kGatherSmemFixed<ANY> + G.state_bytes + 2 * G.stage_bytes) return false;
+  G.stages = (avail - kGatherSmemFixed<ANY> - G.state_bytes) / G.stage_bytes;
   if (G.stages > 4u) G.stages = 4u;                           // more measured no faster (W = 2..32)
   if (rd && GatherShape<CW, true>::kDriftWarps) {
     // wide: what the stages leave goes to the scratch, up to every chunk of a drift warp's replicas
-    const uint32_t left = avail - kGatherSmemFixed - G.state_bytes - G.stages * G.stage_bytes;
+    const uint32_t left = avail - kGatherSmemFixed<ANY> - G.state_bytes - G.stages * G.stage_bytes;
     // a replica's row in 2^lgsplit parts, W * 2^lgsplit parts dealt round robin: the fewest parts that balance the drift warps
     const uint32_t nd = GatherShape<CW, true>::kDriftWarps;
     // (a warp's cost: its share of a row, plus about a sixteenth of a row per part whatever the part holds: W = 17 in 8
     // parts per row, 17 parts per warp, ran at 0.56 where W = 16 in whole rows, 2 per warp, ran at 0.85; W = 12 in
     // halves 0.79 against 0.74 in whole rows; W = 5, P = 512 in quarters 0.86 against 0.83)
     uint32_t best = ~0u, share = 8u;
-    for (uint32_t lg = 0; (1u << lg) <= G.packets_per_tile && lg <= 2u; ++lg) {
+    for (uint32_t lg = 0; lg <= 2u; ++lg) {
       const uint32_t parts = ((c.W << lg) + nd - 1u) / nd;                   // a warp's parts ...
       const uint32_t eighths = parts * (8u >> lg);                            // ... and its share in eighths of a row
       const uint32_t cost = 2u * eighths + parts;
@@ -349,11 +355,15 @@ bool gather_geometry(const lossy_ctx* ctx, bool rd, TmaGeom& G) {
     // scratch of 4 chunks for a mean of 9) the compute warps' reads serve better; the caller falls back to them,
     // unless it was told to use this build (LOSSY_GATHER_PATH: comparison and tests). (W = 16, P = 256, p = 0.3,
     // bf16: 8 chunks for a mean of 4.5; W = 24: 8 for 6.9.)
-    const double mean = share / 8.0 * row_chunks * c.p_param * (c.W - 1.0) / c.W;
-    if (!(c.flags & LOSSY_GATHER_PATH) && G.rd_cap < mean) return false;
+    // (a 512-byte chunk that touches several packets is read if any of them is stale)
+    const double chunk_elems = 512.0 / rb, per_chunk = P % (512u / rb) == 0 ? 1.0 : (512u / rb) % P == 0 ? chunk_elems / P : 1.0 + chunk_elems / P;
+    const double mean = share / 8.0 * row_chunks * (1.0 - pow(1.0 - c.p_param * (c.W - 1.0) / c.W, per_chunk));
+    // (!ANY only: with the packets of the ANY builds drift warps stay ahead: W = 48, P = 736, p = 0.2, a mean of 9.6 chunks
+    // for a scratch of 8: 0.77 against 0.64)
+    if (!ANY && !(c.flags & LOSSY_GATHER_PATH) && G.rd_cap < mean) return false;
   }
   G.tiles_per_packet = 1;
-  const uint64_t tiles = (kfull + G.packets_per_tile - 1) / G.packets_per_tile;
+  const uint64_t tiles = (kfull * P + kTile - 1) / kTile;
   if (tiles >= (1ull << 31)) return false;
   G.num_tiles = (uint32_t)tiles;
   G.status = ctx->status;
@@ -365,15 +375,15 @@ bool gather_geometry(const lossy_ctx* ctx, bool rd, TmaGeom& G) {
   // p = 0.3: +4 %) and with 9-12 or more than 16 workers at any loss (W = 24: +4 % at p = 0, +6 % at 0.1; W = 64,
   // P = 512: +9 %); where most rows are whole, up to 8 or with 13-16 workers, both warps in one row do better
   // (W = 16: 0.98-0.99 against 0.91-0.94 up to p = 0.05; W = 8: +1 %). Same-process A/B pairs, repeatable to 0.002.
-  const double whole_rows = pow(1.0 - c.p_grad, (double)G.packets_per_tile);
+  const double whole_rows = pow(1.0 - c.p_grad, (double)kTile / P);
   if (whole_rows >= 0.6 && (c.W <= 8u || (c.W >= 13u && c.W <= 16u))) G.hints |= 8u;
   return true;
 }
 
-template <class GT, class RT, int OPT, bool DRIFTK, int CW, bool RD>
+template <class GT, class RT, int OPT, bool DRIFTK, int CW, bool RD, bool ANY>
 int launch_gather(lossy_ctx* ctx, const Params& P, const TmaGeom& G, cudaStream_t s, uint32_t* blocks_out) {
-  auto kern = lossy_fused_gather_kernel<GT, RT, OPT, DRIFTK, CW, RD>;
-  const uint32_t smem = kGatherSmemFixed + G.state_bytes + G.stages * G.stage_bytes;
+  auto kern = lossy_fused_gather_kernel<GT, RT, OPT, DRIFTK, CW, RD, ANY>;
+  const uint32_t smem = kGatherSmemFixed<ANY> + G.state_bytes + G.stages * G.stage_bytes;
   uint32_t blocks = (uint32_t)(ctx->num_sms * GatherShape<CW>::kCtasPerSm);
   if (blocks > G.num_tiles) blocks = G.num_tiles;
   *blocks_out = blocks;
@@ -395,27 +405,116 @@ int launch_gather(lossy_ctx* ctx, const Params& P, const TmaGeom& G, cudaStream_
   return LOSSY_OK;
 }
 
-template <bool DRIFTK, int CW, bool RD>
+template <bool DRIFTK, int CW, bool RD, bool ANY>
 int dispatch_gather(lossy_ctx* ctx, const Params& P, const TmaGeom& G, cudaStream_t s, uint32_t* blocks) {
   const bool gb = ctx->cfg.grad_dtype == LOSSY_BF16;
   const bool rb = ctx->cfg.replica_dtype == LOSSY_BF16;
   const bool adam = ctx->cfg.optimizer == LOSSY_ADAM;
-  if (gb && rb) return adam ? launch_gather<BF16, BF16, 1, DRIFTK, CW, RD>(ctx, P, G, s, blocks) : launch_gather<BF16, BF16, 0, DRIFTK, CW, RD>(ctx, P, G, s, blocks);
-  if (gb && !rb) return adam ? launch_gather<BF16, F32, 1, DRIFTK, CW, RD>(ctx, P, G, s, blocks) : launch_gather<BF16, F32, 0, DRIFTK, CW, RD>(ctx, P, G, s, blocks);
-  if (!gb && rb) return adam ? launch_gather<F32, BF16, 1, DRIFTK, CW, RD>(ctx, P, G, s, blocks) : launch_gather<F32, BF16, 0, DRIFTK, CW, RD>(ctx, P, G, s, blocks);
-  return adam ? launch_gather<F32, F32, 1, DRIFTK, CW, RD>(ctx, P, G, s, blocks) : launch_gather<F32, F32, 0, DRIFTK, CW, RD>(ctx, P, G, s, blocks);
+  if (gb && rb) return adam ? launch_gather<BF16, BF16, 1, DRIFTK, CW, RD, ANY>(ctx, P, G, s, blocks) : launch_gather<BF16, BF16, 0, DRIFTK, CW, RD, ANY>(ctx, P, G, s, blocks);
+  if (gb && !rb) return adam ? launch_gather<BF16, F32, 1, DRIFTK, CW, RD, ANY>(ctx, P, G, s, blocks) : launch_gather<BF16, F32, 0, DRIFTK, CW, RD, ANY>(ctx, P, G, s, blocks);
+  if (!gb && rb) return adam ? launch_gather<F32, BF16, 1, DRIFTK, CW, RD, ANY>(ctx, P, G, s, blocks) : launch_gather<F32, BF16, 0, DRIFTK, CW, RD, ANY>(ctx, P, G, s, blocks);
+  return adam ? launch_gather<F32, F32, 1, DRIFTK, CW, RD, ANY>(ctx, P, G, s, blocks) : launch_gather<F32, F32, 0, DRIFTK, CW, RD, ANY>(ctx, P, G, s, blocks);
 }
 
-template <int CW>
-int try_gather(lossy_ctx* ctx, const Params& P, bool drift, bool rd, cudaStream_t s, uint32_t* blocks, bool* used) {
+template <int CW, bool ANY>
+int try_gather_build(lossy_ctx* ctx, const Params& P, bool drift, bool rd, cudaStream_t s, uint32_t* blocks, bool* used) {
   TmaGeom G = {};
-  if (!gather_geometry<CW>(ctx, drift && rd, G)) return LOSSY_OK;
+  if (!gather_geometry<CW, ANY>(ctx, drift && rd, G)) return LOSSY_OK;
   *used = true;
   if (ctx->plan)
     snprintf(ctx->plan, ctx->plan_size, "gather %s packets/tile=%u stages=%u%s", CW == 16 ? "wide" : "twin", G.packets_per_tile, G.stages,
              drift && rd && CW == 16 ? " drift-warps" : "");
-  if (drift && rd) return dispatch_gather<true, CW, true>(ctx, P, G, s, blocks);
-  return drift ? dispatch_gather<true, CW, false>(ctx, P, G, s, blocks) : dispatch_gather<false, CW, false>(ctx, P, G, s, blocks);
+  if (drift && rd) return dispatch_gather<true, CW, true, ANY>(ctx, P, G, s, blocks);
+  return drift ? dispatch_gather<true, CW, false, ANY>(ctx, P, G, s, blocks) : dispatch_gather<false, CW, false, ANY>(ctx, P, G, s, blocks);
+}
+template <int CW>
+int try_gather(lossy_ctx* ctx, const Params& P, bool drift, bool rd, cudaStream_t s, uint32_t* blocks, bool* used) {
+  return GatherShape<CW>::kTile % P.P == 0 ? try_gather_build<CW, false>(ctx, P, drift, rd, s, blocks, used)
+                                           : try_gather_build<CW, true>(ctx, P, drift, rd, s, blocks, used);
+}
+
+// Where the gather pipeline is used, and which of its builds. Fractions of the copy rate below are of steps of buckets
+// of 20-200 M elements, taken back to back in one process; S = (W - 1) p_param = stale replicas per sub-packet.
+struct GatherPolicy {
+  bool use;
+  bool wide;          // 2048-element tiles, one CTA per SM (else 1024, two)
+  bool drift_warps;   // warps of their own read the stale copies
+};
+GatherPolicy gather_policy(const lossy_config& c) {
+  const double pm = c.p_grad > c.p_param ? c.p_grad : c.p_param;
+  const double stale = (c.W - 1u) * c.p_param;
+  const uint32_t P = c.packet_elems, kTwin = (uint32_t)TmaShape<8>::kTile, kWide = (uint32_t)GatherShape<16>::kTile;
+  const bool bf16 = c.replica_dtype == LOSSY_BF16;
+  const bool forced = c.flags & LOSSY_GATHER_PATH;
+  GatherPolicy g = {false, false, false};
+  if (c.flags & LOSSY_PACKED_BULK) return g;
+  if (P < kTwin && kWide % P == 0) {
+    // Packets of 128, 256 or 512 elements, which divide the tile:
+    //  * the wide geometry with drift warps of its own from 4 workers, packets of 256 or 512 elements and bf16 replicas
+    //    (W = 8: 0.97 / 0.97 / 0.94 / 0.85 at p = 0.05 / 0.1 / 0.2 / 0.3, where the compute warps' reads gave 0.89 / 0.84 /
+    //    0.82 / 0.77 and the register kernel 0.77 and 0.67 at p = 0.1 and 0.3; W = 16: 0.90 / 0.86 at p = 0.2 / 0.3 against
+    //    0.81 / 0.69). With up to 16 workers from 0.2 (W - 8) stale replicas on: below that the compute warps' reads are
+    //    ahead (W = 16, p = 0.05: 0.95 against 0.84). With more from one stale replica on (W = 24, P = 256, p = 0.05: 0.93
+    //    against 0.88; W = 32, P = 512: 0.98 / 0.97 / 0.79 at p = 0.1 / 0.2 / 0.3 against 0.93, 0.83 and 0.72 before;
+    //    W = 48, P = 512, p = 0.2: 0.93 against 0.83);
+    //  * up to 12 stale replicas (W = 48, p = 0.3, S = 14: 0.70 against the register kernel's 0.75), but 7.5 where more
+    //    than 35 % of a replica's packets are stale (W = 17, p = 0.5: 0.43 against 0.56);
+    //  * packets of 256 elements and 32 workers or more keep what they had (its build is fixed by a test);
+    //  * fp32 replicas: the compute warps' reads (a row has twice the chunks and the wire ring leaves the drift warps
+    //    little scratch: W = 4, P = 512, p = 0.1: 0.88 against 0.80); LOSSY_GATHER_PATH asks for drift warps all the same;
+    //  * two or three workers, and packets of 128 elements: the twin geometry (W = 2: 0.78-0.81 against 0.69-0.74 for the
+    //    wide one), whose replica warps also read the stale copies up to four workers.
+    const bool wide_fits = P >= 256u;
+    const bool many = P >= 512u || c.W < 32u;
+    const double most = many && pm <= 0.35 ? 12.0 : 7.5, least = many && c.W > 16u ? 1.0 : 0.2 * ((double)c.W - 8.0);
+    g.wide = wide_fits && c.W >= 4u;
+    g.drift_warps = g.wide && (P >= 512u || c.W <= 31u) && stale < most && stale >= least && (bf16 || forced);
+    // The register kernel instead: many workers at high loss, where the compute warps would read the stale copies (bf16:
+    // W = 32, P = 256, p = 0.2: 0.83 against 0.79; fp32 replicas only with packets of 128 elements: P = 256, W = 24 and
+    // 48, p = 0.3: gather 0.89 and 0.90, register kernel 0.80 and 0.82)
+    const bool reg_ahead = !forced && !g.drift_warps &&
+                           (bf16 ? (c.W >= 12 && pm >= 0.25) || (c.W >= 24 && pm >= 0.15) : P < 256u && c.W >= 24 && pm >= 0.25);
+    g.use = !reg_ahead;
+    return g;
+  }
+  if (P < kTwin) {
+    // Other packets from 128 elements, shorter than the twin tile (the alternative is the register kernel, whose last
+    // chunk of a packet is part empty): P = 736: W = 8 0.94 / 0.89 / 0.81 at p = 0.1 / 0.2 / 0.3 against 0.53 / 0.49 / 0.46;
+    // W = 32 0.96 / 0.83 / 0.65 against 0.76 / 0.60 / 0.54; W = 48, p = 0.3 0.58 against 0.57; W = 2 0.73 against 0.49. Drift
+    // warps at every loss rate (W = 16, p = 0.02: 0.97 against 0.91, p = 0.3: 0.76 against 0.58) where their scratch fits,
+    // with fp32 replicas too (W = 4-7: 0.87-0.95 against 0.73-0.84 at p = 0.1).
+    // Packets under 176 elements put more than 12 sub-packets on a wide tile: twin tiles at low loss (W = 8, P = 144, p =
+    // 0.05: 0.68 against 0.59), wide ones from p = 0.15 (p = 0.3: 0.55 against 0.47); up to four workers twin below 256
+    // (W = 4, P = 200: 0.75 against 0.63).
+    g.use = true;
+    g.wide = c.W >= 5u ? P >= 176u || pm >= 0.15 : c.W == 4u && P >= 256u;
+    g.drift_warps = g.wide;
+    // a handful of tiles with fp32 replicas: the register kernel spreads them wider (W = 17, 13 k elements: 15.3 us
+    // against 16.5 us)
+    if (!bf16 && !forced && c.n < 8u * (uint64_t)kWide && g.wide) g.use = false;
+    return g;
+  }
+  if (P % kTwin != 0 && P < (1u << 15)) {
+    // Longer packets that are no multiple of the twin tile. The bulk-copy pipeline cuts each into tiles of its own, the
+    // last of them part empty (`fill` of the tiles' elements are used); here the tiles run on across packets. bf16 replicas,
+    // p = 0.05: W = 8: 0.95-0.96 at any length against 0.61 (P = 1032), 0.79 (1472), 0.93-0.95 (from 1928); W = 40: 0.94-0.97
+    // against 0.55, 0.77, 0.83-0.92. At p = 0.2 W = 8 0.88-0.90 against 0.53, 0.74, 0.83-0.87, but W = 16 0.83-0.86 against
+    // 0.56, 0.76, 0.87-0.90: full tiles are left to the bulk pipeline at high loss, poorly filled ones up to 12 stale
+    // replicas (W = 24, P = 1472, p = 0.3: 0.70 against 0.68; W = 64: 0.57 against 0.76). Few workers only where tiles are half
+    // empty (W = 3, P = 1032: 0.72 against 0.57, P = 1472: 0.73 against 0.77; W = 4, P = 1472: 0.83 against 0.79).
+    // fp32 replicas: W = 4, 8, 16, 48, P = 1032, p = 0.05: 0.90, 0.88, 0.89, 0.96 against 0.80, 0.78, 0.65, 0.68; P = 1928: 0.90,
+    // 0.88, 0.90, 0.96 against 0.84, 0.85, 0.89, 0.86, at p = 0.2 0.74, 0.78, 0.83, 0.86 against 0.87, 0.86, 0.88, 0.93 (and W = 4,
+    // P = 1736, p = 0.01, 5 M elements 54.5 us against 50.5 us): full tiles only from 24 workers and at low loss.
+    // Owner-elided replicas: W = 16, P = 4480, p = 0.05 973 us against the bulk pipeline's 922 us, so full tiles stay there.
+    const double fill = P / (double)((P + kTwin - 1u) / kTwin * kTwin);
+    g.wide = c.W >= 4u;
+    g.drift_warps = g.wide;
+    if (c.W <= 3u) g.use = fill < 0.65;
+    else if (!bf16) g.use = fill < 0.65 || (fill < 0.8 && (c.W >= 12u || pm < 0.1)) || (c.W >= 24u && pm < 0.1);
+    else if (fill < 0.8) g.use = stale < 12.0;
+    else g.use = c.W >= 5u && (pm < 0.175 || (c.W <= 12u && pm < 0.25)) && !(c.flags & LOSSY_REPLICA_SKIP_OWNER);
+  }
+  return g;
 }
 
 // Run the build the policy picks; *used stays false when no bulk-copy launch fits (packets shorter
@@ -424,45 +523,15 @@ int run_tma(lossy_ctx* ctx, const Params& P, bool drift, cudaStream_t s, uint32_
   *used = false;
   if (ctx->cfg.flags & LOSSY_REGISTER_PATH) return LOSSY_OK;
   const TmaPolicy t = tma_policy(ctx->cfg);
-  if (!(ctx->cfg.flags & LOSSY_PACKED_BULK) && ctx->cfg.packet_elems < (uint32_t)TmaShape<8>::kTile) {
-    // Packets shorter than a tile (128, 256 or 512 elements): the gather pipeline, where it beats the register
-    // kernel. Fractions of the copy rate, 20 steps of a 202 M element bucket, P = 256, taken back to back in one
-    // process (power-capped clocks; a point measured alone runs 3-6 % higher), S = (W - 1) p_param = stale replicas
-    // per sub-packet:
-    //  * the wide geometry with drift warps of its own for 4..24 workers, packets of 256 or 512 elements and
-    //    0.2 (W - 8) <= S < 7.5 (W = 8: 0.97 / 0.97 / 0.94 / 0.85 at p = 0.05 / 0.1 / 0.2 / 0.3, where the compute
-    //    warps' reads gave 0.89 / 0.84 / 0.82 / 0.77 and the register kernel 0.77 and 0.67 at p = 0.1 and 0.3; W = 16:
-    //    0.92 / 0.88 / 0.84 at p = 0.1 / 0.2 / 0.3 against 0.90 / 0.81 / 0.69, register kernel 0.82 / 0.79 / 0.76;
-    //    W = 24: 0.83 and 0.78 at p = 0.2 and 0.3 against 0.81 and 0.72; W = 4: 0.77-0.83 against 0.75-0.84 for the
-    //    twin geometry);
-    //  * below that band (many workers, few stale copies) the compute warps' reads stay ahead (W = 16, p = 0.05: 0.98
-    //    against 0.91; W = 24, p = 0.1: 0.88 against 0.85; W = 32, p = 0.05: 0.96 against 0.91);
-    //  * above it the drift warps fall behind (W = 17, p = 0.5: 0.43): many workers at high loss stay with the
-    //    register kernel (p = 0.2, W = 32: 0.85 against 0.79-0.84; W = 17, p = 0.5: 0.56);
-    //  * two or three workers, and packets of 128 elements: the twin geometry (W = 2: 0.78-0.81 against 0.69-0.74
-    //    for the wide one), whose replica warps also read the stale copies up to four workers.
-    const lossy_config& c = ctx->cfg;
-    const double pm = c.p_grad > c.p_param ? c.p_grad : c.p_param;
-    const bool wide_fits = c.packet_elems * (uint32_t)kMaxSub >= (uint32_t)GatherShape<16>::kTile;
-    const double stale = (c.W - 1u) * c.p_param;
-    // (bf16 replicas: with fp32 ones a row has twice the chunks and the wire ring leaves the drift warps little
-    // scratch; the compute warps' reads gave 0.71-0.73 where drift warps gave 0.48-0.59; LOSSY_GATHER_PATH asks
-    // for the drift warps all the same, for tests)
-    const bool drift_warps = wide_fits && c.W >= 4u && c.W <= 24u && stale < 7.5 && stale >= 0.2 * ((double)c.W - 8.0) &&
-                             (c.replica_dtype == LOSSY_BF16 || (c.flags & LOSSY_GATHER_PATH));
-    // (the register kernel's lead at high loss was measured with bf16 replicas; with fp32 ones the compute warps'
-    // reads are ahead at W = 12-16, p = 0.3: 0.71-0.73 against 0.57-0.62)
-    const bool reg_ahead = !(c.flags & LOSSY_GATHER_PATH) && !drift_warps &&
-                           (c.replica_dtype == LOSSY_BF16 ? (c.W >= 12 && pm >= 0.25) || (c.W >= 24 && pm >= 0.15) : c.W >= 24 && pm >= 0.25);
-    if (!reg_ahead) {
-      int rc = LOSSY_OK;
-      if (c.W >= 4u) rc = try_gather<16>(ctx, P, drift, drift_warps, s, blocks, used);
-      if (rc || *used) return rc;
-      if (c.W > kRdTwinMaxWorkers && drift && drift_warps) rc = try_gather<16>(ctx, P, drift, false, s, blocks, used);   // scratch too small
-      if (rc || *used) return rc;
-      rc = try_gather<8>(ctx, P, drift, c.W <= kRdTwinMaxWorkers, s, blocks, used);
-      if (rc || *used) return rc;
-    }
+  const GatherPolicy gp = gather_policy(ctx->cfg);
+  if (gp.use) {
+    int rc = LOSSY_OK;
+    if (gp.wide) rc = try_gather<16>(ctx, P, drift, gp.drift_warps, s, blocks, used);
+    if (rc || *used) return rc;
+    if (gp.wide && gp.drift_warps && drift && ctx->cfg.W > kRdTwinMaxWorkers) rc = try_gather<16>(ctx, P, drift, false, s, blocks, used);   // scratch too small
+    if (rc || *used) return rc;
+    rc = try_gather<8>(ctx, P, drift, ctx->cfg.W <= kRdTwinMaxWorkers, s, blocks, used);
+    if (rc || *used) return rc;
   }
   {
     // Packets of exactly half a wide tile with 13..16 workers at low loss: the PACKED wide build (two packets

@@ -1,7 +1,8 @@
-// Fused lossy step for packets SHORTER than a tile: the "gather" pipeline (sm_100a).
+// Fused lossy step for packets that are not whole tiles: the "gather" pipeline (sm_100a).
 //
-// A tile holds 2, 4 or 8 whole packets ("sub-packets"), each with delivery masks of its own, so every stream
-// of the step has holes at sub-packet granularity: dropped gradient pieces are not read, replicas that miss
+// A tile touches several packets ("sub-packets"), each with delivery masks of its own: 2, 4 or 8 whole ones where they
+// divide the tile, else (ANY builds) up to 16, the first and last of them shared with the neighbouring tiles. So every
+// stream of the step has holes at sub-packet granularity: dropped gradient pieces are not read, replicas that miss
 // a broadcast are not written, and their old copies are read for the drift term. Bulk copies of a few
 // hundred bytes are bound by their issue rate, not by memory, and a worker's whole tile piece in one bulk
 // copy reads the dropped sub-packets too. Here everything with holes moves as 16 bytes per lane (512 bytes per
@@ -20,13 +21,20 @@
 //   drift norms    the old copy of every pair that misses the broadcast is read and its squared difference from
 //                  the wire tile summed, by whichever of three the host picked: eight drift warps of their own
 //                  (wide geometry, RD), the replica warps (twin geometry, RD), or the compute warps
-// A compute warp's 128 elements lie inside one sub-packet (packets here are powers of two from 128 elements
-// that divide the tile). Every wait is bounded as in the other pipelines. No cluster, no multicast.
+// A compute warp's 128 elements lie inside one sub-packet, or (ANY) inside two. The ANY builds are apart because every
+// role looks its sub-packets up per tile there; sharing the code cost the packets that divide the tile 5-10 %. What the
+// ANY builds replace for such packets is the register kernel (P = 736, W = 8, p = 0.1: 0.54 -> 0.94 of the copy rate) and
+// the bulk-copy pipeline with part-empty tiles (P = 1472, W = 8, p = 0.05: 0.79 -> 0.96). Every wait is bounded as in the other pipelines. No cluster, no multicast.
 #pragma once
+#include <type_traits>
+
 #include "lossy_tma.cuh"
 
 namespace lossy {
 
+// ANY: the build for packets that do not divide the tile. The tile then starts anywhere in its first packet and touches up
+// to ceil((P - 8 + tile) / P) of them (else tile / P <= kMaxSub).
+constexpr int kAnySub = 16;
 constexpr uint32_t kGatherRing = 8;     // tiles whose masks may be published ahead of the replica warps
 constexpr uint32_t kWireRing = 4;       // wire tiles between the compute warps and the replica warps
 // RD: the build in which the stale copies are read outside the compute warps (see the kernel): by the replica
@@ -36,7 +44,7 @@ template <int CW, bool RD = false> struct GatherShape {
   static constexpr int kReplicaWarps = (CW >= 16 || RD) ? 4 : 2;
   static constexpr int kDriftWarps = (CW >= 16 && RD) ? 8 : 0;
   static constexpr int kRdBuffers = kDriftWarps ? 1 : 2;                  // scratch buffers per warp that reads stale copies
-  static constexpr int kAccRows = RD ? (kDriftWarps ? kMaxSub : 1) : CW;  // rows of fp64 drift sums: per compute warp, or per part of a row (RD)
+  static constexpr int kAccRows = RD ? (kDriftWarps ? 4 : 1) : CW;  // rows of fp64 drift sums: per compute warp, or per part of a row (RD)
   static constexpr int kThreads = (CW + 2 + kProducers + kReplicaWarps + kDriftWarps) * 32;   // compute + mask + gather + store + replica (+ drift)
   static constexpr int kTile = CW * 32 * kEpl;
   static constexpr int kCtasPerSm = CW >= 16 ? 1 : 2;
@@ -46,12 +54,13 @@ constexpr uint32_t kGatherMaxStages = 8;    // a tile of few workers is small: m
 constexpr uint32_t kGatherBarBytes = 512;   // 3 barriers per stage, 2 per mask-ring and wire-ring entry (8 B each), the abort flag
 static_assert((3 * kGatherMaxStages + 2 * kGatherRing + 2 * kWireRing) * 8 + 4 <= kGatherBarBytes, "barrier area too small");
 
-struct __align__(16) TileMasks {        // one ring entry: what the mask warp publishes about a tile
-  uint64_t recv[kMaxSub];               // per sub-packet: bit i = worker i's piece was delivered
-  uint64_t stale[kMaxSub];              // per sub-packet: bit i = replica i misses the broadcast
-  uint32_t j[kMaxSub];                  // per sub-packet: owner
+template <int SUB> struct __align__(16) TileMasks {   // one ring entry: what the mask warp publishes about a tile
+  uint64_t recv[SUB];            // per sub-packet: bit i = worker i's piece was delivered
+  uint64_t stale[SUB];           // per sub-packet: bit i = replica i misses the broadcast
+  uint32_t j[SUB];               // per sub-packet: owner
   uint64_t e0;                          // first element of the tile
   uint32_t npk, len;                    // sub-packets and elements of the tile
+  uint32_t phase;                       // elements of sub-packet 0 that lie before the tile
 };
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
@@ -60,6 +69,14 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
 // the executing thread's earlier cp.async copies, once complete, count as one arrival on the barrier
 __device__ __forceinline__ void cp_async_arrive(uint32_t bar) {
   asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
+}
+
+// A shared-memory load that stays where it is written (the compiler otherwise moves a wire tile's worth of them out of
+// the loop over the replicas, and spills them)
+__device__ __forceinline__ uint4 lds_here(uint32_t src) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(src));
+  return v;
 }
 
 // One lane's arithmetic at the end of a tile: estimate = sum / count (Algorithm 1 mode: the saved aggregate
@@ -119,10 +136,17 @@ __device__ __forceinline__ void finish_tile_lane(const Params& P, float (&acc)[k
 // Wide geometry: eight drift warps of their own do nothing else (four were the step's bottleneck: 0.61 of the copy
 // rate at W = 16, P = 256, p = 0.3, against 0.85 with eight); one buffer each is enough, because the masks run
 // several tiles ahead of the wire tile.
-template <class GT, class RT, int OPT, bool DRIFTK, int CW, bool RD = false>
+template <class GT, class RT, int OPT, bool DRIFTK, int CW, bool RD, bool ANY>
 __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW, RD>::kCtasPerSm)
     lossy_fused_gather_kernel(const __grid_constant__ Params P, const __grid_constant__ TmaGeom G) {
   static_assert(!RD || DRIFTK, "RD is a way of computing the drift norms");
+  constexpr int kSub = ANY ? kAnySub : kMaxSub;
+  constexpr uint32_t kSubBits = (1u << kSub) - 1u;
+  using Masks = TileMasks<kSub>;
+  // How the replica warps store (see there), and how the stale chunks are walked: the twin builds for packets that divide
+  // the tile keep the forms they had (W = 40, P = 128: 0.85 against 0.79 with the wire tile held in registers).
+  constexpr bool kHoldWire = ANY || CW >= 16;
+  constexpr bool kChunkWalk = ANY || CW >= 16;
   constexpr bool kWarpDrift = DRIFTK && !RD;               // the compute warps read the stale copies
   constexpr int kTile = GatherShape<CW, RD>::kTile;
   constexpr int kNP = GatherShape<CW, RD>::kProducers;
@@ -137,9 +161,9 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
   //         warp and replica | wire ring | stages
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem);
   volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + kGatherBarBytes - 4);
-  TileMasks* ring = reinterpret_cast<TileMasks*>(smem + kGatherBarBytes);
-  StageHdr* hdrs = reinterpret_cast<StageHdr*>(smem + kGatherBarBytes + kGatherRing * sizeof(TileMasks));
-  double* warp_acc = reinterpret_cast<double*>(smem + kGatherBarBytes + kGatherRing * sizeof(TileMasks) + kGatherMaxStages * sizeof(StageHdr));
+  Masks* ring = reinterpret_cast<Masks*>(smem + kGatherBarBytes);
+  StageHdr* hdrs = reinterpret_cast<StageHdr*>(smem + kGatherBarBytes + kGatherRing * sizeof(Masks));
+  double* warp_acc = reinterpret_cast<double*>(smem + kGatherBarBytes + kGatherRing * sizeof(Masks) + kGatherMaxStages * sizeof(StageHdr));
   unsigned char* wring = reinterpret_cast<unsigned char*>(warp_acc + kAccRows * kMaxW);
   const uint32_t rd_buf = G.rd_cap * 512u;                 // RD: bytes of one scratch buffer
   unsigned char* rscratch = wring + kWireRing * kRowR;     // RD: kRdBuffers buffers per warp that reads stale copies
@@ -151,7 +175,10 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   const uint32_t W = P.W;
-  const uint32_t lgP = 31u - (uint32_t)__clz((int)P.P);                 // packets are powers of two here
+  const uint32_t lgP = 31u - (uint32_t)__clz((int)P.P);                 // packets that divide the tile are powers of two
+  // Sub-packet of element el of a tile. ANY: the quotient (phase + el) / P by a multiplication with G.magic = 2^32 / P
+  // rounded up, exact because (phase + el) P < 2^32 for P < 2^15.
+  auto sub_of = [&](uint32_t phase, uint32_t el) { return ANY ? __umulhi(phase + el, G.magic) : el >> lgP; };
   auto full_bar = [&](uint32_t s) { return smem_u32(&bars[s]); };
   auto done_bar = [&](uint32_t s) { return smem_u32(&bars[kGatherMaxStages + s]); };
   auto empty_bar = [&](uint32_t s) { return smem_u32(&bars[2 * kGatherMaxStages + s]); };
@@ -183,68 +210,86 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
 
   constexpr int kChunks = kRowR / 512u;                     // a replica's row of a tile in 512-byte chunks
   constexpr uint32_t kElemsPerChunk = 512u / kRB;
-  // Wide RD builds. A replica's row of a tile is cut into 2^lgf parts (the host balances the W * 2^lgf parts over
-  // the drift warps); a warp takes parts first, first + stride, ... PASS 0 requests the old copies of their stale
-  // (replica, sub-packet) pairs into `buffer`, chunk after chunk in the order (part, chunk); pass 1 takes their
+  // A row's chunks that hold elements of sub-packet s, as bits: lane l of a warp keeps those of sub-packet l mod kSub, and the
+  // chunks a replica's stale sub-packets touch are the OR over their lanes.
+  auto chunks_of = [&](const Masks& tm) {
+    const uint32_t s0 = ((uint32_t)lane & (kSub - 1)) * P.P;         // the sub-packet, counted from sub-packet 0
+    const uint32_t first = s0 > tm.phase ? s0 - tm.phase : 0u;
+    const uint32_t end = min(s0 + P.P - tm.phase, tm.len);
+    if (((uint32_t)lane & (kSub - 1)) >= tm.npk) return 0u;
+    return (2u << ((end - 1u) / kElemsPerChunk)) - (1u << (first / kElemsPerChunk));
+  };
+  // Where replica i's row of a tile begins (as if nothing were elided before it), and which of the tile's sub-packets lie
+  // behind worker i's own shard, rep_skip[i] elements lower: none with full replicas, mostly all or none otherwise, so
+  // that the per-chunk test is needed in the few tiles at a shard's end only. j_l: the owner of sub-packet l mod kSub.
+  auto row_base = [&](uint32_t i, uint32_t j_l, uint32_t live_tile, uint64_t e0, uint32_t& behind) {
+    unsigned char* base = reinterpret_cast<unsigned char*>(P.replicas[i]) + e0 * kRB;
+    behind = 0u;
+    if (P.flags & kSkipOwner) {
+      behind = __ballot_sync(0xFFFFFFFFu, j_l > i) & live_tile;
+      if (behind == live_tile) { base -= P.rep_skip[i] * kRB; behind = 0u; }
+    }
+    return base;
+  };
+  // Wide RD builds. A replica's row of a tile is cut into 2^lgf parts of equal chunks (the host balances the W * 2^lgf
+  // parts over the drift warps); a warp takes parts first, first + stride, ... PASS 0 requests the old copies of their
+  // stale (replica, sub-packet) pairs into `buffer`, chunk after chunk in the order (part, chunk); pass 1 takes their
   // squared differences against the wire tile: fp32 per lane within a part's chunks, one warp reduction per part
   // and tile, fp64 from there on (each (replica, part) has one accumulator, touched by one warp alone, in tile
   // order; the CTA's exit adds a replica's parts in ascending order).
   // One warp runs this alone, so its instructions are fetched for it alone: the walk visits the stale chunks only
-  // and is kept short (one loop body for both passes, nothing unrolled), and each role calls it from one place.
-  constexpr uint32_t kLgEpc = kElemsPerChunk == 256u ? 8u : 7u;
-  auto drift_pass = [&](const TileMasks& tm, uint32_t first, uint32_t stride, unsigned char* buffer, int pass, const unsigned char* wt) {
-    const uint32_t lgf = G.rd_lgsplit, part = G.packets_per_tile >> lgf;   // a replica's row in 2^lgf parts of `part` sub-packets
-    const uint64_t stale_l = tm.stale[lane & (kMaxSub - 1)];
-    const uint32_t j_l = tm.j[lane & (kMaxSub - 1)];
-    const uint32_t live_tile = (1u << tm.npk) - 1u;       // entries behind a short last tile are marked stale everywhere
+  // and is kept short (one loop body for both passes, nothing unrolled), and each role calls it from one place. The walk
+  // over a row's chunks takes one reduction over the lanes' chunk sets; over its sub-packets, with a loop over each one's
+  // chunks, W = 16, P = 256, p = 0.3 ran at 0.85 against 0.88.
+  auto drift_pass = [&](const Masks& tm, uint32_t first, uint32_t stride, unsigned char* buffer, int pass, const unsigned char* wt) {
+    const uint32_t lgf = G.rd_lgsplit, part = (uint32_t)kChunks >> lgf;     // a replica's row in 2^lgf parts of `part` chunks
+    const uint64_t stale_l = tm.stale[lane & (kSub - 1)];
+    const uint32_t j_l = tm.j[lane & (kSub - 1)];
+    const uint32_t live_tile = (1u << tm.npk) - 1u;       // entries behind the tile's last sub-packet are marked stale everywhere
+    const uint32_t chunks_l = chunks_of(tm), phase = tm.phase;
     const uint64_t e0 = tm.e0;
-    const bool whole = lgP >= kLgEpc;                      // a sub-packet is one or more whole chunks (else a chunk holds several)
-    const uint32_t sh = whole ? lgP - kLgEpc : kLgEpc - lgP;
     uint32_t n = 0;                                        // stale chunks met so far (warp-uniform)
 #pragma unroll 1
     for (uint32_t u = first; u < (W << lgf); u += stride) {
       const uint32_t i = u >> lgf, h = u & ((1u << lgf) - 1u);
-      const uint32_t live = __ballot_sync(0xFFFFFFFFu, (stale_l >> i) & 1ull) & live_tile & (((1u << part) - 1u) << (h * part));
-      if (live == 0u) continue;
-      const unsigned char* base = reinterpret_cast<const unsigned char*>(P.replicas[i]);
+      const bool st = (stale_l >> i) & 1ull;
+      const uint32_t live = __ballot_sync(0xFFFFFFFFu, st) & live_tile;
+      uint32_t rem = __reduce_or_sync(0xFFFFFFFFu, st ? chunks_l : 0u) & (((1u << part) - 1u) << (h * part));
+      if (rem == 0u) continue;
+      uint32_t behind;
+      const unsigned char* base = row_base(i, j_l, live_tile, e0, behind);
       float2 sq2 = make_float2(0.0f, 0.0f);                // two running sums (packed fp32 pairs of sm_100)
-      uint32_t rem = live;
 #pragma unroll 1
       while (rem) {
-        const uint32_t sp0 = (uint32_t)__ffs((int)rem) - 1u;
-        uint32_t c, c_end;
-        if (whole) { c = sp0 << sh; c_end = c + (1u << sh); rem &= rem - 1u; }
-        else { c = sp0 >> sh; c_end = c + 1u; rem &= ~(((1u << (1u << sh)) - 1u) << (c << sh)); }
-#pragma unroll 1
-        for (; c < c_end; ++c) {
-          const uint32_t q = n++;
-          const uint32_t off = c * 512u + (uint32_t)lane * 16u;
-          const uint32_t el = off / kRB, sp = el >> lgP;
-          const uint32_t j_sp = __shfl_sync(0xFFFFFFFFu, j_l, (int)sp);
-          if (!((live >> sp) & 1u)) continue;              // this lane's 16 bytes are not stale ones
-          unsigned char* sc = buffer + q * 512u + (uint32_t)lane * 16u;
-          const unsigned char* old = base + rep_index(P, i, j_sp, e0 + el) * kRB;
-          if (pass == 0) {
-            if (q < G.rd_cap) cp_async16(smem_u32(sc), old);
-          } else {
-            // each lane reads back what it copied itself; a chunk the scratch had no room for comes from memory now
-            const uint4 ov = q < G.rd_cap ? *reinterpret_cast<const uint4*>(sc) : __ldcs(reinterpret_cast<const uint4*>(old));
-            const uint4 wv = *reinterpret_cast<const uint4*>(wt + off);
-            const uint32_t ow[4] = {ov.x, ov.y, ov.z, ov.w}, ww[4] = {wv.x, wv.y, wv.z, wv.w};
-            if constexpr (RT::kVecs == 2) {                // fp32 replicas: one element per word
+        const uint32_t c = (uint32_t)__ffs((int)rem) - 1u;
+        rem &= rem - 1u;
+        const uint32_t q = n++;
+        const uint32_t off = c * 512u + (uint32_t)lane * 16u;
+        const uint32_t sp = sub_of(phase, off / kRB);
+        if (!((live >> sp) & 1u)) continue;                // this lane's 16 bytes are not stale ones
+        unsigned char* sc = buffer + q * 512u + (uint32_t)lane * 16u;
+        const unsigned char* old = base + off;
+        if (behind && ((behind >> sp) & 1u)) old -= P.rep_skip[i] * kRB;
+        if (pass == 0) {
+          if (q < G.rd_cap) cp_async16(smem_u32(sc), old);
+        } else {
+          // each lane reads back what it copied itself; a chunk the scratch had no room for comes from memory now
+          const uint4 ov = q < G.rd_cap ? *reinterpret_cast<const uint4*>(sc) : __ldcs(reinterpret_cast<const uint4*>(old));
+          const uint4 wv = *reinterpret_cast<const uint4*>(wt + off);
+          const uint32_t ow[4] = {ov.x, ov.y, ov.z, ov.w}, ww[4] = {wv.x, wv.y, wv.z, wv.w};
+          if constexpr (RT::kVecs == 2) {                  // fp32 replicas: one element per word
 #pragma unroll
-              for (int h = 0; h < 4; h += 2) {
-                const float2 d = __fadd2_rn(make_float2(__uint_as_float(ow[h]), __uint_as_float(ow[h + 1])),
-                                            make_float2(-__uint_as_float(ww[h]), -__uint_as_float(ww[h + 1])));
-                sq2 = __fadd2_rn(sq2, __fmul2_rn(d, d));
-              }
-            } else {                                        // bf16 replicas: two elements per word
+            for (int y = 0; y < 4; y += 2) {
+              const float2 d = __fadd2_rn(make_float2(__uint_as_float(ow[y]), __uint_as_float(ow[y + 1])),
+                                          make_float2(-__uint_as_float(ww[y]), -__uint_as_float(ww[y + 1])));
+              sq2 = __fadd2_rn(sq2, __fmul2_rn(d, d));
+            }
+          } else {                                          // bf16 replicas: two elements per word
 #pragma unroll
-              for (int h = 0; h < 4; ++h) {
-                const float2 d = __fadd2_rn(make_float2(__uint_as_float(ow[h] << 16), __uint_as_float(ow[h] & 0xFFFF0000u)),
-                                            make_float2(-__uint_as_float(ww[h] << 16), -__uint_as_float(ww[h] & 0xFFFF0000u)));
-                sq2 = __fadd2_rn(sq2, __fmul2_rn(d, d));
-              }
+            for (int y = 0; y < 4; ++y) {
+              const float2 d = __fadd2_rn(make_float2(__uint_as_float(ow[y] << 16), __uint_as_float(ow[y] & 0xFFFF0000u)),
+                                          make_float2(-__uint_as_float(ww[y] << 16), -__uint_as_float(ww[y] & 0xFFFF0000u)));
+              sq2 = __fadd2_rn(sq2, __fmul2_rn(d, d));
             }
           }
         }
@@ -270,25 +315,50 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
     // (G.hints bit 2: the host asks for it where few pairs per tile are stale — it gains about 5 % there and
     // loses as much where they are many: the prefetches then crowd the bulk-copy unit that moves theta, m, v)
     const bool prefetch_on = kWarpDrift && (G.hints & 4u);
-    auto prefetch_stale = [&](uint32_t i, uint32_t j, uint32_t k) {
-      bulk_prefetch_l2(reinterpret_cast<const typename RT::raw*>(P.replicas[i]) + rep_index(P, i, j, (uint64_t)k * P.P), P.P * kRB);
+    const uint64_t e_end = (uint64_t)G.full_packets * P.P;
+    // ANY: the first packet of a tile and the tile's offset in it, carried from tile to tile
+    uint32_t kfirst = 0, phase = 0;
+    [[maybe_unused]] uint32_t k_step = 0, phase_step = 0;
+    if constexpr (ANY) {
+      const uint64_t at = (uint64_t)blockIdx.x * kTile, step = (uint64_t)gridDim.x * kTile;
+      kfirst = (uint32_t)(at / P.P);
+      phase = (uint32_t)(at - (uint64_t)kfirst * P.P);
+      k_step = (uint32_t)(step / P.P);
+      phase_step = (uint32_t)(step - (uint64_t)k_step * P.P);
+    }
+    auto next_tile = [&]() {
+      if constexpr (ANY) {
+        kfirst += k_step;
+        phase += phase_step;
+        if (phase >= P.P) { phase -= P.P; ++kfirst; }
+      }
     };
-    for (uint32_t tile = blockIdx.x; tile < G.num_tiles; tile += gridDim.x) {
+    for (uint32_t tile = blockIdx.x; tile < G.num_tiles; tile += gridDim.x, next_tile()) {
       if (!mbar_wait(mempty_bar(slot), par ^ 1u, abort_flag)) break;
-      const uint32_t kfirst = tile * G.packets_per_tile;
-      const uint32_t npk = min(G.packets_per_tile, G.full_packets - kfirst);
+      if constexpr (!ANY) kfirst = tile * G.packets_per_tile;
+      const uint64_t e0 = (uint64_t)tile * kTile;
+      const uint32_t len = (uint32_t)min((uint64_t)kTile, e_end - e0);
+      const uint32_t npk = ANY ? sub_of(phase, len - 1u) + 1u : min(G.packets_per_tile, G.full_packets - kfirst);
+      // the part of sub-packet sp that lies in this tile
+      auto sub_begin = [&](uint32_t sp) { return sp == 0 ? 0u : sp * P.P - phase; };
+      auto sub_end = [&](uint32_t sp) { return min((sp + 1u) * P.P - phase, len); };
+      auto prefetch_stale = [&](uint32_t i, uint32_t j, uint32_t sp) {
+        const uint32_t b = sub_begin(sp);
+        bulk_prefetch_l2(reinterpret_cast<const typename RT::raw*>(P.replicas[i]) + rep_index(P, i, j, e0 + b), (sub_end(sp) - b) * kRB);
+      };
       if constexpr (kDevCheck) {   // debug build: every sub-packet's range, in the slab and in every replica
         bool fine = true;
         for (uint32_t sp = 0; sp < npk; ++sp)
-          fine = tile_ok(P, kfirst + sp, (P.k0 + kfirst + sp) / P.pps, (uint64_t)(kfirst + sp) * P.P, P.P, kSiteGather, lane) && fine;
+          fine = tile_ok(P, kfirst + sp, (P.k0 + kfirst + sp) / P.pps, e0 + sub_begin(sp), sub_end(sp) - sub_begin(sp), kSiteGather, lane) && fine;
         if (!fine) { *abort_flag = 1u; break; }
       }
-      TileMasks& tm = ring[slot];
+      Masks& tm = ring[slot];
       auto report = [&](uint32_t sp, uint32_t j, uint64_t r, uint64_t st, uint64_t gbad, uint64_t pbad) {   // one lane
         const uint32_t k = kfirst + sp;
         tm.recv[sp] = r;
         tm.stale[sp] = st;
         tm.j[sp] = j;
+        if (ANY && sp == 0 && phase != 0) return;                   // the tile before this one has reported the packet
         if (P.count) P.count[k] = (uint8_t)__popcll(r);
         if (P.recv_bits) P.recv_bits[k] = r;
         if (P.stale_bits) P.stale_bits[k] = st;
@@ -311,7 +381,7 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
             if (x == ((uint32_t)lane >> lgWp)) st_l = st;
             if ((uint32_t)lane == x) report(q0 + x, j_x, r, st, gbad, pbad);
           }
-          if (prefetch_on && sp_l < npk && i_l < W && ((st_l >> i_l) & 1ull)) prefetch_stale(i_l, j_l, k_l);
+          if (prefetch_on && sp_l < npk && i_l < W && ((st_l >> i_l) & 1ull)) prefetch_stale(i_l, j_l, sp_l);
         }
       } else {
         for (uint32_t sp = 0; sp < npk; ++sp) {
@@ -321,19 +391,20 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
           if (lane == 0) report(sp, j_sp, r, st, gbad, pbad);
           if (prefetch_on) {
             for (uint32_t i = lane; i < W; i += 32)
-              if ((st >> i) & 1ull) prefetch_stale(i, j_sp, kfirst + sp);
+              if ((st >> i) & 1ull) prefetch_stale(i, j_sp, sp);
           }
         }
       }
-      if ((uint32_t)lane >= npk && lane < kMaxSub) {      // entries behind a short last tile: nothing delivered, nothing to do
+      if ((uint32_t)lane >= npk && lane < kSub) {   // entries behind the last sub-packet: nothing delivered, nothing to do
         tm.recv[lane] = 0;
         tm.stale[lane] = ~0ull;
         tm.j[lane] = 0;
       }
       if (lane == 0) {
-        tm.e0 = (uint64_t)kfirst * P.P;
+        tm.e0 = e0;
         tm.npk = npk;
-        tm.len = npk * P.P;
+        tm.len = len;
+        tm.phase = phase;
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(mfull_bar(slot));
@@ -342,17 +413,23 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
   } else if (warp > CW && warp <= CW + kNP) {
     // ================================ gather warps ================================
     const uint32_t pw = (uint32_t)(warp - CW - 1);          // which gather warp
+    constexpr uint32_t kRowChunks = kRowG / 512u;
+    [[maybe_unused]] uint32_t sub_c[kRowChunks];            // ANY: the sub-packet this lane's bytes of chunk c lie in
     uint32_t s = 0, par = 0, slot = 0, mpar = 0;
     bool ok = true;
     auto next_stage = [&]() { if (++s == S) { s = 0; par ^= 1u; } };
     for (uint32_t tile = blockIdx.x; ok && tile < G.num_tiles; tile += gridDim.x) {
       if (!mbar_wait(mfull_bar(slot), mpar, abort_flag)) { ok = false; break; }
-      const TileMasks& tm = ring[slot];
+      const Masks& tm = ring[slot];
       const uint64_t e0 = tm.e0;
       const uint32_t len = tm.len;
-      // lane l holds sub-packet (l & 7)'s receive mask; a ballot per worker turns that column into the worker's
+      // lane l holds sub-packet l mod kSub's receive mask; a ballot per worker turns that column into the worker's
       // row of delivered sub-packets
-      const uint64_t recv_l = tm.recv[lane & (kMaxSub - 1)];
+      const uint64_t recv_l = tm.recv[lane & (kSub - 1)];
+      if constexpr (ANY) {
+#pragma unroll
+        for (uint32_t c = 0; c < kRowChunks; ++c) sub_c[c] = sub_of(tm.phase, (c * 512u + (uint32_t)lane * 16u) / kGB);
+      }
       for (uint32_t g = 0; g < G.groups; ++g, next_stage()) {
         if (!mbar_wait(empty_bar(s), par ^ 1u, abort_flag)) { ok = false; break; }
         const bool last = g + 1 == G.groups;
@@ -378,14 +455,22 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
         // Delivered pieces of this group's workers: a row is copied in chunks of 512 bytes (one warp
         // instruction, 16 bytes per lane), each lane testing the sub-packet its 16 bytes lie in.
         auto copy_row = [&](uint32_t u, uint32_t c_first, uint32_t c_step) {
-          const uint32_t rowmask = __ballot_sync(0xFFFFFFFFu, (recv_l >> (g * kGroup + u)) & 1ull) & 0xFFu;
+          const uint32_t rowmask = __ballot_sync(0xFFFFFFFFu, (recv_l >> (g * kGroup + u)) & 1ull) & kSubBits;
           if (rowmask == 0u) return;
           const unsigned char* src = reinterpret_cast<const unsigned char*>(P.grads[g * kGroup + u]) + e0 * kGB;
           const uint32_t dst = st + u * kRowG;
+          if constexpr (ANY) {
 #pragma unroll
-          for (uint32_t c = c_first; c < kRowG / 512u; c += c_step) {
-            const uint32_t off = c * 512u + (uint32_t)lane * 16u;   // byte within the row
-            if ((rowmask >> ((off / kGB) >> lgP)) & 1u) cp_async16(dst + off, src + off);
+            for (uint32_t c = 0; c < kRowChunks; ++c) {
+              const uint32_t off = c * 512u + (uint32_t)lane * 16u;
+              if ((c_step == 1u || c % c_step == c_first) && ((rowmask >> sub_c[c]) & 1u)) cp_async16(dst + off, src + off);
+            }
+          } else {
+#pragma unroll
+            for (uint32_t c = c_first; c < kRowChunks; c += c_step) {
+              const uint32_t off = c * 512u + (uint32_t)lane * 16u;   // byte within the row
+              if ((rowmask >> ((off / kGB) >> lgP)) & 1u) cp_async16(dst + off, src + off);
+            }
           }
         };
         // Two gather warps deal out either the group's workers (a row of several chunks per warp and turn: half the
@@ -440,7 +525,7 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
     bool ok = true;
     for (uint32_t tile = blockIdx.x; ok && tile < G.num_tiles; tile += gridDim.x) {
       if (!mbar_wait(mfull_bar(slot), mpar, abort_flag)) break;
-      const TileMasks& tm = ring[slot];
+      const Masks& tm = ring[slot];
 #pragma unroll 1
       for (int pass = 0; pass < 2; ++pass) {
         if (pass == 1) {
@@ -471,30 +556,37 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
     // (chunk after chunk in the order (replica, chunk)); pass 1 takes their squared differences against the wire
     // tile: fp32 per lane within a replica's chunks, one warp reduction per replica and tile, fp64 from there on
     // (each replica has one accumulator, touched by this warp alone, in tile order).
-    auto row_pass = [&](const TileMasks& tm, uint32_t b, int pass, const unsigned char* wt) {
-      const uint64_t stale_l = tm.stale[lane & (kMaxSub - 1)];
-      const uint32_t j_l = tm.j[lane & (kMaxSub - 1)];
-      const uint32_t live_tile = (1u << tm.npk) - 1u;       // entries behind a short last tile are marked stale everywhere
+    auto row_pass = [&](const Masks& tm, uint32_t b, int pass, const unsigned char* wt) {
+      const uint64_t stale_l = tm.stale[lane & (kSub - 1)];
+      const uint32_t j_l = tm.j[lane & (kSub - 1)];
+      const uint32_t live_tile = (1u << tm.npk) - 1u;       // entries behind the tile's last sub-packet are marked stale everywhere
+      const uint32_t chunks_l = chunks_of(tm), phase = tm.phase;
       const uint64_t e0 = tm.e0;
       uint32_t n = 0;                                       // chunks with a stale sub-packet met so far (warp-uniform)
       for (uint32_t i = rw; i < W; i += kNR) {
-        const uint32_t live = __ballot_sync(0xFFFFFFFFu, (stale_l >> i) & 1ull) & 0xFFu & live_tile;
+        const bool st = (stale_l >> i) & 1ull;
+        const uint32_t live = __ballot_sync(0xFFFFFFFFu, st) & live_tile;
         if (live == 0u) continue;
-        const unsigned char* base = reinterpret_cast<const unsigned char*>(P.replicas[i]);
+        [[maybe_unused]] const uint32_t hit = kChunkWalk ? __reduce_or_sync(0xFFFFFFFFu, st ? chunks_l : 0u) : 0u;   // the row's chunks with a stale sub-packet
+        uint32_t behind;
+        const unsigned char* base = row_base(i, j_l, live_tile, e0, behind);
         float2 sq2 = make_float2(0.0f, 0.0f);                                 // two running sums (packed fp32 pairs of sm_100)
 #pragma unroll
         for (int c = 0; c < kChunks; ++c) {
-          const uint32_t el0 = (uint32_t)c * kElemsPerChunk;                    // the chunk's sub-packets, as bits
-          const uint32_t in_chunk = ((2u << ((el0 + kElemsPerChunk - 1u) >> lgP)) - 1u) & ~((1u << (el0 >> lgP)) - 1u);
-          if ((live & in_chunk) == 0u) continue;
+          if constexpr (kChunkWalk) {
+            if (!((hit >> c) & 1u)) continue;
+          } else {
+            const uint32_t el0 = (uint32_t)c * kElemsPerChunk;                    // the chunk's sub-packets, as bits
+            const uint32_t in_chunk = ((2u << ((el0 + kElemsPerChunk - 1u) >> lgP)) - 1u) & ~((1u << (el0 >> lgP)) - 1u);
+            if ((live & in_chunk) == 0u) continue;
+          }
           const uint32_t q = n++;
           const uint32_t off = (uint32_t)c * 512u + (uint32_t)lane * 16u;
-          const uint32_t el = off / kRB, sp = el >> lgP;
-          const uint32_t j_sp = __shfl_sync(0xFFFFFFFFu, j_l, (int)sp);
+          const uint32_t sp = sub_of(phase, off / kRB);
           const bool mine = (live >> sp) & 1u;                                  // this lane's 16 bytes are stale ones
           unsigned char* sc = scratch + (size_t)b * rd_buf + q * 512u + (uint32_t)lane * 16u;
           if (pass == 0) {
-            if (mine) cp_async16(smem_u32(sc), base + rep_index(P, i, j_sp, e0 + el) * kRB);
+            if (mine) cp_async16(smem_u32(sc), base + off - (behind && ((behind >> sp) & 1u) ? P.rep_skip[i] * kRB : 0ull));
           } else if (mine) {
             const uint4 ov = *reinterpret_cast<const uint4*>(sc);               // each lane reads back what it copied itself
             const uint4 wv = *reinterpret_cast<const uint4*>(wt + off);
@@ -540,27 +632,62 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
       }
       // the wire tile is complete: every compute warp has arrived, and each had waited for the tile's masks first
       if (!mbar_wait(wfull_bar(wslot), wpar, abort_flag)) break;
-      const TileMasks& tm = ring[slot];
+      const Masks& tm = ring[slot];
       const uint64_t e0 = tm.e0;
       const unsigned char* wt = wring + (size_t)wslot * kRowR;
-      // lane l holds sub-packet (l & 7)'s masks; a ballot per replica turns that column into the replica's row
-      const uint32_t j_l = tm.j[lane & (kMaxSub - 1)];
-      const uint64_t keep_l = tm.stale[lane & (kMaxSub - 1)] | own_bit(P, j_l);   // not written: missed the broadcast, or does not exist
-      uint32_t jc[kChunks];                                 // owner of the sub-packet this lane's bytes of chunk c lie in
+      // lane l holds sub-packet l mod kSub's masks; a ballot per replica turns that column into the replica's row
+      const uint32_t j_l = tm.j[lane & (kSub - 1)];
+      const uint64_t keep_l = tm.stale[lane & (kSub - 1)] | own_bit(P, j_l);   // not written: missed the broadcast, or does not exist
+      if constexpr (!kHoldWire) {
+        uint32_t jc[kChunks];                                 // owner of the sub-packet this lane's bytes of chunk c lie in
 #pragma unroll
-      for (int c = 0; c < kChunks; ++c)
-        jc[c] = __shfl_sync(0xFFFFFFFFu, j_l, (int)((((uint32_t)c * 512u + (uint32_t)lane * 16u) / kRB) >> lgP));
-      for (uint32_t i = rw; i < W; i += kNR) {
-        const uint32_t fresh = __ballot_sync(0xFFFFFFFFu, !((keep_l >> i) & 1ull)) & 0xFFu;   // bit sp: replica i takes it
-        if (fresh == 0u) continue;
-        unsigned char* base = reinterpret_cast<unsigned char*>(P.replicas[i]);
+        for (int c = 0; c < kChunks; ++c)
+          jc[c] = __shfl_sync(0xFFFFFFFFu, j_l, (int)((((uint32_t)c * 512u + (uint32_t)lane * 16u) / kRB) >> lgP));
+        for (uint32_t i = rw; i < W; i += kNR) {
+          const uint32_t fresh = __ballot_sync(0xFFFFFFFFu, !((keep_l >> i) & 1ull)) & 0xFFu;   // bit sp: replica i takes it
+          if (fresh == 0u) continue;
+          unsigned char* base = reinterpret_cast<unsigned char*>(P.replicas[i]);
 #pragma unroll
-        for (int c = 0; c < kChunks; ++c) {
-          const uint32_t off = (uint32_t)c * 512u + (uint32_t)lane * 16u;
-          const uint32_t el = off / kRB;
-          if ((fresh >> (el >> lgP)) & 1u)
-            __stcs(reinterpret_cast<uint4*>(base + rep_index(P, i, jc[c], e0 + el) * kRB),
-                   *reinterpret_cast<const uint4*>(wt + off));
+          for (int c = 0; c < kChunks; ++c) {
+            const uint32_t off = (uint32_t)c * 512u + (uint32_t)lane * 16u;
+            const uint32_t el = off / kRB;
+            if ((fresh >> (el >> lgP)) & 1u)
+              __stcs(reinterpret_cast<uint4*>(base + rep_index(P, i, jc[c], e0 + el) * kRB),
+                     *reinterpret_cast<const uint4*>(wt + off));
+          }
+        }
+      } else {
+        uint32_t sub_c[kChunks];                              // the sub-packet this lane's bytes of chunk c lie in
+        const uint32_t live_tile = (1u << tm.npk) - 1u;
+#pragma unroll
+        for (int c = 0; c < kChunks; ++c) sub_c[c] = sub_of(tm.phase, ((uint32_t)c * 512u + (uint32_t)lane * 16u) / kRB);
+        // Four chunks of the wire tile at a time in registers, for all of this warp's replicas: read again for every replica
+        // they are a shared-memory round trip before each store (fp32, W = 4, P = 512, p = 0.1: 0.81 -> 0.94 of the copy
+        // rate)
+        constexpr int kHold = 4;
+#pragma unroll
+        for (int c0 = 0; c0 < kChunks; c0 += kHold) {
+          const uint32_t from = smem_u32(wt) + (uint32_t)lane * 16u + c0 * 512u;
+          uint4 v[kHold];
+#pragma unroll
+          for (int c = 0; c < kHold; ++c) v[c] = lds_here(from + c * 512u);
+          for (uint32_t i = rw; i < W; i += kNR) {
+            const uint32_t fresh = __ballot_sync(0xFFFFFFFFu, !((keep_l >> i) & 1ull)) & kSubBits;   // bit sp: replica i takes it
+            if (fresh == 0u) continue;
+            uint32_t behind;
+            unsigned char* base = row_base(i, j_l, live_tile, e0, behind) + (uint32_t)lane * 16u + c0 * 512u;
+            if (behind == 0u) {
+#pragma unroll
+              for (int c = 0; c < kHold; ++c)
+                if ((fresh >> sub_c[c0 + c]) & 1u) __stcs(reinterpret_cast<uint4*>(base + c * 512), v[c]);
+            } else {
+              const uint64_t skip = P.rep_skip[i] * kRB;
+#pragma unroll
+              for (int c = 0; c < kHold; ++c)
+                if ((fresh >> sub_c[c0 + c]) & 1u)
+                  __stcs(reinterpret_cast<uint4*>(base + c * 512 - ((behind >> sub_c[c0 + c]) & 1u ? skip : 0ull)), v[c]);
+            }
+          }
         }
       }
       if constexpr (kReadsStale) {
@@ -580,8 +707,9 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
   } else {
     // =============================== compute warps ===============================
     const uint32_t idx = threadIdx.x * kEpl;               // first element of this lane within the tile
-    const uint32_t my_sp = ((uint32_t)(threadIdx.x & ~31) * kEpl) >> lgP;   // this warp's sub-packet, always the same
+    const uint32_t idx_w = (uint32_t)(threadIdx.x & ~31) * kEpl;           // first element of this warp: its 128 elements lie in at most two packets
     uint32_t s = 0, par = 0, slot = 0, mpar = 0, wslot = 0, wpar = 0;
+    uint32_t my_sp = idx_w >> lgP;                          // this lane's sub-packet, always the same unless ANY
     bool ok = true;
     float acc[kEpl];
     auto next_stage = [&]() { if (++s == S) { s = 0; par ^= 1u; } };
@@ -592,30 +720,35 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
     constexpr int kPre = 4;
     for (uint32_t tile = blockIdx.x; ok && tile < G.num_tiles; tile += gridDim.x) {
       if (!mbar_wait(mfull_bar(slot), mpar, abort_flag)) { ok = false; break; }
-      const TileMasks& tm = ring[slot];
+      const Masks& tm = ring[slot];
       const uint32_t len = tm.len;
       const uint64_t e0 = tm.e0;
       const bool active = idx < len;
+      if constexpr (ANY) my_sp = sub_of(tm.phase, idx);
       const uint64_t my_recv = tm.recv[my_sp];             // zero behind a short last tile
       // The old copies this warp compares against for the drift term (in L2 by now: the mask warp asked for them
       // tiles ago) are requested first, so that their latency hides behind the wait for the tile and its arithmetic.
       [[maybe_unused]] uint32_t pre_raw[kPre][4];
       [[maybe_unused]] uint64_t early = 0;                 // the replicas whose copies were requested early
       [[maybe_unused]] uint32_t my_j = 0;
-      uint64_t stale_rest = 0;
+      [[maybe_unused]] uint64_t my_stale = 0;              // the replicas that miss this lane's sub-packet ...
+      uint64_t stale_rest = 0;                             // ... and those that miss one of the warp's (warp-uniform)
       if constexpr (kWarpDrift) {
         if (active) {
-          stale_rest = tm.stale[my_sp];
+          my_stale = tm.stale[my_sp];
           my_j = tm.j[my_sp];
         }
+        if (!ANY) stale_rest = my_stale;
+        else if (idx_w < len) stale_rest = tm.stale[__shfl_sync(0xFFFFFFFFu, my_sp, 0)] | tm.stale[min(__shfl_sync(0xFFFFFFFFu, my_sp, 31), tm.npk - 1u)];
 #pragma unroll
         for (int b = 0; b < kPre; ++b) {
           if (stale_rest) {
             const int id = __ffsll((long long)stale_rest) - 1;
             stale_rest &= stale_rest - 1;
             early |= 1ull << id;
-            load_words_stream<kWords>(reinterpret_cast<const typename RT::raw*>(P.replicas[id]) +
-                                          rep_index(P, (uint32_t)id, my_j, e0 + idx), pre_raw[b]);
+            if (!ANY || ((my_stale >> id) & 1ull))
+              load_words_stream<kWords>(reinterpret_cast<const typename RT::raw*>(P.replicas[id]) +
+                                            rep_index(P, (uint32_t)id, my_j, e0 + idx), pre_raw[b]);
           }
         }
       }
@@ -660,7 +793,7 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
               for (int x = 1; x < 4; ++x) id = b == x ? ids[x] : id;
               if ((lane & 7) == 0 && id >= 0) warp_acc[warp * kMaxW + id] += (double)tot;
             };
-            if (early) {              // warp-uniform: the warp's elements lie in one sub-packet
+            if (early) {              // warp-uniform
               float sq[4];
 #pragma unroll
               for (int b0 = 0; b0 < kPre; b0 += 4) {
@@ -673,12 +806,14 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
                   if (early) {
                     ids[b] = __ffsll((long long)early) - 1;
                     early &= early - 1;
-                    float old[kEpl];
-                    unpack_lane<RT>(pre_raw[b0 + b], old);
+                    if (!ANY || ((my_stale >> ids[b]) & 1ull)) {
+                      float old[kEpl];
+                      unpack_lane<RT>(pre_raw[b0 + b], old);
 #pragma unroll
-                    for (int x = 0; x < kEpl; ++x) {
-                      const float d = __fsub_rn(old[x], wire[x]);
-                      sq[b] = __fadd_rn(sq[b], __fmul_rn(d, d));
+                      for (int x = 0; x < kEpl; ++x) {
+                        const float d = __fsub_rn(old[x], wire[x]);
+                        sq[b] = __fadd_rn(sq[b], __fmul_rn(d, d));
+                      }
                     }
                   }
                 }
@@ -693,14 +828,15 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
                   if (stale_rest) {
                     ids[b] = __ffsll((long long)stale_rest) - 1;
                     stale_rest &= stale_rest - 1;
-                    load_words_stream<kWords>(reinterpret_cast<const typename RT::raw*>(P.replicas[ids[b]]) +
-                                                  rep_index(P, (uint32_t)ids[b], my_j, e0 + idx), raw[b]);
+                    if (!ANY || ((my_stale >> ids[b]) & 1ull))
+                      load_words_stream<kWords>(reinterpret_cast<const typename RT::raw*>(P.replicas[ids[b]]) +
+                                                    rep_index(P, (uint32_t)ids[b], my_j, e0 + idx), raw[b]);
                   }
                 }
 #pragma unroll
                 for (int b = 0; b < 4; ++b) {
                   sq[b] = 0.0f;
-                  if (ids[b] >= 0) {
+                  if (ids[b] >= 0 && (!ANY || ((my_stale >> ids[b]) & 1ull))) {
                     float old[kEpl];
                     unpack_lane<RT>(raw[b], old);
 #pragma unroll

@@ -64,6 +64,7 @@ struct TmaGeom {
   uint32_t full_packets;      // PACKED build: complete packets of the bucket
   uint32_t rd_cap;            // gather pipeline, RD builds: 512-byte chunks per scratch buffer
   uint32_t rd_lgsplit;        // gather pipeline, wide RD builds: log2 of the parts a replica's row of a tile is cut into
+  uint32_t magic;             // gather pipeline: 2^32 / P rounded up (x / P = umulhi(x, magic) while x P < 2^32)
   uint32_t* status;           // device status word (0 = fine)
 };
 

@@ -1,0 +1,72 @@
+"""The gather pipeline on packets that do not divide its tile: a tile starts anywhere in a packet, a packet may span two
+tiles, a warp's elements two packets. Against the oracle element by element, and against the register kernel bit for bit
+on everything that has one right value."""
+import pytest
+import torch
+
+import paper_2507_07114_b200 as L
+import workload
+from parity_util import GpuRun, run_parity
+
+pytestmark = pytest.mark.gpu
+ELIDE, REG, GATHER, SKIP, LOSSLESS = (L.LOSSY_REPLICA_SKIP_OWNER, L.LOSSY_REGISTER_PATH, L.LOSSY_GATHER_PATH,
+                                      L.LOSSY_ZERO_SKIP, L.LOSSY_SELF_LOSSLESS)
+
+CASES = [
+    # name, W, n, P, p, opt, gd, rd, flags
+    ("ethernet_w8", 8, 736 * 61 + 100, 736, 0.1, "adam", "bf16", "bf16", 0),
+    ("ethernet_w16_heavy", 16, 736 * 41, 736, 0.3, "adam", "bf16", "bf16", 0),
+    ("shortest_136", 6, 136 * 200 + 8, 136, 0.2, "adam", "bf16", "bf16", 0),
+    ("shortest_136_w4", 4, 136 * 100, 136, 0.3, "sgd", "f32", "f32", 0),
+    ("longest_1016_w3", 3, 1016 * 30 + 3, 1016, 0.3, "adam", "bf16", "f32", 0),
+    ("longest_1016_w12", 12, 1016 * 25, 1016, 0.25, "sgd", "f32", "bf16", 0),
+    ("w2_twin_f32", 2, 200 * 90, 200, 0.4, "adam", "f32", "f32", SKIP),
+    ("w40_two_packets_per_warp", 40, 136 * 77 + 16, 136, 0.05, "adam", "bf16", "bf16", 0),
+    ("w24_early_and_late_copies", 24, 264 * 60, 264, 0.12, "sgd", "bf16", "bf16", GATHER),
+    ("w64_f32_replicas", 64, 520 * 30 + 8, 520, 0.2, "adam", "bf16", "f32", GATHER),
+    ("drift_warps_quarters_w5", 5, 312 * 80, 312, 0.4, "adam", "bf16", "bf16", 0),
+    ("drift_warps_scratch_overflow_w24", 24, 328 * 70, 328, 0.3, "adam", "bf16", "bf16", GATHER),
+    ("one_packet", 8, 1000, 1000, 0.3, "adam", "bf16", "bf16", 0),
+    ("less_than_a_tile", 9, 304 * 3 + 8, 304, 0.3, "adam", "bf16", "bf16", LOSSLESS),
+    ("nothing_received", 2, 248 * 300, 248, 0.7, "adam", "bf16", "bf16", SKIP),
+]
+
+
+@pytest.mark.parametrize("case", CASES, ids=[c[0] for c in CASES])
+@pytest.mark.parametrize("elided", [0, ELIDE], ids=["full", "elided"])
+def test_packets_that_do_not_divide_the_tile(case, elided):
+    name, W, n, P, p, opt, gd, rd, flags = case
+    w = workload.Workload(name, W, n, P, p, opt, 1e-2 if opt == "sgd" else 3e-4, gd, rd, 4, seed=31)
+    gpu, orc = run_parity(w, 4, flags=flags | elided)
+    assert L.lossy_describe_plan(gpu.ctx).startswith("gather"), L.lossy_describe_plan(gpu.ctx)
+    if name == "nothing_received":
+        assert int((gpu.count == 0).sum()) > 0
+
+
+@pytest.mark.parametrize("W,P,gd,rd", [(8, 736, "bf16", "bf16"), (3, 184, "f32", "f32"), (20, 904, "bf16", "bf16"), (7, 296, "f32", "bf16")])
+@pytest.mark.parametrize("mode", ["plain", "alg1", "bursty", "range"])
+def test_gather_equals_the_register_kernel(W, P, gd, rd, mode):
+    """Whole tiles and ring turns (more tiles than CTAs), every optional output, Algorithm 1's aggregate, bursty links and
+    a packet range that starts inside a shard: state, masks and outputs are the same bits; the norms are the same numbers
+    in another order (fp32 sums of up to 2048 squares, 12 * 2^-24 each way, then fp64)."""
+    n = P * (148 * 2048 * 5 // 2 // P) + 40
+    K = -(-n // P)
+    w = workload.Workload("any_packet", W, n, P, 0.2, "adam", 3e-4, gd, rd, 3, seed=5)
+    kw = {"alg1": mode == "alg1", "burst": (0.1, 0.4) if mode == "bursty" else None}
+    if mode == "range":
+        kw.update(shard_packet0=3 * K // 2 + 1, bucket_packets=3 * K // 2 + 1 + K)
+    a, b = GpuRun(w, flags=GATHER, **kw), GpuRun(w, flags=REG, **kw)
+    assert L.lossy_describe_plan(a.ctx).startswith("gather") and L.lossy_describe_plan(b.ctx).startswith("register")
+    for t in range(1, 4):
+        gd_ = [workload.grad_slab(w, t, i, 0, n, "cuda") for i in range(W)]
+        a.step_fused(t, gd_)
+        b.step_fused(t, gd_)
+    torch.cuda.synchronize()
+    L.lossy_device_status(a.ctx)
+    for x in ("master", "m", "v", "ghat", "count", "recv", "stale") + (("ghat_prev",) if mode == "alg1" else ()):
+        assert torch.equal(getattr(a, x), getattr(b, x)), x
+    for i in range(W):
+        assert torch.equal(a.replicas[i], b.replicas[i]), i
+    if mode == "bursty":
+        assert torch.equal(a.burst_state, b.burst_state)
+    assert torch.allclose(a.norms, b.norms, rtol=2e-6, atol=0)
