@@ -35,6 +35,7 @@ template <class GT, bool MANY>
 static __global__ void __launch_bounds__(256) packet_sqnorms_kernel(const __grid_constant__ SqnormArgs A) {
   const int lane = threadIdx.x & 31;
   const uint32_t i = blockIdx.y;
+  wait_for_previous();
   const void* grads = A.grads[i];
   const uint32_t warps = gridDim.x * (blockDim.x >> 5), warp0 = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   auto add = [](float s, const Vec8<GT>& raw, int nvalid) {
@@ -165,6 +166,7 @@ static __global__ void __launch_bounds__(128) drift_pairwise_few_kernel(const __
 #pragma unroll
   for (int x = 0; x < kPairs; ++x) acc[x] = 0.0;
   uint32_t bad = 0;                                       // replicas seen to hold an infinity or NaN: x - x is NaN
+  wait_for_previous();
   const uint64_t total = (uint64_t)A.segs * A.chunks_per_seg;
   for (uint64_t q = (uint64_t)blockIdx.x * 4u + warp; q < total; q += (uint64_t)gridDim.x * 4u) {
     const uint32_t seg = ELIDE ? (uint32_t)q / A.chunks_per_seg : 0u, j = A.seg0 + seg;
@@ -265,6 +267,7 @@ static __global__ void __launch_bounds__(PairShape<M, SMALL>::kMaxWarps * 32, 1)
   unsigned char* slots = pair_smem + (size_t)warp * wb + (nt * 8u + 15u) / 16u * 16u;
   volatile uint32_t* slot_id = reinterpret_cast<volatile uint32_t*>(slots + kPairSlots * kChunk * kRB);
   for (uint32_t q = lane; q < nt; q += 32) tab[q] = 0.0;
+  wait_for_previous();
   __syncwarp();
   M bad_diag = 0;                                         // replicas seen to hold an infinity or NaN: x - x is NaN
   const M everyone = W == sizeof(M) * 8 ? ~(M)0 : ((M)1 << W) - 1;
