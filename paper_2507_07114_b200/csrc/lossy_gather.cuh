@@ -899,17 +899,12 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
     }
   }
 
-  // ---- common exit: per-CTA drift partials in fixed order, status word ---------------
-  __syncthreads();
-  if (*abort_flag && threadIdx.x == 0) atomicExch(G.status, 1u);
+  // ---- common exit: status word, per-CTA drift partials in fixed order ---------------
+  if (lane == 0 && *abort_flag) atomicExch(G.status, 1u);   // (the warp that raised the flag sees it)
   if constexpr (DRIFTK) {
-    if (threadIdx.x < kMaxW) {
-      double t = 0.0;
-#pragma unroll
-      for (int w = 0; w < kAccRows; ++w) t += warp_acc[w * kMaxW + threadIdx.x];
-      P.partials[(size_t)blockIdx.x * kMaxW + threadIdx.x] = t;
-    }
-    if (P.ticket) drift_last_block(P, warp, lane, GatherShape<CW, RD>::kThreads / 32);
+    constexpr int kStoreWarp = CW + kNP + 1;
+    if (warp == kStoreWarp) return;
+    drift_finish(P, warp_acc, kAccRows, blockIdx.x, warp < kStoreWarp ? warp : warp - 1, GatherShape<CW, RD>::kThreads / 32 - 1, lane);
   }
 }
 

@@ -49,32 +49,52 @@ __device__ __forceinline__ void optimizer8(const Params& P, const float (&g)[8],
   optimizer_n<OPT, 8>(P, g, th, m, v);
 }
 
-// Last-block drift finalisation. Every block has stored its row of `partials`; the block that draws the
-// last ticket sums the rows of each replica in a fixed order (lane l takes rows l, l+32, ..., then a shuffle
-// tree), so the result does not depend on which block happens to be last. Nothing here waits on another
-// block. Call with all threads of the block; `nwarps` warps share the replicas.
-__device__ __forceinline__ void drift_last_block(const Params& P, int warp, int lane, int nwarps) {
+// The end of a kernel with drift norms. The `nwarps` warps that call this have left their sums of squares in shared
+// memory, `rows` rows of kMaxW; the first of them adds the rows up and stores the block's row of `partials`, and the block
+// that draws the last ticket sums the rows of each replica in a fixed order (lane l takes rows l, l + 32, ..., then a shuffle
+// tree), so the result does not depend on which block happens to be last. Nothing here waits on another block.
+// This is the tail of every step, a chain of latencies (2 us), so only one warp fences, behind nothing but its own stores,
+// the warp that drains the bulk stores is not waited for, and a lane's rows are requested together.
+__device__ __forceinline__ void drift_finish(const Params& P, const double* sums, int rows, uint32_t row, int warp, int nwarps, int lane) {
   __shared__ uint32_t is_last;
-  __threadfence();                       // this block's partial row is visible device-wide ...
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const uint32_t prev = atomicAdd(P.ticket, 1u);   // ... before its ticket is
-    is_last = prev + 1u == P.total_rows ? 1u : 0u;
+  auto sync = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(nwarps * 32) : "memory"); };
+  sync();
+  if (warp == 0) {
+    double t0 = 0.0, t1 = 0.0;
+    for (int w = 0; w < rows; ++w) {
+      t0 += sums[w * kMaxW + lane];
+      t1 += sums[w * kMaxW + lane + 32];
+    }
+    double* out = P.partials + (size_t)row * kMaxW;
+    out[lane] = t0;
+    out[lane + 32] = t1;
+    __syncwarp();
+    if (P.ticket && lane == 0) {
+      __threadfence();                                // the warp's row is visible device-wide ...
+      const uint32_t prev = atomicAdd(P.ticket, 1u);  // ... before its ticket is
+      __threadfence();
+      is_last = prev + 1u == P.total_rows ? 1u : 0u;
+    }
   }
-  __syncthreads();
+  if (!P.ticket) return;
+  sync();
   if (!is_last) return;
-  __threadfence();
   for (uint32_t i = warp; i < P.W; i += nwarps) {
     double t = 0.0;
-    for (uint32_t b = lane; b < P.total_rows; b += 32) t += __ldcg(&P.partials[(size_t)b * kMaxW + i]);
+    for (uint32_t b0 = lane; b0 < P.total_rows; b0 += 32 * 5) {
+      double x[5];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
+      for (int u = 0; u < 5; ++u) x[u] = b0 + 32u * u < P.total_rows ? __ldcg(&P.partials[(size_t)(b0 + 32u * u) * kMaxW + i]) : 0.0;
+#pragma unroll
+      for (int u = 0; u < 5; ++u) t += x[u];
+    }
+    t = warp_sum64(t);
     if (lane == 0) {
       if (P.sumsq) P.sumsq[i] += t;
       if (P.norms) P.norms[i] = (float)sqrt(t);
     }
   }
-  if (threadIdx.x == 0) *P.ticket = 0u;  // ready for the next call on this context
+  if (warp == 0 && lane == 0) *P.ticket = 0u;  // ready for the next call on this context
 }
 
 // Delivery indicators of packet k (owner j), evaluated one worker per lane and gathered by ballot:
@@ -409,17 +429,10 @@ __global__ void __launch_bounds__(kThreads, LOSSY_MIN_BLOCKS) lossy_kernel(const
 
   // ---- per-block drift partials, fixed order ------------------------------------
   if constexpr (PH & DRIFT) {
-    __shared__ double sh[kWarps][kMaxW];
-    sh[warp][lane] = dacc0;
-    sh[warp][lane + 32] = dacc1;
-    __syncthreads();
-    if (threadIdx.x < kMaxW) {
-      double t = 0.0;
-#pragma unroll
-      for (int w = 0; w < kWarps; ++w) t += sh[w][threadIdx.x];
-      P.partials[(size_t)(P.partials_row0 + blockIdx.x) * kMaxW + threadIdx.x] = t;
-    }
-    if (P.ticket) drift_last_block(P, warp, lane, kWarps);
+    __shared__ double sh[kWarps * kMaxW];
+    sh[warp * kMaxW + lane] = dacc0;
+    sh[warp * kMaxW + lane + 32] = dacc1;
+    drift_finish(P, sh, kWarps, P.partials_row0 + blockIdx.x, warp, kWarps, lane);
   }
   if constexpr (TAIL) asm volatile("griddepcontrol.wait;" ::: "memory");
 }

@@ -353,22 +353,15 @@ __global__ void __launch_bounds__(TmaShape<CW>::kThreads, TmaShape<CW>::kCtasPer
   }
 
   // ---- common exit: status word; per-CTA drift partials in fixed order ----------------
-  __syncthreads();
-  if (*abort_flag && threadIdx.x == 0) atomicExch(G.status, 1u);
+  if (lane == 0 && *abort_flag) atomicExch(G.status, 1u);   // (the warp that raised the flag sees it)
   if constexpr (PH == DRIFT) {
+    __syncthreads();
     double* sh = reinterpret_cast<double*>(stage0);   // stages are idle now
     if (warp < kConsumerWarps) {
       sh[warp * kMaxW + lane] = dacc0;
       sh[warp * kMaxW + lane + 32] = dacc1;
     }
-    __syncthreads();
-    if (threadIdx.x < kMaxW) {
-      double t = 0.0;
-#pragma unroll
-      for (int w = 0; w < kConsumerWarps; ++w) t += sh[w * kMaxW + threadIdx.x];
-      P.partials[((size_t)P.partials_row0 + blockIdx.x) * kMaxW + threadIdx.x] = t;
-    }
-    if (P.ticket) drift_last_block(P, warp, lane, kConsumerWarps + 2);
+    drift_finish(P, sh, kConsumerWarps, P.partials_row0 + blockIdx.x, warp, kConsumerWarps + 2, lane);
   }
 }
 

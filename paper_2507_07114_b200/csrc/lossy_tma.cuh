@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(TmaShape<CW>::kThreads, TmaShape<CW>::kCtasPer
   const uint32_t S = G.stages;
   // SPLIT builds: two state slots behind the stages
   unsigned char* state0 = stage0 + (size_t)S * G.stage_bytes;
-  // stale-stage builds: fp64 drift sums per compute warp and replica, behind everything else
+  // fp64 drift sums per compute warp and replica, behind everything else
   double* warp_acc = reinterpret_cast<double*>(state0 + (SPLIT ? 2u * G.state_bytes : 0u));
   const uint32_t off_th = SPLIT ? 0u : G.grad_slots * kTile * kGB;   // within the stage, or within the state slot
   const uint32_t off_m = off_th + kTile * 4, off_v = off_m + kTile * 4, off_wire = off_v + kTile * 4;
@@ -901,25 +901,17 @@ __global__ void __launch_bounds__(TmaShape<CW>::kThreads, TmaShape<CW>::kCtasPer
     }
   }
 
-  // ---- common exit: per-CTA drift partials in fixed order, status word ---------------
-  __syncthreads();
-  if (*abort_flag && threadIdx.x == 0) atomicExch(G.status, 1u);
+  // ---- common exit: status word, per-CTA drift partials in fixed order ---------------
+  if (lane == 0 && *abort_flag) atomicExch(G.status, 1u);   // (the warp that raised the flag sees it)
   if constexpr (DRIFTK) {
-    double* sh = kStaleStages ? warp_acc : reinterpret_cast<double*>(stage0);   // stages are idle now
+    if (warp == kConsumerWarps + 1) return;                   // the store warp
     if constexpr (!kStaleStages) {
       if (warp < kConsumerWarps) {
-        sh[warp * kMaxW + lane] = dacc0;
-        sh[warp * kMaxW + lane + 32] = dacc1;
+        warp_acc[warp * kMaxW + lane] = dacc0;
+        warp_acc[warp * kMaxW + lane + 32] = dacc1;
       }
-      __syncthreads();
     }
-    if (threadIdx.x < kMaxW) {
-      double t = 0.0;
-#pragma unroll
-      for (int w = 0; w < kConsumerWarps; ++w) t += sh[w * kMaxW + threadIdx.x];
-      P.partials[(size_t)blockIdx.x * kMaxW + threadIdx.x] = t;
-    }
-    if (P.ticket) drift_last_block(P, warp, lane, kConsumerWarps + 2);
+    drift_finish(P, warp_acc, kConsumerWarps, blockIdx.x, warp, kConsumerWarps + 1, lane);
   }
 }
 
