@@ -71,7 +71,7 @@ __device__ __forceinline__ void cp_async_arrive(uint32_t bar) {
 }
 
 // A shared-memory load that stays where it is written (the compiler otherwise moves a wire tile's worth of them out of
-// the loop over the replicas, and spills them)
+// the loop over the replicas)
 __device__ __forceinline__ uint4 lds_here(uint32_t src) {
   uint4 v;
   asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(src));
@@ -142,11 +142,6 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
   constexpr int kSub = ANY ? kAnySub : kMaxSub;
   constexpr uint32_t kSubBits = (1u << kSub) - 1u;
   using Masks = TileMasks<kSub>;
-  // How the replica warps store (see there). Of the builds for packets that divide the tile only the wide ones for fp32
-  // replicas hold the wire tile in registers (W = 5, P = 512, p = 0.1: 1.32 times as fast); a bf16 row is eight chunks, and
-  // visiting every replica twice for four of them costs more than the second read saves (W = 8, P = 512, p = 0.05: 0.955,
-  // W = 12, P = 256, p = 0.1: 0.925), as it does in the twin builds (W = 40, P = 128: 0.79 against 0.85 of the copy rate).
-  constexpr bool kHoldWire = ANY || (CW >= 16 && RT::kVecs == 2);
   constexpr bool kLaneWide = ANY && RT::kVecs == 2;        // stale rows: lane sums widened after each chunk
   constexpr bool kWarpDrift = DRIFTK && !RD;               // the compute warps read the stale copies
   constexpr int kTile = GatherShape<CW, RD>::kTile;
@@ -679,56 +674,24 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
       // lane l holds sub-packet l mod kSub's masks; a ballot per replica turns that column into the replica's row
       const uint32_t j_l = tm.j[lane & (kSub - 1)];
       const uint64_t keep_l = tm.stale[lane & (kSub - 1)] | own_bit(P, j_l);   // not written: missed the broadcast, or does not exist
-      if constexpr (!kHoldWire) {
-        uint32_t jc[kChunks];                                 // owner of the sub-packet this lane's bytes of chunk c lie in
+      uint32_t sub_c[kChunks];                                // the sub-packet this lane's bytes of chunk c lie in
+      const uint32_t live_tile = (1u << tm.npk) - 1u;
+#pragma unroll
+      for (int c = 0; c < kChunks; ++c) sub_c[c] = sub_of(tm.phase, ((uint32_t)c * 512u + (uint32_t)lane * 16u) / kRB);
+      const uint32_t from = smem_u32(wt) + (uint32_t)lane * 16u;
+      for (uint32_t i = rw; i < W; i += kNR) {
+        const uint32_t fresh = __ballot_sync(0xFFFFFFFFu, !((keep_l >> i) & 1ull)) & kSubBits;   // bit sp: replica i takes it
+        if (fresh == 0u) continue;
+        uint32_t behind;
+        unsigned char* base = row_base(i, j_l, live_tile, e0, behind) + (uint32_t)lane * 16u;
+        const uint64_t skip = behind ? P.rep_skip[i] * kRB : 0ull;
+        // One ballot and one base per row, and the wire tile read where it is stored, each read in front of its store: with four
+        // chunks of it held in registers every row was visited two to four times (W = 8, P = 736, p = 0.1, 135 M elements:
+        // 1245 us, this 1191; W = 4, P = 512, fp32, 67 M: 628 and 584), with eight there were no registers left (1280).
 #pragma unroll
         for (int c = 0; c < kChunks; ++c)
-          jc[c] = __shfl_sync(0xFFFFFFFFu, j_l, (int)((((uint32_t)c * 512u + (uint32_t)lane * 16u) / kRB) >> lgP));
-        for (uint32_t i = rw; i < W; i += kNR) {
-          const uint32_t fresh = __ballot_sync(0xFFFFFFFFu, !((keep_l >> i) & 1ull)) & 0xFFu;   // bit sp: replica i takes it
-          if (fresh == 0u) continue;
-          unsigned char* base = reinterpret_cast<unsigned char*>(P.replicas[i]);
-#pragma unroll
-          for (int c = 0; c < kChunks; ++c) {
-            const uint32_t off = (uint32_t)c * 512u + (uint32_t)lane * 16u;
-            const uint32_t el = off / kRB;
-            if ((fresh >> (el >> lgP)) & 1u)
-              __stcs(reinterpret_cast<uint4*>(base + rep_index(P, i, jc[c], e0 + el) * kRB),
-                     *reinterpret_cast<const uint4*>(wt + off));
-          }
-        }
-      } else {
-        uint32_t sub_c[kChunks];                              // the sub-packet this lane's bytes of chunk c lie in
-        const uint32_t live_tile = (1u << tm.npk) - 1u;
-#pragma unroll
-        for (int c = 0; c < kChunks; ++c) sub_c[c] = sub_of(tm.phase, ((uint32_t)c * 512u + (uint32_t)lane * 16u) / kRB);
-        // Four chunks of the wire tile at a time in registers, for all of this warp's replicas: read again for every replica
-        // they are a shared-memory round trip before each store (fp32, W = 4, P = 512, p = 0.1: 1.15-1.2 times as fast)
-        constexpr int kHold = 4;
-#pragma unroll
-        for (int c0 = 0; c0 < kChunks; c0 += kHold) {
-          const uint32_t from = smem_u32(wt) + (uint32_t)lane * 16u + c0 * 512u;
-          uint4 v[kHold];
-#pragma unroll
-          for (int c = 0; c < kHold; ++c) v[c] = lds_here(from + c * 512u);
-          for (uint32_t i = rw; i < W; i += kNR) {
-            const uint32_t fresh = __ballot_sync(0xFFFFFFFFu, !((keep_l >> i) & 1ull)) & kSubBits;   // bit sp: replica i takes it
-            if (fresh == 0u) continue;
-            uint32_t behind;
-            unsigned char* base = row_base(i, j_l, live_tile, e0, behind) + (uint32_t)lane * 16u + c0 * 512u;
-            if (behind == 0u) {
-#pragma unroll
-              for (int c = 0; c < kHold; ++c)
-                if ((fresh >> sub_c[c0 + c]) & 1u) __stcs(reinterpret_cast<uint4*>(base + c * 512), v[c]);
-            } else {
-              const uint64_t skip = P.rep_skip[i] * kRB;
-#pragma unroll
-              for (int c = 0; c < kHold; ++c)
-                if ((fresh >> sub_c[c0 + c]) & 1u)
-                  __stcs(reinterpret_cast<uint4*>(base + c * 512 - ((behind >> sub_c[c0 + c]) & 1u ? skip : 0ull)), v[c]);
-            }
-          }
-        }
+          if ((fresh >> sub_c[c]) & 1u)
+            __stcs(reinterpret_cast<uint4*>(base + c * 512 - ((behind >> sub_c[c]) & 1u ? skip : 0ull)), lds_here(from + c * 512u));
       }
       if constexpr (kReadsStale) {
         asm volatile("cp.async.wait_group 1;" ::: "memory");   // everything but the next tile's requests has landed
