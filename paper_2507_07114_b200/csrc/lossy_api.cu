@@ -140,6 +140,7 @@ void fill_common(const lossy_ctx* ctx, uint64_t step, Params& P) {
   P.ibc1 = (float)(1.0 / (1.0 - pow((double)c.beta1, (double)step)));
   P.ibc2 = (float)(1.0 / (1.0 - pow((double)c.beta2, (double)step)));
   P.eps = c.eps;
+  P.neg_zero = -0.0f;
   P.partials = ctx->partials;
   P.K = (uint32_t)ctx->K;
   P.reliable = ctx->reliable;

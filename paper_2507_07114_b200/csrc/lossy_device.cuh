@@ -67,6 +67,7 @@ struct Params {
   uint32_t flags;
   uint32_t prefetch_next; // register kernel: L2-prefetch the warp's next chunk
   float lr, b1, b2, omb1, omb2, ibc1, ibc2, eps;
+  float neg_zero;         // -0 (optimizer_n)
   // Owner-elided replicas (kSkipOwner): replica i stores this context's elements WITHOUT the packets worker i
   // owns, so everything behind worker i's shard sits rep_skip[i] elements lower in its array. All zero otherwise.
   uint64_t rep_skip[kMaxW];
@@ -254,6 +255,43 @@ __device__ __forceinline__ void widen(const Vec8<T>& v, float (&f)[8]) {
       f[2 * i] = __uint_as_float(w[i] << 16);
       f[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
     }
+  }
+}
+// f += the two elements of a word, f - the two elements, and the elements - f, for bf16 elements: the sum of an fp32 and a
+// widened bf16 value is one instruction of sm_100 (exact widening, one rounding), so nothing is unpacked first.
+__device__ __forceinline__ void add_pair_bf16(uint32_t w, float& a, float& b) {
+  asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tadd.rn.f32.bf16 %0, lo, %0;\n\tadd.rn.f32.bf16 %1, hi, %1;\n\t}" : "+f"(a), "+f"(b) : "r"(w));
+}
+__device__ __forceinline__ float2 pair_minus_bf16(uint32_t w, float a, float b) {
+  float2 d;
+  asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tsub.rn.f32.bf16 %0, lo, %3;\n\tsub.rn.f32.bf16 %1, hi, %4;\n\t}" : "=f"(d.x), "=f"(d.y) : "r"(w), "f"(a), "f"(b));
+  return d;
+}
+// acc += the 8 elements of v
+template <class T>
+__device__ __forceinline__ void add8(const Vec8<T>& v, float (&acc)[8]) {
+  const uint32_t* w = reinterpret_cast<const uint32_t*>(&v.q[0]);
+#pragma unroll
+  for (int x = 0; x < 8; x += 2) {
+    if constexpr (T::kVecs == 2) {
+      const float2 s = __fadd2_rn(make_float2(acc[x], acc[x + 1]), make_float2(__uint_as_float(w[x]), __uint_as_float(w[x + 1])));
+      acc[x] = s.x;
+      acc[x + 1] = s.y;
+    } else {
+      add_pair_bf16(w[x / 2], acc[x], acc[x + 1]);
+    }
+  }
+}
+// d = the 8 elements of v minus x
+template <class T>
+__device__ __forceinline__ void minus8(const Vec8<T>& v, const float (&x)[8], float (&d)[8]) {
+  const uint32_t* w = reinterpret_cast<const uint32_t*>(&v.q[0]);
+#pragma unroll
+  for (int y = 0; y < 8; y += 2) {
+    const float2 s = T::kVecs == 2 ? __fadd2_rn(make_float2(__uint_as_float(w[y]), __uint_as_float(w[(y + 1) % (4 * T::kVecs)])), make_float2(-x[y], -x[y + 1]))
+                                   : pair_minus_bf16(w[y / 2], x[y], x[y + 1]);
+    d[y] = s.x;
+    d[y + 1] = s.y;
   }
 }
 // narrow 8 fp32 values to the wire type (bf16: IEEE round-to-nearest-even)

@@ -400,18 +400,15 @@ static __global__ void __launch_bounds__(PairShape<M, SMALL>::kMaxWarps * 32, 1)
         constexpr int N = decltype(count)::value;
         float f[8];
         widen<RT>(partner, f);
-        float2 neg[4];
-#pragma unroll
-        for (int x = 0; x < 4; ++x) neg[x] = make_float2(-f[2 * x], -f[2 * x + 1]);
         float s[N];
 #pragma unroll
         for (int u = 0; u < N; ++u) {
           float g[8];
-          widen<RT>(get(u), g);
+          minus8<RT>(get(u), f, g);
           float2 t = make_float2(0.0f, 0.0f);
 #pragma unroll
           for (int x = 0; x < 4; ++x) {
-            const float2 d = __fadd2_rn(make_float2(g[2 * x], g[2 * x + 1]), neg[x]);
+            const float2 d = make_float2(g[2 * x], g[2 * x + 1]);
             // (bf16: a square fits 24 bits in any case. fp32: rounded squares cancel some of the sums' error, a pair of copies
             // N(0, 3e-4) apart is 2e-10 off, fused ones 8e-10)
             if constexpr (RT::kVecs == 2) t = __fadd2_rn(t, __fmul2_rn(d, d));

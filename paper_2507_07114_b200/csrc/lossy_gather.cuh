@@ -80,7 +80,8 @@ __device__ __forceinline__ uint4 lds_here(uint32_t src) {
 
 // One lane's arithmetic at the end of a tile: estimate = sum / count (Algorithm 1 mode: the saved aggregate
 // on a drop), the optimizer in place in shared memory, the wire value written once into `wire_tile` and returned widened.
-template <class RT, int OPT>
+// (PAIRED: as in optimizer_n)
+template <class RT, int OPT, bool PAIRED>
 __device__ __forceinline__ void finish_tile_lane(const Params& P, float (&acc)[kEpl], uint32_t cnt, unsigned char* sb,
                                                  uint32_t off_th, uint32_t off_m, uint32_t off_v, unsigned char* wire_tile,
                                                  uint32_t idx, uint64_t e, float (&wire)[kEpl]) {
@@ -109,7 +110,7 @@ __device__ __forceinline__ void finish_tile_lane(const Params& P, float (&acc)[k
       lds_lane<F32>(sb + off_m, idx, m);
       lds_lane<F32>(sb + off_v, idx, v);
     }
-    optimizer_n<OPT, kEpl>(P, acc, th, m, v);
+    optimizer_n<OPT, kEpl, PAIRED>(P, acc, th, m, v);
     sts_lane_f32(sb + off_th, idx, th);
     if constexpr (OPT == 1) {
       sts_lane_f32(sb + off_m, idx, m);
@@ -142,6 +143,7 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
   constexpr int kSub = ANY ? kAnySub : kMaxSub;
   constexpr uint32_t kSubBits = (1u << kSub) - 1u;
   using Masks = TileMasks<kSub>;
+  constexpr bool kPairedOpt = ANY || RT::kVecs == 1;       // (fp32, packets that divide the tile: registers run out, W = 4, P = 512: 584 -> 605 us)
   constexpr bool kLaneWide = ANY && RT::kVecs == 2;        // stale rows: lane sums widened after each chunk
   constexpr bool kWarpDrift = DRIFTK && !RD;               // the compute warps read the stale copies
   constexpr int kTile = GatherShape<CW, RD>::kTile;
@@ -301,8 +303,7 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
           } else {                                          // bf16 replicas: two elements per word
 #pragma unroll
             for (int y = 0; y < 4; ++y) {
-              const float2 d = __fadd2_rn(make_float2(__uint_as_float(ow[y] << 16), __uint_as_float(ow[y] & 0xFFFF0000u)),
-                                          make_float2(-__uint_as_float(ww[y] << 16), -__uint_as_float(ww[y] & 0xFFFF0000u)));
+              const float2 d = pair_minus_bf16(ow[y], __uint_as_float(ww[y] << 16), __uint_as_float(ww[y] & 0xFFFF0000u));
               sq2 = __fadd2_rn(sq2, __fmul2_rn(d, d));
             }
           }
@@ -635,8 +636,7 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
             } else {                                        // bf16 replicas: two elements per word
 #pragma unroll
               for (int h = 0; h < 4; ++h) {
-                const float2 d = __fadd2_rn(make_float2(__uint_as_float(ow[h] << 16), __uint_as_float(ow[h] & 0xFFFF0000u)),
-                                            make_float2(-__uint_as_float(ww[h] << 16), -__uint_as_float(ww[h] & 0xFFFF0000u)));
+                const float2 d = pair_minus_bf16(ow[h], __uint_as_float(ww[h] << 16), __uint_as_float(ww[h] & 0xFFFF0000u));
                 sq2 = __fadd2_rn(sq2, __fmul2_rn(d, d));
               }
             }
@@ -763,12 +763,7 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
         const uint32_t bits = (uint32_t)(my_recv >> (g * kGroup)) & 0xFFu;
 #pragma unroll
         for (int u = 0; u < kGroup; ++u)
-          if ((bits >> u) & 1u) {
-            float f[kEpl];
-            lds_lane<GT>(st + (size_t)u * kRowG, idx, f);
-#pragma unroll
-            for (int x = 0; x < kEpl; ++x) acc[x] = __fadd_rn(acc[x], f[x]);
-          }
+          if ((bits >> u) & 1u) add_lane<GT>(st + (size_t)u * kRowG, idx, acc);
         if (g + 1 == G.groups) {
           // the wire tile goes into the ring the replica warps drain
           if (!mbar_wait(wempty_bar(wslot), wpar ^ 1u, abort_flag)) { ok = false; break; }
@@ -776,7 +771,7 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
 #pragma unroll
           for (int x = 0; x < kEpl; ++x) wire[x] = 0.0f;
           if (active)
-            finish_tile_lane<RT, OPT>(P, acc, (uint32_t)__popcll(my_recv), st, off_th, off_m, off_v,
+            finish_tile_lane<RT, OPT, kPairedOpt>(P, acc, (uint32_t)__popcll(my_recv), st, off_th, off_m, off_v,
                                       wring + (size_t)wslot * kRowR, idx, e0 + idx, wire);
           fence_proxy_async();          // make theta / m / v visible to the bulk stores
           __syncwarp();

@@ -255,12 +255,7 @@ __global__ void __launch_bounds__(TmaShape<CW>::kThreads, TmaShape<CW>::kCtasPer
           if (active) {
 #pragma unroll
             for (int u = 0; u < GS; ++u)
-              if ((bits >> u) & 1u) {
-                float f[kEpl];
-                lds_lane<T>(st + (size_t)u * kTile * kEB, idx, f);
-#pragma unroll
-                for (int x = 0; x < kEpl; ++x) acc[x] = __fadd_rn(acc[x], f[x]);
-              }
+              if ((bits >> u) & 1u) add_lane<T>(st + (size_t)u * kTile * kEB, idx, acc);
             if (g + 1 == G.groups) {
               divide_by_count<kEpl>(acc, h.cnt);
               if (P.ghat_prev) {

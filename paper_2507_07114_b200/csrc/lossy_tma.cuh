@@ -222,6 +222,41 @@ __device__ __forceinline__ void lds_lane(const unsigned char* base, uint32_t idx
   load_words<LaneWords<T>::value>(base + (size_t)idx * sizeof(typename T::raw), w);
   unpack_lane<T>(w, f);
 }
+// acc += kEpl elements in shared memory. bf16: one instruction per element, nothing is unpacked; fp32: one per two.
+template <class T>
+__device__ __forceinline__ void add_lane(const unsigned char* base, uint32_t idx, float (&acc)[kEpl]) {
+  uint32_t w[4];
+  load_words<LaneWords<T>::value>(base + (size_t)idx * sizeof(typename T::raw), w);
+#pragma unroll
+  for (int x = 0; x < kEpl; x += 2) {
+    if constexpr (T::kVecs == 2) {
+      const float2 s = __fadd2_rn(make_float2(acc[x], acc[x + 1]), make_float2(__uint_as_float(w[x]), __uint_as_float(w[x + 1])));
+      acc[x] = s.x;
+      acc[x + 1] = s.y;
+    } else {
+      add_pair_bf16(w[x / 2], acc[x], acc[x + 1]);
+    }
+  }
+}
+// the squares of kEpl elements minus x, summed one by one
+template <class T>
+__device__ __forceinline__ float squares_lane(const uint32_t (&w)[4], const float (&x)[kEpl]) {
+  float d[kEpl], sq = 0.0f;
+#pragma unroll
+  for (int y = 0; y < kEpl; y += 2) {
+    if constexpr (T::kVecs == 2) {
+      d[y] = __fsub_rn(__uint_as_float(w[y]), x[y]);
+      d[y + 1] = __fsub_rn(__uint_as_float(w[y + 1]), x[y + 1]);
+    } else {
+      const float2 s = pair_minus_bf16(w[y / 2], x[y], x[y + 1]);
+      d[y] = s.x;
+      d[y + 1] = s.y;
+    }
+  }
+#pragma unroll
+  for (int y = 0; y < kEpl; ++y) sq = __fadd_rn(sq, __fmul_rn(d[y], d[y]));
+  return sq;
+}
 __device__ __forceinline__ void sts_lane_f32(unsigned char* base, uint32_t idx, const float (&f)[kEpl]) {
   uint32_t w[4];
 #pragma unroll
@@ -678,12 +713,7 @@ __global__ void __launch_bounds__(TmaShape<CW>::kThreads, TmaShape<CW>::kCtasPer
         if (active) {
 #pragma unroll
           for (int u = 0; u < kGroup; ++u)
-            if ((bits >> u) & 1u) {
-              float f[kEpl];
-              lds_lane<GT>(st + (size_t)u * kTile * kGB, idx, f);
-#pragma unroll
-              for (int x = 0; x < kEpl; ++x) acc[x] = __fadd_rn(acc[x], f[x]);
-            }
+            if ((bits >> u) & 1u) add_lane<GT>(st + (size_t)u * kTile * kGB, idx, acc);
         }
         if (g + 1 < G.groups) {
           __syncwarp();
@@ -755,21 +785,7 @@ __global__ void __launch_bounds__(TmaShape<CW>::kThreads, TmaShape<CW>::kCtasPer
               lds_lane<F32>(sb + off_m, idx, m);
               lds_lane<F32>(sb + off_v, idx, v);
             }
-#pragma unroll
-            for (int x = 0; x < kEpl; ++x) {
-              if constexpr (OPT == 0) {
-                th[x] = __fsub_rn(th[x], __fmul_rn(P.lr, acc[x]));
-              } else {
-                const float mn = __fadd_rn(__fmul_rn(P.b1, m[x]), __fmul_rn(P.omb1, acc[x]));
-                const float vn = __fadd_rn(__fmul_rn(P.b2, v[x]), __fmul_rn(__fmul_rn(P.omb2, acc[x]), acc[x]));
-                const float mh = __fmul_rn(mn, P.ibc1);
-                const float vh = __fmul_rn(vn, P.ibc2);
-                const float den = __fadd_rn(__fsqrt_rn(vh), P.eps);
-                th[x] = __fsub_rn(th[x], __fdiv_rn(__fmul_rn(P.lr, mh), den));
-                m[x] = mn;
-                v[x] = vn;
-              }
-            }
+            optimizer_n<OPT, kEpl>(P, acc, th, m, v);
             sts_lane_f32(sb + off_th, idx, th);
             if constexpr (OPT == 1) {
               sts_lane_f32(sb + off_m, idx, m);
@@ -809,13 +825,9 @@ __global__ void __launch_bounds__(TmaShape<CW>::kThreads, TmaShape<CW>::kCtasPer
             for (int u = 0; u < kGroup; ++u) {
               sq[u] = 0.0f;
               if (active && (uint32_t)u < n_in) {
-                float old[kEpl];
-                lds_lane<RT>(sst + (size_t)u * kTile * kGB, idx, old);
-#pragma unroll
-                for (int x = 0; x < kEpl; ++x) {
-                  const float d = __fsub_rn(old[x], wire[x]);
-                  sq[u] = __fadd_rn(sq[u], __fmul_rn(d, d));
-                }
+                uint32_t ow[4];
+                load_words<LaneWords<RT>::value>(sst + (size_t)u * kTile * kGB + (size_t)idx * kRB, ow);
+                sq[u] = squares_lane<RT>(ow, wire);
               }
             }
             // all copies' warp totals at once; the first lane of segment u adds copy u's total to this warp's
@@ -836,20 +848,7 @@ __global__ void __launch_bounds__(TmaShape<CW>::kThreads, TmaShape<CW>::kCtasPer
 #pragma unroll
           for (int b = 0; b < kPre; ++b) {
             if (pre_id[b] >= 0) {
-              float old[kEpl];
-              if (active) {
-                unpack_lane<RT>(pre_raw[b], old);
-              } else {
-#pragma unroll
-                for (int x = 0; x < kEpl; ++x) old[x] = 0.0f;
-              }
-              float sq = 0.0f;
-#pragma unroll
-              for (int x = 0; x < kEpl; ++x) {
-                const float d = __fsub_rn(old[x], wire[x]);
-                sq = __fadd_rn(sq, __fmul_rn(d, d));
-              }
-              const float tot = warp_sum(sq);
+              const float tot = warp_sum(active ? squares_lane<RT>(pre_raw[b], wire) : 0.0f);
               if ((pre_id[b] & 31) == lane) {
                 if (pre_id[b] < 32) dacc0 += (double)tot; else dacc1 += (double)tot;
               }
@@ -859,7 +858,7 @@ __global__ void __launch_bounds__(TmaShape<CW>::kThreads, TmaShape<CW>::kCtasPer
           while (sm) {
             // up to kStaleBatch stale copies are fetched before the first is used
             int ids[kStaleBatch];
-            float old[kStaleBatch][kEpl];
+            uint32_t old[kStaleBatch][4];
             int nb = 0;
 #pragma unroll
             for (int b = 0; b < kStaleBatch; ++b) {
@@ -871,25 +870,14 @@ __global__ void __launch_bounds__(TmaShape<CW>::kThreads, TmaShape<CW>::kCtasPer
                 if (active) {
                   const typename RT::raw* rp =
                       reinterpret_cast<const typename RT::raw*>(P.replicas[ids[b]]) + rep_index(P, (uint32_t)ids[b], jj, e0 + idx);
-                  uint32_t ow[4];
-                  load_words_stream<LaneWords<RT>::value>(rp, ow);
-                  unpack_lane<RT>(ow, old[b]);
-                } else {
-#pragma unroll
-                  for (int x = 0; x < kEpl; ++x) old[b][x] = 0.0f;
+                  load_words_stream<LaneWords<RT>::value>(rp, old[b]);
                 }
               }
             }
 #pragma unroll
             for (int b = 0; b < kStaleBatch; ++b) {
               if (b < nb) {
-                float sq = 0.0f;
-#pragma unroll
-                for (int x = 0; x < kEpl; ++x) {
-                  const float d = __fsub_rn(old[b][x], wire[x]);
-                  sq = __fadd_rn(sq, __fmul_rn(d, d));
-                }
-                const float tot = warp_sum(sq);
+                const float tot = warp_sum(active ? squares_lane<RT>(old[b], wire) : 0.0f);
                 if ((ids[b] & 31) == lane) {
                   if (ids[b] < 32) dacc0 += (double)tot; else dacc1 += (double)tot;
                 }
