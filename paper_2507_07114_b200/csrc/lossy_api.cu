@@ -810,7 +810,7 @@ template <class RT, bool ELIDE, class M, bool SMALL>
 cudaError_t launch_pairwise(lossy_ctx* ctx, PairwiseArgs<ELIDE>& A, cudaStream_t s) {
   auto kern = drift_pairwise_kernel<RT, ELIDE, M, SMALL>;
   const uint32_t wb = pair_warp_bytes(A.W, sizeof(typename RT::raw));
-  const uint32_t room = (uint32_t)ctx->smem_optin;
+  const uint32_t room = (uint32_t)ctx->smem_optin - 128u;   // (less what is static)
   uint32_t warps = room / wb;
   if (warps > (uint32_t)PairShape<M, SMALL>::kMaxWarps) warps = PairShape<M, SMALL>::kMaxWarps;
   if (warps == 0) return cudaErrorInvalidConfiguration;

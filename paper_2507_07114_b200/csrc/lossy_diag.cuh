@@ -104,11 +104,13 @@ static __global__ void __launch_bounds__(256) packet_sqnorms_kernel(const __grid
 // warp's tree in fp32 as well a pair of bf16 copies that differ by N(0, 3e-4) came out 8.5e-9 low, as it is 3.4e-10;
 // differences from 1.2e18 on overflowed where they now do from 6.5e18 on.
 // Measured on B200, W = 16 bf16 replicas of 16 M elements (floor of one read: 79 us), by the share of packets a
-// replica missed: none 92 us, 5 % 115 us, 15 % 153 us, 35 % 261 us, all copies distinct 696 us; 4 x 4 blocks of replicas
+// replica missed: 5 % 97 us, 15 % 129 us, 35 % 197 us; 4 x 4 blocks of replicas
 // with every pair computed and fp64 sums per lane took 2512 us whatever the data. Bound by its issue slots and the latency
 // of the steps per differing piece, not by memory, once pieces differ.
-// Warps take chunks grid-stride: how many pieces differ is the same for a whole packet, so consecutive chunks per warp
-// left some warps with twice the work of others. Where there are fewer chunks than warps, 2^lgsplit warps share a chunk: each
+// How many pieces differ is the same for a whole packet and differs from packet to packet, and with it a chunk's work, so a
+// block's chunks are every gridDim.x-th one and its warps take them as they come free, by a counter in shared memory (dealt
+// out in advance, grid-stride, the three times above were 119, 161 and 263 us; W = 64, 4 M, 15 %: 242 and 469 us). Runs of four
+// chunks per turn, with the lanes' sums kept over a run, unbalance the warps again (216 us for 161). Where there are fewer chunks than warps, 2^lgsplit warps share a chunk: each
 // finds the differing pieces and computes every 2^lgsplit-th row of pairs (60 k elements, W = 64, fp32, all copies distinct: 246 ->
 // 126 us; W = 16, 35 % of the packets late: 27 -> 23 us).
 // (a kernel's arguments cost the host about 1 ns per byte: rep_skip only where it is read)
@@ -256,6 +258,7 @@ __host__ __device__ inline uint32_t pair_warp_bytes(uint32_t W, uint32_t elem_by
 template <class RT, bool ELIDE, class M, bool SMALL>
 static __global__ void __launch_bounds__(PairShape<M, SMALL>::kMaxWarps * 32, 1) drift_pairwise_kernel(const __grid_constant__ PairwiseArgs<ELIDE> A) {
   extern __shared__ __align__(16) unsigned char pair_smem[];
+  __shared__ uint32_t taken;                              // tasks of this block that its warps have taken
   constexpr unsigned kFull = 0xFFFFFFFFu;
   constexpr uint32_t kRB = sizeof(typename RT::raw);
   constexpr int kW = RT::kVecs * 4;                       // 32-bit words of a lane's 8 elements
@@ -267,8 +270,9 @@ static __global__ void __launch_bounds__(PairShape<M, SMALL>::kMaxWarps * 32, 1)
   unsigned char* slots = pair_smem + (size_t)warp * wb + (nt * 8u + 15u) / 16u * 16u;
   volatile uint32_t* slot_id = reinterpret_cast<volatile uint32_t*>(slots + kPairSlots * kChunk * kRB);
   for (uint32_t q = lane; q < nt; q += 32) tab[q] = 0.0;
+  if (threadIdx.x == 0) taken = 0;
   wait_for_previous();
-  __syncwarp();
+  __syncthreads();
   M bad_diag = 0;                                         // replicas seen to hold an infinity or NaN: x - x is NaN
   const M everyone = W == sizeof(M) * 8 ? ~(M)0 : ((M)1 << W) - 1;
   auto first_of = [](M x) { return (uint32_t)(sizeof(M) == 8 ? __ffsll((long long)x) : __ffs((int)x)) - 1u; };
@@ -299,7 +303,11 @@ static __global__ void __launch_bounds__(PairShape<M, SMALL>::kMaxWarps * 32, 1)
   const uint64_t total = ((uint64_t)A.segs * A.chunks_per_seg) << A.lgsplit;
   const uint32_t others = (1u << A.lgsplit) - 1u;         // warps a chunk is shared with
   uint32_t guess = 0;                                     // the reference of the chunk before
-  for (uint64_t task = (uint64_t)blockIdx.x * nwarps + warp; task < total; task += (uint64_t)gridDim.x * nwarps) {
+  for (;;) {
+    uint32_t next = 0;
+    if (lane == 0) next = atomicAdd(&taken, 1u);
+    const uint64_t task = (uint64_t)__shfl_sync(kFull, next, 0) * gridDim.x + blockIdx.x;
+    if (task >= total) break;
     const uint64_t q = task >> A.lgsplit;
     uint32_t turn = (uint32_t)task & others;              // rows of pairs are dealt out: this warp takes those met at turn 0
     auto mine = [&]() { const bool m = turn == 0u; turn = (turn - 1u) & others; return m; };
