@@ -140,10 +140,11 @@ template <class GT, class RT, int OPT, bool DRIFTK, int CW, bool RD, bool ANY>
 __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW, RD>::kCtasPerSm)
     lossy_fused_gather_kernel(const __grid_constant__ Params P, const __grid_constant__ TmaGeom G) {
   static_assert(!RD || DRIFTK, "RD is a way of computing the drift norms");
+  static_assert(GatherShape<CW, RD>::kTile * sizeof(typename RT::raw) / 512u % 4u == 0, "the replica warps read four chunks at a time");
   constexpr int kSub = ANY ? kAnySub : kMaxSub;
   constexpr uint32_t kSubBits = (1u << kSub) - 1u;
   using Masks = TileMasks<kSub>;
-  constexpr bool kPairedOpt = ANY || RT::kVecs == 1;       // (fp32, packets that divide the tile: registers run out, W = 4, P = 512: 584 -> 605 us)
+  constexpr bool kPairedOpt = RT::kVecs == 1 || (ANY && CW >= 16);   // (other fp32 builds: registers run out, W = 4, P = 512: 584 -> 605 us)
   constexpr bool kLaneWide = ANY && RT::kVecs == 2;        // stale rows: lane sums widened after each chunk
   constexpr bool kWarpDrift = DRIFTK && !RD;               // the compute warps read the stale copies
   constexpr int kTile = GatherShape<CW, RD>::kTile;
@@ -685,13 +686,19 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
         uint32_t behind;
         unsigned char* base = row_base(i, j_l, live_tile, e0, behind) + (uint32_t)lane * 16u;
         const uint64_t skip = behind ? P.rep_skip[i] * kRB : 0ull;
-        // One ballot and one base per row, and the wire tile read where it is stored, each read in front of its store: with four
-        // chunks of it held in registers every row was visited two to four times (W = 8, P = 736, p = 0.1, 135 M elements:
+        // One ballot and one base per row, and four chunks of the wire tile at a time read in front of their stores: held in
+        // registers for all replicas every row was visited two to four times (W = 8, P = 736, p = 0.1, 135 M elements:
         // 1245 us, this 1191; W = 4, P = 512, fp32, 67 M: 628 and 584), with eight there were no registers left (1280).
 #pragma unroll
-        for (int c = 0; c < kChunks; ++c)
-          if ((fresh >> sub_c[c]) & 1u)
-            __stcs(reinterpret_cast<uint4*>(base + c * 512 - ((behind >> sub_c[c]) & 1u ? skip : 0ull)), lds_here(from + c * 512u));
+        for (int c0 = 0; c0 < kChunks; c0 += 4) {
+          uint4 v[4];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) v[c] = lds_here(from + (c0 + c) * 512u);
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            if ((fresh >> sub_c[c0 + c]) & 1u)
+              __stcs(reinterpret_cast<uint4*>(base + (c0 + c) * 512 - ((behind >> sub_c[c0 + c]) & 1u ? skip : 0ull)), v[c]);
+        }
       }
       if constexpr (kReadsStale) {
         asm volatile("cp.async.wait_group 1;" ::: "memory");   // everything but the next tile's requests has landed
