@@ -21,6 +21,7 @@ struct GatherPolicy {
   bool use;
   bool wide;          // 2048-element tiles, one CTA per SM (else 1024, two)
   bool drift_warps;   // warps of their own read the stale copies
+  bool few_tiles;     // a small bucket of packets that divide the tile: the register kernel, not the packed build either
 };
 
 struct lossy_ctx {
@@ -476,8 +477,10 @@ int try_gather(lossy_ctx* ctx, const Params& P, bool drift, bool rd, cudaStream_
 // Where the gather pipeline is used, and which of its builds. Figures are times of the build it would replace over its own,
 // or (three digits) fractions of the copy rate; S = (W - 1) p_param = stale replicas per sub-packet. The lines were drawn
 // through 4700 random steps timed with every build in turn (2 to 64 workers, 50 thousand to 60 M elements, packets of 128
-// to 8960 elements, p = 0 to 0.3, both types, both optimizers, full and owner-elided replicas), so that none of the steps
-// taken is more than 2 % slower than on the build replaced; some that would be more than 5 % faster are left there.
+// to 8960 elements, p = 0 to 0.3, both types, both optimizers, full and owner-elided replicas), so that hardly any of the steps
+// taken is slower than on the build replaced; some that would be more than 5 % faster are left there. The lines for few tiles
+// per SM and packets under 1024 elements are from 3500 steps after kernels began behind the one ahead and the replica
+// warps' single visit of a row.
 GatherPolicy gather_policy(const lossy_ctx* ctx) {
   const lossy_config& c = ctx->cfg;
   const double pm = c.p_grad > c.p_param ? c.p_grad : c.p_param;
@@ -485,13 +488,14 @@ GatherPolicy gather_policy(const lossy_ctx* ctx) {
   const uint32_t P = c.packet_elems, kTwin = (uint32_t)TmaShape<8>::kTile, kWide = (uint32_t)GatherShape<16>::kTile;
   const bool bf16 = c.replica_dtype == LOSSY_BF16, sgd = c.optimizer == LOSSY_SGD;
   const bool forced = c.flags & LOSSY_GATHER_PATH;
-  GatherPolicy g = {false, false, false};
+  GatherPolicy g = {false, false, false, false};
   if (c.flags & LOSSY_PACKED_BULK || P < 128u) return g;
   TmaGeom G;
   // Tiles per SM. The pipeline fills and drains over several tiles, which a bucket of a few tiles per SM pays for: under
   // two the register kernel and the bulk-copy pipeline take 0.5-1.0 of its time (n = 0.9 M, W = 16, P = 336: 0.55). The
   // line lies higher with many workers (more groups per tile) and for SGD (less to move per tile).
-  const double per_sm = (double)c.n / ((double)kWide * ctx->num_sms) / ((c.W > 16u ? 1.5 : 1.0) * (sgd ? 1.25 : 1.0));
+  const double tiles = (double)c.n / ((double)kWide * ctx->num_sms);
+  const double per_sm = tiles / ((c.W > 16u ? 1.5 : 1.0) * (sgd ? 1.25 : 1.0));
   if (P < kTwin && kWide % P == 0) {
     // Packets of 128, 256 or 512 elements, which divide the tile:
     //  * the wide geometry with drift warps of its own from 4 workers, packets of 256 or 512 elements and bf16 replicas
@@ -514,11 +518,18 @@ GatherPolicy gather_policy(const lossy_ctx* ctx) {
     const bool beyond = many_lossy && c.W > 24u && pm < 0.225 && (forced || per_sm >= 32.0);
     g.wide = P >= 256u && c.W >= 4u;
     g.drift_warps = g.wide && (bf16 || forced) && (band || beyond) && gather_geometry<16, false>(ctx, true, G);
-    g.use = forced || g.drift_warps || !many_lossy || (!bf16 && P >= 256u && per_sm >= 7.0);
+    // Buckets of up to two tiles per SM with bf16 replicas, of up to one with fp32 ones (packets of 512 elements up to 8 workers
+    // only): the register kernel, one chunk or two per warp, is done before the pipeline has filled (1000 random steps,
+    // register kernel's time over the pipeline's: bf16 0.66-1.02, mean 0.85, P = 128 1.2 and more; fp32 0.8-1.04, but 512 with
+    // more workers up to 1.23). Under an eighth of a tile per SM either is a launch and little else, and it stays.
+    g.few_tiles = !forced && P >= 256u && tiles >= 0.125 && (bf16 ? tiles < 2.0 : tiles < 1.0 && (P == 256u || c.W <= 8u));
+    g.use = forced || (!g.few_tiles && (g.drift_warps || !many_lossy || (!bf16 && P >= 256u && per_sm >= 7.0)));
   } else if (P < kTwin) {
     // Other packets shorter than the twin tile. The alternative is the register kernel, whose chunks of 256 elements each
-    // packet ends with are filled to `fill`. From 5, 8, 12 or 16 tiles per SM with fill up to 0.6, 0.8, 0.9 or 1: 1.0-3.9
-    // (P = 736, W = 8, p = 0.1: 1.79; P = 200: 2.0; W = 64, P = 520: 1.1). Full chunks: not for SGD (W = 15, P = 768, p = 0: 0.91),
+    // packet ends with are filled to `fill`. From 3.5, 5, 6 or 8 tiles per SM with fill up to 0.6, 0.8, 0.9 or 1: 1.0-3.9
+    // (P = 736, W = 8, p = 0.1: 1.79; P = 200: 2.0; W = 64, P = 520: 1.1), 1.6 and 2.2 times as many from 17 workers and for SGD (of 1700
+    // steps, 110 lie between these lines and the ones before the replica warps' single visit, 5 to 16 tiles: mean 1.46, two
+    // of them under 0.9). Full chunks: not for SGD (W = 15, P = 768, p = 0: 0.91),
     // nearly full ones not with eight stale replicas (W = 41, P = 760, p = 0.3: 0.87); 12 of them only with the emptiest chunks.
     // Nor SGD at high loss with bf16 gradients and fp32 replicas that the drift warps cannot serve, up to a chunk (W = 9, P = 216,
     // p = 0.2: 0.87, P = 176: 0.83; P = 592 from 1.0).
@@ -526,12 +537,12 @@ GatherPolicy gather_policy(const lossy_ctx* ctx) {
     // 0.05: 0.68 against 0.59), wide ones from p = 0.15 (p = 0.3: 0.55 against 0.47); up to four workers twin below 256
     // (W = 4, P = 200: 0.75 against 0.63).
     const double fill = P / (256.0 * ((P + 255u) / 256u));
-    const double least = fill <= 0.6 ? 5.0 : fill <= 0.8 ? 8.0 : fill <= 0.9 ? 12.0 : 16.0;
+    const double least = (fill <= 0.6 ? 3.5 : fill <= 0.8 ? 5.0 : fill <= 0.9 ? 6.0 : 8.0) * (c.W > 16u ? 1.6 : 1.0) * (sgd ? 2.2 : 1.0);
     const bool full_lossy = (sgd && fill > 0.98) || (bf16 && ((fill > 0.9 && stale >= 8.0) || (fill > 0.6 && stale >= 12.0)));
     g.wide = c.W >= 5u ? P >= 176u || pm >= 0.15 : c.W == 4u && P >= 256u;
     g.drift_warps = g.wide && gather_geometry<16, true>(ctx, true, G);
     const bool sgd_lossy = sgd && pm >= 0.175 && !bf16 && c.grad_dtype == LOSSY_BF16 && P <= 256u && fill > 0.6 && g.wide && !g.drift_warps;
-    g.use = forced || (per_sm >= least && !full_lossy && !sgd_lossy);
+    g.use = forced || (tiles >= least && !full_lossy && !sgd_lossy);
   } else if (P % kTwin != 0 && P < (1u << 15)) {
     // Longer packets that are no multiple of the twin tile. The bulk-copy pipeline cuts each into tiles of its own, the
     // last of them part empty (`fill` of the tiles' elements are used); here the tiles run on across packets. From 6 tiles
@@ -553,11 +564,27 @@ GatherPolicy gather_policy(const lossy_ctx* ctx) {
   return g;
 }
 
+// A small bucket that ends in a short packet: packets from 1024 elements, all of it as one launch of the register kernel instead
+// of the bulk-copy pipeline's and one for the short packet, which ends some microseconds after it. In tiles (of 2048 elements)
+// per SM, register kernel's time over the other's in 700 random steps: bf16 replicas from one to 3.6 tiles (0.59-0.99, mean 0.79;
+// from there on 0.94-1.05; below one 0.64-0.99, mean 0.89, left as it was), up to two for packets that are no multiple of 1024
+// (0.62-1.0); fp32 replicas up to two tiles and 8 workers (0.63-1.02, mean 0.89; more workers 0.7-1.3). Not measured, so as before:
+// under an eighth of a tile per SM, no drift norms. LOSSY_PACKED_BULK asks for the bulk-copy pipeline all the same.
+bool one_launch(const lossy_ctx* ctx, bool drift) {
+  const lossy_config& c = ctx->cfg;
+  const uint32_t kTwin = (uint32_t)TmaShape<8>::kTile;
+  if (!drift || c.packet_elems < kTwin || c.n % c.packet_elems == 0) return false;
+  if (c.flags & (LOSSY_PACKED_BULK | LOSSY_GATHER_PATH)) return false;
+  const double tiles = (double)c.n / ((double)TmaShape<16>::kTile * ctx->num_sms);
+  if (c.replica_dtype != LOSSY_BF16) return tiles >= 0.125 && tiles < 2.0 && c.W <= 8u;
+  return tiles >= 1.0 && tiles < (c.packet_elems % kTwin == 0 ? 3.6 : 2.0);
+}
+
 // Run the build the policy picks; *used stays false when no bulk-copy launch fits (packets shorter
 // than a tile, or no complete packet): the register path then takes everything.
 int run_tma(lossy_ctx* ctx, const Params& P, bool drift, cudaStream_t s, uint32_t* blocks, bool* used) {
   *used = false;
-  if (ctx->cfg.flags & LOSSY_REGISTER_PATH) return LOSSY_OK;
+  if (ctx->cfg.flags & LOSSY_REGISTER_PATH || ctx->gather.few_tiles || one_launch(ctx, drift)) return LOSSY_OK;
   const TmaPolicy t = tma_policy(ctx->cfg);
   const GatherPolicy& gp = ctx->gather;
   if (gp.use) {
