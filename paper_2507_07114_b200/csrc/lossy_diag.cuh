@@ -273,6 +273,10 @@ static __global__ void __launch_bounds__(PairShape<M, SMALL>::kMaxWarps * 32, 1)
   if (threadIdx.x == 0) taken = 0;
   wait_for_previous();
   __syncthreads();
+  // (debug build: one warp of a block far ahead of the others, so that it takes more than one of the tasks they share)
+  if constexpr (kDevCheck) {
+    if (A.lgsplit && warp) __nanosleep(1000000u);
+  }
   M bad_diag = 0;                                         // replicas seen to hold an infinity or NaN: x - x is NaN
   const M everyone = W == sizeof(M) * 8 ? ~(M)0 : ((M)1 << W) - 1;
   auto first_of = [](M x) { return (uint32_t)(sizeof(M) == 8 ? __ffsll((long long)x) : __ffs((int)x)) - 1u; };
@@ -302,14 +306,17 @@ static __global__ void __launch_bounds__(PairShape<M, SMALL>::kMaxWarps * 32, 1)
 
   const uint64_t total = ((uint64_t)A.segs * A.chunks_per_seg) << A.lgsplit;
   const uint32_t others = (1u << A.lgsplit) - 1u;         // warps a chunk is shared with
-  uint32_t guess = 0;                                     // the reference of the chunk before
+  uint32_t guess = 0;                                     // the reference of the chunk before (a shared chunk: 0)
   for (;;) {
     uint32_t next = 0;
     if (lane == 0) next = atomicAdd(&taken, 1u);
     const uint64_t task = (uint64_t)__shfl_sync(kFull, next, 0) * gridDim.x + blockIdx.x;
     if (task >= total) break;
     const uint64_t q = task >> A.lgsplit;
-    uint32_t turn = (uint32_t)task & others;              // rows of pairs are dealt out: this warp takes those met at turn 0
+    // Rows of pairs are dealt out: this warp takes those met at turn 0. The warps that share a chunk meet the same rows only
+    // if they choose the same reference, so the search for it starts from replica 0 and not from the warp's last one: a
+    // warp may have taken a task before, of another chunk, and its siblings none.
+    uint32_t turn = (uint32_t)task & others;
     auto mine = [&]() { const bool m = turn == 0u; turn = (turn - 1u) & others; return m; };
     const uint32_t seg = ELIDE ? (uint32_t)q / A.chunks_per_seg : 0u, j = A.seg0 + seg;
     const uint64_t c = (uint32_t)q - seg * A.chunks_per_seg;
@@ -384,7 +391,7 @@ static __global__ void __launch_bounds__(PairShape<M, SMALL>::kMaxWarps * 32, 1)
       else if (r == best_r) break;
       else r = best_r;
     }
-    guess = r;
+    guess = A.lgsplit ? 0u : r;                            // (shared: see mine)
     if (!__all_sync(kFull, ref_finite)) bad_diag |= (M)1 << r;
     const M fresh = present & ~differ;              // pieces equal to the reference, itself among them
     // ---- the differing pieces, kPairSlots rows at a time, against everything behind them ----

@@ -26,6 +26,28 @@ CASES = [
 ]
 
 
+def shared_chunks(W, n, dtype):
+    """Pairwise drift of a small bucket: several warps share a chunk's pairs, and must choose the same reference. This build
+    lets one warp of a block run ahead, which takes several of the shared tasks then. In every second chunk (of 256) all
+    copies but replica 0 agree, in the others they are distinct: the best reference of the one is not the first choice in
+    the other. (bound: 10 * 2^-24, as in test_gpu_pairwise.py)"""
+    torch.manual_seed(W)
+    base = torch.randn(n, device="cuda") * 0.02
+    copies = [(base + 1e-3 * torch.randn(n, device="cuda")).to(dtype) for _ in range(W)]
+    for i in range(1, W):
+        for c in range(0, n, 512):
+            copies[i][c:c + 256] = copies[W - 1][c:c + 256]
+    ctx = L.lossy_init(W=W, n=n, packet_elems=256, p_grad=0.1, p_param=0.1, seed=1, grad_dtype=dtype, replica_dtype=dtype,
+                       optimizer="sgd", lr=0.1)
+    d2 = torch.zeros(W * W, dtype=torch.float64, device="cuda")
+    L.drift_pairwise(ctx, copies, d2)
+    R = torch.stack(copies).double()
+    want = ((R[:, None] - R[None]) ** 2).sum(2)
+    assert torch.all((d2.view(W, W) - want).abs() <= 6e-7 * want), (W, n, dtype)
+    L.lossy_destroy(ctx)
+    print("ok shared chunks", W, n, flush=True)
+
+
 def main():
     assert L.lossy_has_device_checks(), "the child process did not bind to the debug library"
     for name, W, n, P, p, opt, gd, rd, flags, fused, where in CASES:
@@ -49,6 +71,8 @@ def main():
         L.lossy_device_status(gpu.ctx)                          # clean again
         gpu.close()
         print("ok", name, flush=True)
+    for W, n, dtype in [(9, 30_000, torch.float32), (12, 20_000, torch.bfloat16), (40, 5000, torch.bfloat16), (64, 9001, torch.float32)]:
+        shared_chunks(W, n, dtype)
     print("DEVCHECK-WORKER-PASSED")
 
 
