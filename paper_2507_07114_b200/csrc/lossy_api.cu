@@ -39,6 +39,8 @@ struct lossy_ctx {
   uint32_t* status;      // device status words: [0] 0 = fine, 1 = a bounded wait in a kernel gave up; [1..4] debug build: a failed index check
   uint64_t check_shrink; // debug build self-test: the index checks hold ranges against n - check_shrink
   uint32_t* ticket;      // device counter of finished blocks (last-block drift finalisation), zero between calls
+  uint32_t* gate;        // device word by which a call's two launches tell that the kernels ahead of them are done, zero between calls
+  uint32_t calls;        // number of the last call that may have two launches
   bool plan_only;        // launch helpers only report their grid size
   const uint64_t* reliable;  // caller-owned device array [2][K] of reliable-link bits, or NULL
   uint64_t* burst_state; // bursty loss: caller-owned device array [2 buffers][2 rows][K], or NULL
@@ -118,7 +120,7 @@ cudaError_t launch_after(bool early, void (*kern)(Formal...), dim3 grid, uint32_
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-void fill_common(const lossy_ctx* ctx, uint64_t step, Params& P) {
+void fill_common(lossy_ctx* ctx, uint64_t step, Params& P) {
   memset(&P, 0, sizeof P);
   const lossy_config& c = ctx->cfg;
   P.n = c.n;
@@ -147,6 +149,11 @@ void fill_common(const lossy_ctx* ctx, uint64_t step, Params& P) {
   P.reliable = ctx->reliable;
   P.check = ctx->status + 1;
   P.check_n = c.n - (ctx->check_shrink < c.n ? ctx->check_shrink : c.n);
+  if (c.n % c.packet_elems != 0) {   // the short last packet may have a launch of its own
+    if (++ctx->calls == 0u) ctx->calls = 1u;
+    P.gate = ctx->gate;
+    P.gate_id = ctx->calls;
+  }
   fill_rep_skip(P, (c.flags & LOSSY_REPLICA_SKIP_OWNER) != 0);
   if (ctx->burst_state) {
     // the states after step t-1 live in buffer (t-1)&1, those after step t go to buffer t&1
@@ -909,6 +916,7 @@ int lossy_init(const lossy_config* cfg, lossy_ctx** out) {
   if (e != cudaSuccess) { delete ctx; return e == cudaErrorMemoryAllocation ? LOSSY_ENOMEM : LOSSY_ECUDA; }
   ctx->status = reinterpret_cast<uint32_t*>(reinterpret_cast<unsigned char*>(ctx->partials) + pbytes);
   ctx->ticket = ctx->status + 16;
+  ctx->gate = ctx->status + 32;
   e = cudaMemset(ctx->status, 0, 256);
   if (e != cudaSuccess) { cudaFree(ctx->partials); delete ctx; return LOSSY_ECUDA; }
   *out = ctx;

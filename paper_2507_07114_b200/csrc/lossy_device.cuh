@@ -76,6 +76,10 @@ struct Params {
   // the self-test shrinks it). Unused otherwise.
   uint32_t* check;
   uint64_t check_n;
+  // A call whose short last packet has a launch of its own beside the launch of the complete ones (open_gate): the context's
+  // gate word, and this call's number. Else NULL.
+  uint32_t* gate;
+  uint32_t gate_id;
 };
 
 // Programmatic dependent launch: most kernels are launched with leave to begin before the kernel ahead of them in the stream
@@ -85,6 +89,27 @@ struct Params {
 __device__ __forceinline__ void wait_for_previous() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+// The launch of a short last packet (lossy_kernel, TAIL) runs beside the launch of the complete packets, on what the kernels
+// ahead of both have written. Those writes are visible to a grid that has waited, and that is the complete packets' one: it
+// says so in a word of the context, with a release, and the short packet's threads read the word with an acquire before
+// anything else. That it may begin at all says nothing about memory. A thread that does not find this call's number there
+// waits like any other kernel (for the complete packets' launch to end), so nothing spins and no launch depends on another one
+// running. The word is cleared by the short packet's launch, for a graph replays a call's number.
+__device__ __forceinline__ void wait_for_previous(const Params& P) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (P.gate && blockIdx.x == 0 && threadIdx.x == 0) asm volatile("st.release.gpu.u32 [%0], %1;" ::"l"(P.gate), "r"(P.gate_id) : "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void begin_beside_previous(const Params& P) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  uint32_t open;
+  asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(open) : "l"(P.gate) : "memory");
+  if (open != P.gate_id) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void end_after_previous(const Params& P) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (blockIdx.x == 0 && threadIdx.x == 0) *P.gate = 0u;   // (a block that has not looked yet will wait)
 }
 
 // Owner-elided replicas: rep_skip[i] = elements of worker i's shard inside the context's packet range

@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_proxy_async();
   }
-  wait_for_previous();
+  wait_for_previous(P);
   __syncthreads();
 
   constexpr int kChunks = kRowR / 512u;                     // a replica's row of a tile in 512-byte chunks

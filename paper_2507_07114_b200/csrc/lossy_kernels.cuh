@@ -257,17 +257,17 @@ __device__ __forceinline__ void batch_masks(const Params& P, const BatchDraws& d
 // ELIDE = owner-elided replicas: a build of its own, so that the index arithmetic of that layout costs the
 // default layout nothing (this kernel is bound by its issue slots, not by memory).
 // TAIL = the launch of a call's short last packet, behind the launch that has the complete ones. It shares nothing but the
-// ticket counter with that launch, whose blocks let it begin once they have passed their own wait: everything before that
-// launch is complete then. So it need not wait to begin, only to end (what follows waits for this launch alone). A build of
-// its own: with the wait behind the loop of every build the single phases ran 5-28 % slower where packets leave lanes idle
-// (W = 3, P = 128, n = 65 M, step: 518 -> 661 us).
+// ticket counter with that launch, whose blocks let it begin once they have passed their own wait. So it need not wait
+// for that launch to begin (how it knows that the kernels ahead of both are done: wait_for_previous in lossy_device.cuh), only to
+// end (what follows waits for this launch alone). A build of its own: with the wait behind the loop of every build the single phases
+// ran 5-28 % slower where packets leave lanes idle (W = 3, P = 128, n = 65 M, step: 518 -> 661 us).
 template <int PH, class GT, class RT, int OPT, bool ELIDE = false, bool TAIL = false>
 __global__ void __launch_bounds__(kThreads, LOSSY_MIN_BLOCKS) lossy_kernel(const __grid_constant__ Params P) {
   auto rep_at = [&](uint32_t i, uint32_t j, uint64_t e) { return ELIDE ? rep_index(P, i, j, e) : e; };
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   const uint32_t W = P.W;
-  if constexpr (TAIL) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if constexpr (TAIL) begin_beside_previous(P);
   else wait_for_previous();
 
   // per-lane drift accumulators: lane l holds replicas l and l + 32
@@ -471,7 +471,7 @@ __global__ void __launch_bounds__(kThreads, LOSSY_MIN_BLOCKS) lossy_kernel(const
     sh[warp * kMaxW + lane + 32] = dacc1;
     drift_finish(P, sh, kWarps, P.partials_row0 + blockIdx.x, warp, kWarps, lane);
   }
-  if constexpr (TAIL) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if constexpr (TAIL) end_after_previous(P);
 }
 
 // Sum the per-block partials of replica blockIdx.x in a fixed order (lane l takes rows l, l+32, ...,

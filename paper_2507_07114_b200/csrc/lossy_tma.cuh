@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(TmaShape<CW>::kThreads, TmaShape<CW>::kCtasPer
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_proxy_async();
   }
-  wait_for_previous();
+  wait_for_previous(P);
   __syncthreads();
 
   double dacc0 = 0.0, dacc1 = 0.0;   // compute warps: lane l holds replicas l and l + 32
