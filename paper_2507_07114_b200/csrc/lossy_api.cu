@@ -60,7 +60,10 @@ int fail(lossy_ctx* ctx, int code, const char* msg) {
   if (ctx) snprintf(ctx->err, sizeof ctx->err, "%s", msg);
   return code;
 }
+// The caller gets the error from here; in the runtime it is cleared, or the next look at the last error, behind a launch that
+// went well, would find it there.
 int fail_cuda(lossy_ctx* ctx, const char* what, cudaError_t e) {
+  cudaGetLastError();
   if (ctx) snprintf(ctx->err, sizeof ctx->err, "%s: %s", what, cudaGetErrorString(e));
   return LOSSY_ECUDA;
 }
@@ -118,6 +121,11 @@ cudaError_t launch_after(bool early, void (*kern)(Formal...), dim3 grid, uint32_
   cfg.attrs = at;
   cfg.numAttrs = early ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+// behind a call that failed: a ticketed launch may already be queued, and the counter must be zero again before the next call
+void reset_ticket(lossy_ctx* ctx, cudaStream_t s) {
+  if (cudaMemsetAsync(ctx->ticket, 0, sizeof(uint32_t), s) != cudaSuccess) cudaGetLastError();
 }
 
 void fill_common(lossy_ctx* ctx, uint64_t step, Params& P) {
@@ -827,8 +835,7 @@ int run_phase(lossy_ctx* ctx, const Params& P, float* norms, double* sumsq, cuda
     }
     ctx->plan_only = false;
     if (rc) {
-      // a ticketed launch may already be queued: the counter must be zero again before the next call
-      if (Q.ticket) cudaMemsetAsync(ctx->ticket, 0, sizeof(uint32_t), s);
+      if (Q.ticket) reset_ticket(ctx, s);
       return rc;
     }
   }
@@ -1143,8 +1150,7 @@ static int fused_impl(lossy_ctx* ctx, uint64_t step, const void* const* grads, f
     }
     ctx->plan_only = false;
     if (rc) {
-      // a ticketed launch may already be queued: the counter must be zero again before the next call
-      if (Q.ticket) cudaMemsetAsync(ctx->ticket, 0, sizeof(uint32_t), s);
+      if (Q.ticket) reset_ticket(ctx, s);
       return rc;
     }
   }

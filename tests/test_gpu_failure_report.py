@@ -1,11 +1,13 @@
 """The library's failure report, exercised without a failure: a bounded wait that runs out sets the context's
 status word; nothing faults, traps or hangs, and the context works again after a reset."""
+import ctypes
+
 import pytest
 import torch
 
 import paper_2507_07114_b200 as L
 import workload
-from parity_util import run_parity
+from parity_util import GpuRun, run_parity
 
 pytestmark = pytest.mark.gpu
 
@@ -33,6 +35,37 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_recovers():
         ref = orc.step(t, [to_np(g) for g in gs])
         compare_outputs(gpu.outputs(), ref, f"after reset, step {t}")
         compare_state(gpu, orc, f"after reset, step {t}")
+    L.lossy_device_status(gpu.ctx)
+
+
+@pytest.mark.parametrize("W,n,P", [(4, 1024 * 40 + 8, 1024), (4, 64 * 10, 64)])        # bulk-copy pipeline, register kernel
+def test_a_failed_launch_is_reported_once(W, n, P):
+    """The runtime refuses a launch into a capture that has been invalidated (here by a synchronisation). The call says so,
+    and a launch behind it that goes well is not reported as failed."""
+    w = workload.Workload("refused", W, n, P, 0.1, "sgd", 1e-2, "f32", "f32", 2, seed=5)
+    gpu, want = GpuRun(w), GpuRun(w)
+    grads = [workload.grad_slab(w, 1, i, 0, n, "cuda") for i in range(W)]
+    ids = torch.arange(256, device="cuda", dtype=torch.int32)
+    packet, out = torch.arange(256, device="cuda", dtype=torch.int64), torch.zeros(256, dtype=torch.uint8, device="cuda")
+    stream, rt = torch.cuda.Stream(), ctypes.CDLL("libcudart.so.12")
+    handle, graph = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p()
+    step = L.lossy_fused_step_prepared(gpu.ctx, grads, gpu.master, None, None, gpu.replicas, norms=gpu.norms, stream=stream)
+    step(1)                                                 # (what a kernel's first launch sets up is not captured)
+    want.step_fused(1, grads, outputs=False)
+    torch.cuda.synchronize()
+    launches = L.lossy_kernel_launches(gpu.ctx)
+    assert rt.cudaStreamBeginCapture(handle, 1) == 0
+    assert rt.cudaStreamSynchronize(handle) != 0
+    with pytest.raises(L.LossyError) as ei:
+        step(2)
+    rt.cudaStreamEndCapture(handle, ctypes.byref(graph))
+    rt.cudaGetLastError()                                   # (torch's runtime: this test's own two errors)
+    assert ei.value.code == L.LOSSY_ECUDA and L.lossy_kernel_launches(gpu.ctx) == launches
+    L.lossy_mask_grid(gpu.ctx, 1, ids, ids, packet, out)
+    step(2)
+    want.step_fused(2, grads, outputs=False)
+    torch.cuda.synchronize()
+    assert torch.equal(gpu.master, want.master) and torch.equal(gpu.norms, want.norms)
     L.lossy_device_status(gpu.ctx)
 
 
