@@ -21,7 +21,7 @@ struct GatherPolicy {
   bool use;
   bool wide;          // 2048-element tiles, one CTA per SM (else 1024, two)
   bool drift_warps;   // warps of their own read the stale copies
-  bool few_tiles;     // a small bucket of packets that divide the tile: the register kernel, not the packed build either
+  bool few_tiles[2];  // (with drift norms: [1]) a small bucket of packets that divide the tile: the register kernel, not the packed build either
 };
 
 struct lossy_ctx {
@@ -503,7 +503,7 @@ GatherPolicy gather_policy(const lossy_ctx* ctx) {
   const uint32_t P = c.packet_elems, kTwin = (uint32_t)TmaShape<8>::kTile, kWide = (uint32_t)GatherShape<16>::kTile;
   const bool bf16 = c.replica_dtype == LOSSY_BF16, sgd = c.optimizer == LOSSY_SGD;
   const bool forced = c.flags & LOSSY_GATHER_PATH;
-  GatherPolicy g = {false, false, false, false};
+  GatherPolicy g = {};
   if (c.flags & LOSSY_PACKED_BULK || P < 128u) return g;
   TmaGeom G;
   // Tiles per SM. The pipeline fills and drains over several tiles, which a bucket of a few tiles per SM pays for: under
@@ -536,9 +536,13 @@ GatherPolicy gather_policy(const lossy_ctx* ctx) {
     // Buckets of up to two tiles per SM with bf16 replicas, of up to one with fp32 ones (packets of 512 elements up to 8 workers
     // only): the register kernel, one chunk or two per warp, is done before the pipeline has filled (1000 random steps,
     // register kernel's time over the pipeline's: bf16 0.66-1.02, mean 0.85, P = 128 1.2 and more; fp32 0.8-1.04, but 512 with
-    // more workers up to 1.23). Under an eighth of a tile per SM either is a launch and little else, and it stays.
-    g.few_tiles = !forced && P >= 256u && tiles >= 0.125 && (bf16 ? tiles < 2.0 : tiles < 1.0 && (P == 256u || c.W <= 8u));
-    g.use = forced || (!g.few_tiles && (g.drift_warps || !many_lossy || (!bf16 && P >= 256u && per_sm >= 7.0)));
+    // more workers up to 1.23). Steps without drift norms, 2200 random ones: bf16 0.45-1.04, mean 0.78; fp32 up to 24 workers
+    // 0.59-1.23, mean 0.81; with more workers 0.73-1.27, mean 0.95, and they stay with the pipeline. Under an eighth of a tile per
+    // SM either is a launch and little else, and it stays.
+    const bool few = !forced && P >= 256u && tiles >= 0.125 && (bf16 ? tiles < 2.0 : tiles < 1.0 && (P == 256u || c.W <= 8u));
+    g.few_tiles[0] = few && (bf16 || c.W <= 24u);
+    g.few_tiles[1] = few;
+    g.use = forced || g.drift_warps || !many_lossy || (!bf16 && P >= 256u && per_sm >= 7.0);
   } else if (P < kTwin) {
     // Other packets shorter than the twin tile. The alternative is the register kernel, whose chunks of 256 elements each
     // packet ends with are filled to `fill`. From 3.5, 5, 6 or 8 tiles per SM with fill up to 0.6, 0.8, 0.9 or 1: 1.0-3.9
@@ -599,7 +603,7 @@ bool one_launch(const lossy_ctx* ctx, bool drift) {
 // than a tile, or no complete packet): the register path then takes everything.
 int run_tma(lossy_ctx* ctx, const Params& P, bool drift, cudaStream_t s, uint32_t* blocks, bool* used) {
   *used = false;
-  if (ctx->cfg.flags & LOSSY_REGISTER_PATH || ctx->gather.few_tiles || one_launch(ctx, drift)) return LOSSY_OK;
+  if (ctx->cfg.flags & LOSSY_REGISTER_PATH || ctx->gather.few_tiles[drift] || one_launch(ctx, drift)) return LOSSY_OK;
   const TmaPolicy t = tma_policy(ctx->cfg);
   const GatherPolicy& gp = ctx->gather;
   if (gp.use) {

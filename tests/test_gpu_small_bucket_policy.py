@@ -67,3 +67,32 @@ def test_small_buckets(case):
         assert torch.equal(a.replicas[i], b.replicas[i]), f"replica {i}"
     L.lossy_device_status(a.ctx)
     L.lossy_device_status(b.ctx)
+
+
+# W, n, P, gradients, replicas, start of the build's name without drift norms, and with
+NO_NORMS = [(32, SM_TILE // 2, 256, "f32", "f32", "gather wide", "register"),
+            (24, SM_TILE // 2, 256, "f32", "f32", "register", "register"),
+            (32, SM_TILE // 2, 256, "bf16", "bf16", "register", "register"),
+            (25, SM_TILE - 256 + 40, 256, "bf16", "f32", "gather wide", "register"),      # a short last packet
+            (8, SM_TILE, 2048, "bf16", "bf16", "bulk-copy wide", "bulk-copy wide"),
+            (8, SM_TILE + 5, 2048, "bf16", "bf16", "bulk-copy wide", "register")]
+
+
+@pytest.mark.parametrize("W,n,P,g,r,without,with_norms", NO_NORMS)
+def test_small_buckets_without_drift_norms(W, n, P, g, r, without, with_norms):
+    w = workload.Workload("no_norms", W, n, P, 0.1, "adam", 3e-4, g, r, 2, seed=n % 97)
+    a, b = GpuRun(w), GpuRun(w)
+    assert L.lossy_describe_plan(a.ctx, with_drift=False).startswith(without)
+    assert L.lossy_describe_plan(b.ctx).startswith(with_norms)
+    grads = [workload.grad_slab(w, 1, i, 0, n, "cuda") for i in range(W)]
+    for t in (1, 2):
+        L.lossy_fused_step(a.ctx, t, grads, a.master, a.m, a.v, a.replicas, a.ghat, a.count, a.recv, a.stale)
+        b.step_fused(t, grads)
+    oa, ob = a.outputs(), b.outputs()
+    for k in ("ghat", "count", "recv_bits", "stale_bits"):
+        assert_same(oa[k], ob[k], k)
+    for name in ("master", "m", "v"):
+        assert_same(to_np(getattr(a, name)), to_np(getattr(b, name)), name)
+    for i in range(W):
+        assert torch.equal(a.replicas[i], b.replicas[i]), f"replica {i}"
+    L.lossy_device_status(a.ctx)
