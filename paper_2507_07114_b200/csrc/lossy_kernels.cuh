@@ -443,21 +443,43 @@ __global__ void __launch_bounds__(kThreads, LOSSY_MIN_BLOCKS) lossy_kernel(const
               old[b] = load8_any<RT>(P.replicas[ids[b]], rep_at((uint32_t)ids[b], j, e), nvalid);
             }
           }
+          // A lane's eight squares are added in fp32, everything else in fp64, as the pairwise drift's are: bf16 copies N(0, 3e-4)
+          // apart come out 3e-10 low, with a tree of 256 squares in fp32 8.8e-9, and the pipelines' 128 squares, whose small
+          // buckets this kernel takes, 6.0e-9. One reduction of several copies makes up for the wider exchange: W = 64, P = 256,
+          // 16 M, p = 0.3: 788 -> 778 us; W = 16, P = 512, 0.6 M, p = 0.3: 16.35 -> 16.09; W = 8, P = 304, 1 M, p = 0.1: 20.7 -> 20.9.
+          float sq[4];
 #pragma unroll
           for (int b = 0; b < 4; ++b) {
+            sq[b] = 0.0f;
             if (b < nb) {
-              float diff[8], s = 0.0f;
+              float diff[8];
               minus8<RT>(old[b], xw, diff);
 #pragma unroll
               for (int x = 0; x < 8; ++x) {
                 const float d = x < nvalid ? diff[x] : 0.0f;
-                s = __fadd_rn(s, __fmul_rn(d, d));
-              }
-              const float tot = warp_sum(s);
-              if ((ids[b] & 31) == lane) {
-                if (ids[b] < 32) dacc0 += (double)tot; else dacc1 += (double)tot;
+                sq[b] = __fadd_rn(sq[b], __fmul_rn(d, d));
               }
             }
+          }
+          auto credit = [&](int id, double tot) {
+            if ((id & 31) == lane) {
+              if (id < 32) dacc0 += tot; else dacc1 += tot;
+            }
+          };
+          if (nb > 2) {
+            const double t = warp_sum_multi64<4>(sq, lane);
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+              const double x = __shfl_sync(0xFFFFFFFFu, t, b * 8);
+              if (b < nb) credit(ids[b], x);
+            }
+          } else if (nb == 2) {
+            const float two[2] = {sq[0], sq[1]};
+            const double t = warp_sum_multi64<2>(two, lane);
+#pragma unroll
+            for (int b = 0; b < 2; ++b) credit(ids[b], __shfl_sync(0xFFFFFFFFu, t, b * 16));
+          } else {
+            credit(ids[0], warp_sum64((double)sq[0]));
           }
         }
       }
