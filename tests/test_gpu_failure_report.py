@@ -38,12 +38,13 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_recovers():
     L.lossy_device_status(gpu.ctx)
 
 
-@pytest.mark.parametrize("W,n,P", [(4, 1024 * 40 + 8, 1024), (4, 64 * 10, 64)])        # bulk-copy pipeline, register kernel
-def test_a_failed_launch_is_reported_once(W, n, P):
+@pytest.mark.parametrize("W,n,P,plan", [(4, 1024 * 40, 1024, "bulk-copy"), (4, 64 * 10, 64, "register")])
+def test_a_failed_launch_is_reported_once(W, n, P, plan):
     """The runtime refuses a launch into a capture that has been invalidated (here by a synchronisation). The call says so,
     and a launch behind it that goes well is not reported as failed."""
     w = workload.Workload("refused", W, n, P, 0.1, "sgd", 1e-2, "f32", "f32", 2, seed=5)
     gpu, want = GpuRun(w), GpuRun(w)
+    assert L.lossy_describe_plan(gpu.ctx).startswith(plan)
     grads = [workload.grad_slab(w, 1, i, 0, n, "cuda") for i in range(W)]
     ids = torch.arange(256, device="cuda", dtype=torch.int32)
     packet, out = torch.arange(256, device="cuda", dtype=torch.int64), torch.zeros(256, dtype=torch.uint8, device="cuda")

@@ -31,15 +31,18 @@ def test_config2_shape_scaled_ragged(mode):
 @PATHS
 @pytest.mark.parametrize("name", ["cfg3_w64_layer_p01", "cfg3_w64_layer_p10"])
 def test_config3_shape_scaled(name, path_flag):
-    w = workload.scaled(CFG[name], 4096 * 130 + 40)
-    run_parity(w, 6, flags=path_flag)
+    w = workload.scaled(CFG[name], 4096 * 72 + 40)           # (a short last packet: under one tile of 2048 elements per SM)
+    gpu, _ = run_parity(w, 6, flags=path_flag)
+    assert L.lossy_describe_plan(gpu.ctx).startswith("register" if path_flag else "bulk-copy")
 
 
 @pytest.mark.parametrize("P", [256, 1024, 2048, 4096])
 @pytest.mark.parametrize("p", [0.0, 0.01, 0.05, 0.1, 0.3])
 def test_config5_sweep_scaled(P, p):
-    w = workload.scaled(CFG["cfg5_w16_layer_sweep"], 4096 * 40 + 256 * 3, packet_elems=P, p=p)
+    # packets of 256 elements: on the gather pipeline from two tiles of 2048 elements per SM
+    w = workload.scaled(CFG["cfg5_w16_layer_sweep"], 4096 * (150 if P == 256 else 40) + 256 * 3, packet_elems=P, p=p)
     gpu, orc = run_parity(w, 4)
+    assert L.lossy_describe_plan(gpu.ctx).startswith("gather" if P == 256 else "bulk-copy")
     if p == 0.0:
         assert float(gpu.norms.abs().max()) == 0.0
         assert int(gpu.count.min()) == 16

@@ -73,8 +73,9 @@ def test_elided_replicas_match_the_oracle(case, fused):
 def test_elided_equals_the_full_layout_on_everything_a_worker_does_not_own():
     """Same run with and without the flag: identical masks, parameters and norms; each elided replica is the full
     one with the owner's range cut out."""
-    w = workload.scaled(workload.baseline_workloads()["cfg2_w8_layer_adam"], 2048 * 300 + 24)
+    w = workload.scaled(workload.baseline_workloads()["cfg2_w8_layer_adam"], 2048 * 600 + 24)
     a, b = GpuRun(w), GpuRun(w, flags=ELIDE)
+    assert all(L.lossy_describe_plan(x.ctx).startswith("bulk-copy") for x in (a, b))
     K, W, P = w.K, w.W, w.packet_elems
     pps = (K + W - 1) // W
     for t in range(1, 5):
