@@ -99,10 +99,10 @@ static __global__ void __launch_bounds__(256) packet_sqnorms_kernel(const __grid
 // Differing pieces are kept in shared memory, kPairSlots at a time (fetching them again cost an L2 round trip per row
 // of pairs). The pieces behind the slots meet all slots at once, so one fetch serves kPairSlots pairs, whose totals
 // come from one multi-value reduction.
-// Sums: fp32 over a lane's eight elements, fp64 from there on: over the warp, in a table of pairs per warp in shared
-// memory, and with fp64 atomics into d2 at the end (their order is not fixed: results agree to ~1e-15 relative). With the
-// warp's tree in fp32 as well a pair of bf16 copies that differ by N(0, 3e-4) came out 8.5e-9 low, as it is 3.4e-10;
-// differences from 1.2e18 on overflowed where they now do from 6.5e18 on.
+// Sums: fp32 over a lane's eight elements, two multiply-add chains of four, fp64 from there on: over the warp, in a table of
+// pairs per warp in shared memory, and with fp64 atomics into d2 at the end (their order is not fixed: results agree to ~1e-15
+// relative). With the warp's tree in fp32 as well a pair of bf16 copies that differ by N(0, 3e-4) came out 8.5e-9 low, as it
+// is 4e-10 (fp32 copies: 6e-10 high); differences from 1.2e18 on overflowed where they now do from 6.5e18 on.
 // Measured on B200, W = 16 bf16 replicas of 16 M elements (floor of one read: 79 us), by the share of packets a
 // replica missed: 5 % 97 us, 15 % 129 us, 35 % 197 us; 4 x 4 blocks of replicas
 // with every pair computed and fp64 sums per lane took 2512 us whatever the data. Bound by its issue slots and the latency
@@ -215,7 +215,7 @@ static __global__ void __launch_bounds__(128) drift_pairwise_few_kernel(const __
 #pragma unroll
           for (int x = 0; x < 4; ++x) {
             const float2 d = __fadd2_rn(f[i][x], make_float2(-f[k][x].x, -f[k][x].y));
-            t = __fadd2_rn(t, __fmul2_rn(d, d));
+            t = __ffma2_rn(d, d, t);
           }
           acc[at] += (double)__fadd_rn(t.x, t.y);
         }
@@ -424,10 +424,7 @@ static __global__ void __launch_bounds__(PairShape<M, SMALL>::kMaxWarps * 32, 1)
 #pragma unroll
           for (int x = 0; x < 4; ++x) {
             const float2 d = make_float2(g[2 * x], g[2 * x + 1]);
-            // (bf16: a square fits 24 bits in any case. fp32: rounded squares cancel some of the sums' error, a pair of copies
-            // N(0, 3e-4) apart is 2e-10 off, fused ones 8e-10)
-            if constexpr (RT::kVecs == 2) t = __fadd2_rn(t, __fmul2_rn(d, d));
-            else t = __ffma2_rn(d, d, t);
+            t = __ffma2_rn(d, d, t);
           }
           s[u] = live ? __fadd_rn(t.x, t.y) : 0.0f;
         }

@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
             for (int y = 0; y < 4; y += 2) {
               const float2 d = __fadd2_rn(make_float2(__uint_as_float(ow[y]), __uint_as_float(ow[y + 1])),
                                           make_float2(-__uint_as_float(ww[y]), -__uint_as_float(ww[y + 1])));
-              sq2 = __fadd2_rn(sq2, __fmul2_rn(d, d));
+              sq2 = __ffma2_rn(d, d, sq2);
             }
             if constexpr (kLaneWide) {
               wide += (double)__fadd_rn(sq2.x, sq2.y);
@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
 #pragma unroll
             for (int y = 0; y < 4; ++y) {
               const float2 d = pair_minus_bf16(ow[y], __uint_as_float(ww[y] << 16), __uint_as_float(ww[y] & 0xFFFF0000u));
-              sq2 = __fadd2_rn(sq2, __fmul2_rn(d, d));
+              sq2 = __ffma2_rn(d, d, sq2);
             }
           }
         }
@@ -628,7 +628,7 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
               for (int h = 0; h < 4; h += 2) {
                 const float2 d = __fadd2_rn(make_float2(__uint_as_float(ow[h]), __uint_as_float(ow[h + 1])),
                                             make_float2(-__uint_as_float(ww[h]), -__uint_as_float(ww[h + 1])));
-                sq2 = __fadd2_rn(sq2, __fmul2_rn(d, d));
+                sq2 = __ffma2_rn(d, d, sq2);
               }
               if constexpr (kLaneWide) {
                 wide += (double)__fadd_rn(sq2.x, sq2.y);
@@ -638,7 +638,7 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
 #pragma unroll
               for (int h = 0; h < 4; ++h) {
                 const float2 d = pair_minus_bf16(ow[h], __uint_as_float(ww[h] << 16), __uint_as_float(ww[h] & 0xFFFF0000u));
-                sq2 = __fadd2_rn(sq2, __fmul2_rn(d, d));
+                sq2 = __ffma2_rn(d, d, sq2);
               }
             }
           }
