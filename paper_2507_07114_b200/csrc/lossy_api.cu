@@ -232,10 +232,12 @@ uint32_t tma_smem_budget(const lossy_ctx* ctx) {
 
 // Dynamic shared memory a launch asks for. Blocks that may begin while the kernel ahead still runs go to the SMs that are
 // free first, as many as fit: a kernel of one block per SM that needs less than half an SM's memory was then laid out two by
-// two (the four single-phase calls on the MLP bucket: 1885 -> 2005 us). So each block asks for enough that no more than
-// `per_sm` of them fit, and only one where there are no more blocks than SMs.
-uint32_t spread_smem(const lossy_ctx* ctx, uint32_t smem, uint32_t per_sm, uint32_t blocks) {
-  if (blocks <= (uint32_t)ctx->num_sms) per_sm = 1;
+// two (the four single-phase calls, W = 8: 135 M elements 1830 -> 2031 us, 1 M 28.2 -> 30.5). So each block asks for enough
+// that no more than `per_sm` of them fit. What it asks for, kernels of other streams cannot have: four streams of single-phase calls
+// on 1 M elements each take 25.2 us a call sequence, without this 20.6 (two streams 25.0 and 22.7, one 31.7 and 34.6). One block per SM
+// also for grids of two per SM that are smaller than the chip gained nothing on one stream and cost four of them
+// (W = 4, P = 1024, 131 k elements, fused: 2.3 -> 4.0 us a step).
+uint32_t spread_smem(const lossy_ctx* ctx, uint32_t smem, uint32_t per_sm) {
   const uint32_t least = 228u * 1024u / (per_sm + 1u), most = (uint32_t)ctx->smem_optin - 1024u;
   return smem >= least ? smem : least < most ? least : most;
 }
@@ -305,7 +307,7 @@ int launch_tma(lossy_ctx* ctx, const Params& P, const TmaGeom& G, cudaStream_t s
       if (ctx->device < kMaxDevices) opted_in[ctx->device] = true;
     }
   }
-  e = launch_after(true, kern, blocks, kThreadsTma, spread_smem(ctx, smem, TmaShape<CW>::kCtasPerSm, blocks), s, P, G);
+  e = launch_after(true, kern, blocks, kThreadsTma, spread_smem(ctx, smem, TmaShape<CW>::kCtasPerSm), s, P, G);
   if (e != cudaSuccess) return fail_cuda(ctx, "bulk-copy kernel launch", e);
   ctx->launches++;
   return LOSSY_OK;
@@ -455,7 +457,7 @@ int launch_gather(lossy_ctx* ctx, const Params& P, const TmaGeom& G, cudaStream_
       if (ctx->device < kMaxDevices) opted_in[ctx->device] = true;
     }
   }
-  e = launch_after(true, kern, blocks, GatherShape<CW, RD>::kThreads, spread_smem(ctx, smem, GatherShape<CW>::kCtasPerSm, blocks), s, P, G);
+  e = launch_after(true, kern, blocks, GatherShape<CW, RD>::kThreads, spread_smem(ctx, smem, GatherShape<CW>::kCtasPerSm), s, P, G);
   if (e != cudaSuccess) return fail_cuda(ctx, "gather kernel launch", e);
   ctx->launches++;
   return LOSSY_OK;
@@ -778,7 +780,7 @@ int launch_phase_tma(lossy_ctx* ctx, const Params& P, const TmaGeom& G, cudaStre
       if (ctx->device < kMaxDevices) opted_in[ctx->device] = true;
     }
   }
-  e = launch_after(true, kern, blocks, TmaShape<CW>::kThreads, spread_smem(ctx, smem, TmaShape<CW>::kCtasPerSm, blocks), s, P, G);
+  e = launch_after(true, kern, blocks, TmaShape<CW>::kThreads, spread_smem(ctx, smem, TmaShape<CW>::kCtasPerSm), s, P, G);
   if (e != cudaSuccess) return fail_cuda(ctx, "bulk-copy kernel launch", e);
   ctx->launches++;
   return LOSSY_OK;
