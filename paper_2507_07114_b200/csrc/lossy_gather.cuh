@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_proxy_async();
   }
-  wait_for_previous(P);
+  wait_for_previous();
   __syncthreads();
 
   constexpr int kChunks = kRowR / 512u;                     // a replica's row of a tile in 512-byte chunks
@@ -521,6 +521,7 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
     if (!ok || *abort_flag) asm volatile("cp.async.wait_all;" ::: "memory");
   } else if (warp == CW + kNP + 1) {
     // ================================ store warp =================================
+    open_gate(P, lane);
     uint32_t s = 0, par = 0;
     bool ok = true;
     const bool sh_hint = G.hints & 2u;
@@ -688,7 +689,8 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
         const uint64_t skip = behind ? P.rep_skip[i] * kRB : 0ull;
         // One ballot and one base per row, and four chunks of the wire tile at a time read in front of their stores: held in
         // registers for all replicas every row was visited two to four times (W = 8, P = 736, p = 0.1, 135 M elements:
-        // 1245 us, this 1191; W = 4, P = 512, fp32, 67 M: 628 and 584), with eight there were no registers left (1280).
+        // 1239 us, this 1205; W = 5, P = 512, owner-elided, 20 M: 164.5 and 159.9). One read in front of each store is as fast
+        // under the power limit (1211) and 2.5 % slower below it.
 #pragma unroll
         for (int c0 = 0; c0 < kChunks; c0 += 4) {
           uint4 v[4];

@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(TmaShape<CW>::kThreads, TmaShape<CW>::kCtasPer
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_proxy_async();
   }
-  wait_for_previous(P);
+  wait_for_previous();
   __syncthreads();
 
   double dacc0 = 0.0, dacc1 = 0.0;   // compute warps: lane l holds replicas l and l + 32
@@ -535,6 +535,7 @@ __global__ void __launch_bounds__(TmaShape<CW>::kThreads, TmaShape<CW>::kCtasPer
     }
   } else if (warp == kConsumerWarps + 1) {
     // ================================ store warp =================================
+    open_gate(P, lane);
     uint32_t s = 0, par = 0, sq = 0;
     bool ok = true;
     const bool sh_hint = G.hints & 2u;
