@@ -56,7 +56,8 @@ __device__ __forceinline__ void divide_by_count(float (&a)[N], uint32_t cnt) {
 // power, and the large steps run at the power limit (W = 8, P = 736, 135 M elements: 1245 -> 1191 us).
 // The assembler joins a packed product and the packed addition behind it into one multiply-add, whatever rounding either
 // asks for (-fmad=false holds for scalars). A product that is added to something is therefore a multiply-add already, with
-// P.neg_zero: x + (-0) is x for every x, and the assembler cannot know that the parameter is -0.
+// P.neg_zero: x + (-0) is x for every x, and the assembler cannot know that the parameter is -0. (The packed sums of squares of the
+// pairwise drift and of the gather pipeline's drift norms are multiply-adds.)
 template <int OPT, int N, bool PAIRED = true>
 __device__ __forceinline__ void optimizer_n(const Params& P, const float (&g)[N], float (&th)[N], float (&m)[N],
                                             float (&v)[N]) {
@@ -258,7 +259,7 @@ __device__ __forceinline__ void batch_masks(const Params& P, const BatchDraws& d
 // default layout nothing (this kernel is bound by its issue slots, not by memory).
 // TAIL = the launch of a call's short last packet, behind the launch that has the complete ones. It shares nothing but the
 // ticket counter with that launch, whose blocks let it begin once they have passed their own wait. So it need not wait
-// for that launch to begin (how it knows that the kernels ahead of both are done: wait_for_previous in lossy_device.cuh), only to
+// for that launch to begin (how it knows that the kernels ahead of both are done: open_gate), only to
 // end (what follows waits for this launch alone). A build of its own: with the wait behind the loop of every build the single phases
 // ran 5-28 % slower where packets leave lanes idle (W = 3, P = 128, n = 65 M, step: 518 -> 661 us).
 template <int PH, class GT, class RT, int OPT, bool ELIDE = false, bool TAIL = false>
@@ -270,8 +271,14 @@ __global__ void __launch_bounds__(kThreads, LOSSY_MIN_BLOCKS) lossy_kernel(const
   if constexpr (TAIL) begin_beside_previous(P);
   else wait_for_previous();
 
-  // per-lane drift accumulators: lane l holds replicas l and l + 32
+  // drift sums per warp and replica; a warp writes its own row alone (standalone: kept in registers, lane l holds l and l + 32)
+  __shared__ double dsum[PH & DRIFT ? kWarps * kMaxW : 1];
   double dacc0 = 0.0, dacc1 = 0.0;
+  if constexpr ((PH & DRIFT) && (PH & BCAST)) {
+    dsum[warp * kMaxW + lane] = 0.0;
+    dsum[warp * kMaxW + lane + 32] = 0.0;
+    __syncwarp();
+  }
 
   const uint32_t warps_in_grid = gridDim.x * kWarps;
   for (uint32_t q = P.chunk_begin + blockIdx.x * kWarps + warp; q < P.num_chunks; q += warps_in_grid) {
@@ -443,43 +450,51 @@ __global__ void __launch_bounds__(kThreads, LOSSY_MIN_BLOCKS) lossy_kernel(const
               old[b] = load8_any<RT>(P.replicas[ids[b]], rep_at((uint32_t)ids[b], j, e), nvalid);
             }
           }
-          // A lane's eight squares are added in fp32, everything else in fp64, as the pairwise drift's are: bf16 copies N(0, 3e-4)
-          // apart come out 3e-10 low, with a tree of 256 squares in fp32 8.8e-9, and the pipelines' 128 squares, whose small
-          // buckets this kernel takes, 6.0e-9. One reduction of several copies makes up for the wider exchange: W = 64, P = 256,
-          // 16 M, p = 0.3: 788 -> 778 us; W = 16, P = 512, 0.6 M, p = 0.3: 16.35 -> 16.09; W = 8, P = 304, 1 M, p = 0.1: 20.7 -> 20.9.
-          float sq[4];
+          // Fused: a lane's eight squares are added in fp32, everything else in fp64, as the pairwise drift's are: bf16 copies
+          // N(0, 3e-4) apart come out 3e-10 low, with a tree of 256 squares in fp32 8.8e-9, and the pipelines' 128 squares, whose
+          // small buckets this kernel takes, 6.0e-9. One reduction of several copies, and sums in shared memory that the lanes add to
+          // which hold a total, make up for the wider exchange: W = 64, P = 256, 16 M, p = 0.3: 792 -> 773 us; W = 16, P = 512, 0.6 M, p =
+          // 0.3: 16.3 -> 15.9; W = 20, P = 336, 0.2 M: 17.7 both; W = 44, P = 352, 1.6 M, fp32: 170.9 -> 174.5. The drift norms alone
+          // read all copies of every chunk and keep the fp32 tree (W = 24, P = 704, 2 M, the four phases: 101 us, with fp64 108).
+          auto squares = [&](int b) {      // of copy b's differences, this lane's eight elements
+            float diff[8], s = 0.0f;
+            minus8<RT>(old[b], xw, diff);
 #pragma unroll
-          for (int b = 0; b < 4; ++b) {
-            sq[b] = 0.0f;
-            if (b < nb) {
-              float diff[8];
-              minus8<RT>(old[b], xw, diff);
-#pragma unroll
-              for (int x = 0; x < 8; ++x) {
-                const float d = x < nvalid ? diff[x] : 0.0f;
-                sq[b] = __fadd_rn(sq[b], __fmul_rn(d, d));
-              }
+            for (int x = 0; x < 8; ++x) {
+              const float d = x < nvalid ? diff[x] : 0.0f;
+              s = __fadd_rn(s, __fmul_rn(d, d));
             }
-          }
-          auto credit = [&](int id, double tot) {
-            if ((id & 31) == lane) {
-              if (id < 32) dacc0 += tot; else dacc1 += tot;
-            }
+            return s;
           };
-          if (nb > 2) {
-            const double t = warp_sum_multi64<4>(sq, lane);
+          if constexpr (PH & BCAST) {
+            float sq[4];
+#pragma unroll
+            for (int b = 0; b < 4; ++b) sq[b] = b < nb ? squares(b) : 0.0f;
+            double tot;
+            int to = 0;                    // the copy whose total this lane adds: the first lane of each segment does
+            if (nb > 2) {
+              tot = warp_sum_multi64<4>(sq, lane);
+              to = lane >> 3;
+            } else if (nb == 2) {
+              const float two[2] = {sq[0], sq[1]};
+              tot = warp_sum_multi64<2>(two, lane);
+              to = lane >> 4;
+            } else {
+              tot = warp_sum64((double)sq[0]);
+            }
+            const int id = to < 2 ? (to ? ids[1] : ids[0]) : (to == 2 ? ids[2] : ids[3]);
+            if ((lane & (nb > 2 ? 7 : nb == 2 ? 15 : 31)) == 0 && to < nb) dsum[warp * kMaxW + id] += tot;
+            __syncwarp();                  // (another lane may add to this copy's sum next time)
+          } else {
 #pragma unroll
             for (int b = 0; b < 4; ++b) {
-              const double x = __shfl_sync(0xFFFFFFFFu, t, b * 8);
-              if (b < nb) credit(ids[b], x);
+              if (b < nb) {
+                const float tot = warp_sum(squares(b));
+                if ((ids[b] & 31) == lane) {
+                  if (ids[b] < 32) dacc0 += (double)tot; else dacc1 += (double)tot;
+                }
+              }
             }
-          } else if (nb == 2) {
-            const float two[2] = {sq[0], sq[1]};
-            const double t = warp_sum_multi64<2>(two, lane);
-#pragma unroll
-            for (int b = 0; b < 2; ++b) credit(ids[b], __shfl_sync(0xFFFFFFFFu, t, b * 16));
-          } else {
-            credit(ids[0], warp_sum64((double)sq[0]));
           }
         }
       }
@@ -488,10 +503,11 @@ __global__ void __launch_bounds__(kThreads, LOSSY_MIN_BLOCKS) lossy_kernel(const
 
   // ---- per-block drift partials, fixed order ------------------------------------
   if constexpr (PH & DRIFT) {
-    __shared__ double sh[kWarps * kMaxW];
-    sh[warp * kMaxW + lane] = dacc0;
-    sh[warp * kMaxW + lane + 32] = dacc1;
-    drift_finish(P, sh, kWarps, P.partials_row0 + blockIdx.x, warp, kWarps, lane);
+    if constexpr (!(PH & BCAST)) {
+      dsum[warp * kMaxW + lane] = dacc0;
+      dsum[warp * kMaxW + lane + 32] = dacc1;
+    }
+    drift_finish(P, dsum, kWarps, P.partials_row0 + blockIdx.x, warp, kWarps, lane);
   }
   if constexpr (TAIL) end_after_previous(P);
 }

@@ -16,24 +16,18 @@ CASES = [(8, 2 * SM_TILE - 512, 512, 0.2, "bf16", 0), (4, 2 * SM_TILE - 256 + 40
 
 
 @pytest.mark.parametrize("W,n,P,p,r,flags", CASES)
-@pytest.mark.parametrize("fused", [True, False])
-def test_drift_sums_are_fp64_from_the_lane_on(W, n, P, p, r, flags, fused):
+def test_drift_sums_are_fp64_from_the_lane_on(W, n, P, p, r, flags):
     """Copies N(0, 3e-4) apart, as a training run has them. Eight bf16 squares added in fp32 and everything else in fp64 come out
     3.4e-10 low (the same order in NumPy; eight fp32 ones 3e-10 at this size), a warp's tree of 256 squares in fp32 8.8e-9,
     of 128 squares 6.0e-9."""
     w = workload.Workload("precision", W, n, P, p, "sgd", 0.0, "bf16", r, 1, seed=n % 89)
-    if not fused:
-        flags |= L.LOSSY_REGISTER_PATH                     # drift_norms as a call of its own
     gpu = GpuRun(w, flags=flags)
     assert L.lossy_describe_plan(gpu.ctx).startswith("register")
     torch.manual_seed(W)
     for rep in gpu.replicas:
         rep.copy_(gpu.master + 3e-4 * torch.randn(n, device="cuda"))
     grads = [torch.zeros(n, device="cuda", dtype=torch.bfloat16) for _ in range(W)]
-    if fused:
-        gpu.step_fused(1, grads)
-    else:
-        L.drift_norms(gpu.ctx, gpu.master, gpu.replicas, gpu.norms, gpu.sumsq)
+    gpu.step_fused(1, grads)
     wire = gpu.master.to(gpu.replicas[0].dtype).double()
     want = torch.stack([((rep.double() - wire) ** 2).sum() for rep in gpu.replicas])
     assert abs(float(gpu.sumsq.sum() / want.sum()) - 1) <= 1.5e-9
