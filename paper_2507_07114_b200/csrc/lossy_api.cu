@@ -103,8 +103,8 @@ int check_replicas(lossy_ctx* ctx, const void* const* tab) {
 
 // A launch with programmatic stream serialisation: the kernel may be set up while the kernel ahead of it in the stream still
 // runs, and waits for that one's end itself (wait_for_previous). Behind anything but a kernel, or behind one that does not
-// give leave, it is an ordinary launch. Host time of a launch: 1.8 us instead of 2.4; W = 8, P = 2048, n = 300 k: 22.4 -> 18.5 us
-// a step; with a short last packet, which takes a second launch: W = 4, n = 100 k, on the device 12.1 -> 7.4 us.
+// give leave, it is an ordinary launch. Host time of a launch: 1.8 us instead of 2.4; W = 8, P = 2048, n = 262 k, in a graph: 10.6 ->
+// 9.4 us a step; with a short last packet on a launch of its own (n = 262 184): 20.0 -> 11.4.
 // early = false, an ordinary launch: for kernels that load through L1 and run long. A block that begins early gets what
 // shared memory the kernel ahead has left its SM, after a gather pipeline 28 KB of L1 (closed-loop gradients of 58 M elements
 // behind it: 690 -> 755 us for the pair; packet norms behind the pairwise drift, W = 9, n = 4.6 M: 92 -> 97 us).
@@ -235,7 +235,7 @@ uint32_t tma_smem_budget(const lossy_ctx* ctx) {
 // two (the four single-phase calls, W = 8: 135 M elements 1830 -> 2031 us, 1 M 28.2 -> 30.5). So each block asks for enough
 // that no more than `per_sm` of them fit. What it asks for, kernels of other streams cannot have: four streams of single-phase calls
 // on 1 M elements each take 25.2 us a call sequence, without this 20.6 (two streams 25.0 and 22.7, one 31.7 and 34.6). One block per SM
-// also for grids of two per SM that are smaller than the chip gained nothing on one stream and cost four of them
+// also for grids of two per SM that are smaller than the chip gained 0 to 3 % on one stream and cost four of them
 // (W = 4, P = 1024, 131 k elements, fused: 2.3 -> 4.0 us a step).
 uint32_t spread_smem(const lossy_ctx* ctx, uint32_t smem, uint32_t per_sm) {
   const uint32_t least = 228u * 1024u / (per_sm + 1u), most = (uint32_t)ctx->smem_optin - 1024u;
@@ -494,10 +494,14 @@ int try_gather(lossy_ctx* ctx, const Params& P, bool drift, bool rd, cudaStream_
 // Where the gather pipeline is used, and which of its builds. Figures are times of the build it would replace over its own,
 // or (three digits) fractions of the copy rate; S = (W - 1) p_param = stale replicas per sub-packet. The lines were drawn
 // through 4700 random steps timed with every build in turn (2 to 64 workers, 50 thousand to 60 M elements, packets of 128
-// to 8960 elements, p = 0 to 0.3, both types, both optimizers, full and owner-elided replicas), so that hardly any of the steps
-// taken is slower than on the build replaced; some that would be more than 5 % faster are left there. The lines for few tiles
-// per SM and packets under 1024 elements are from 3500 steps after kernels began behind the one ahead and the replica
-// warps' single visit of a row.
+// to 8960 elements, p = 0 to 0.3, both types, both optimizers, full and owner-elided replicas), so that none of the steps
+// taken was more than 2 % slower than on the build replaced. The lines for few tiles per SM and packets under 1024 elements are
+// from 3500 steps after kernels began behind the one ahead and the replica warps' single visit of a row, by which the other
+// builds gained more than this one: of 7500 random steps up to 12 M elements since, the build chosen here and in run_tma is
+// behind the best one by 9 % in the mean for packets of 128 to 512 that divide the tile (128 elements: the PACKED build, 1.05-1.3,
+// below half a tile per SM up to 1.9; 256 and 512, bf16, two to eight tiles per SM: the register kernel, 1.05-1.2),
+// by 6 % for other packets under 1024 (on the register kernel from two tiles per SM, 1.2, up to 2.2), by 3-5 % for longer
+// ones (under one tile per SM with a short last packet, 1.1-1.2, up to 1.8; multiples of 1024, whole, from two tiles on: none).
 GatherPolicy gather_policy(const lossy_ctx* ctx) {
   const lossy_config& c = ctx->cfg;
   const double pm = c.p_grad > c.p_param ? c.p_grad : c.p_param;
@@ -549,8 +553,9 @@ GatherPolicy gather_policy(const lossy_ctx* ctx) {
     // Other packets shorter than the twin tile. The alternative is the register kernel, whose chunks of 256 elements each
     // packet ends with are filled to `fill`. From 3.5, 5, 6 or 8 tiles per SM with fill up to 0.6, 0.8, 0.9 or 1: 1.0-3.9
     // (P = 736, W = 8, p = 0.1: 1.79; P = 200: 2.0; W = 64, P = 520: 1.1), 1.6 and 2.2 times as many from 17 workers and for SGD (of 1700
-    // steps, 110 lie between these lines and the ones before the replica warps' single visit, 5 to 16 tiles: mean 1.46, two
-    // of them under 0.9). Full chunks: not for SGD (W = 15, P = 768, p = 0: 0.91),
+    // steps, 110 lie between these lines and the ones before the replica warps' single visit, 5 to 16 tiles: mean 1.46; slower
+    // there: SGD at W = 14, P = 240, p = 0.3: 0.83, W = 6: 0.92, W = 5, P = 224, p = 0.05, fp32 replicas: 0.89, and W = 27, P = 712,
+    // p = 0.3: 0.91. Without drift norms 775 more: mean 1.50, one under 0.98). Full chunks: not for SGD (W = 15, P = 768, p = 0: 0.91),
     // nearly full ones not with eight stale replicas (W = 41, P = 760, p = 0.3: 0.87); 12 of them only with the emptiest chunks.
     // Nor SGD at high loss with bf16 gradients and fp32 replicas that the drift warps cannot serve, up to a chunk (W = 9, P = 216,
     // p = 0.2: 0.87, P = 176: 0.83; P = 592 from 1.0).
