@@ -13,6 +13,7 @@
 #include "lossy_diag.cuh"
 #include "lossy_gather.cuh"
 #include "lossy_phase_tma.cuh"
+#include "lossy_register.cuh"
 
 using namespace lossy;
 
@@ -21,7 +22,7 @@ struct GatherPolicy {
   bool use;
   bool wide;          // 2048-element tiles, one CTA per SM (else 1024, two)
   bool drift_warps;   // warps of their own read the stale copies
-  bool few_tiles[2];  // (with drift norms: [1]) a small bucket of packets that divide the tile: the register kernel, not the packed build either
+  bool small[2];      // (with drift norms: [1]) a small bucket: the step kernel, none of the pipelines
 };
 
 struct lossy_ctx {
@@ -108,6 +109,9 @@ int check_replicas(lossy_ctx* ctx, const void* const* tab) {
 // early = false, an ordinary launch: for kernels that load through L1 and run long. A block that begins early gets what
 // shared memory the kernel ahead has left its SM, after a gather pipeline 28 KB of L1 (closed-loop gradients of 58 M elements
 // behind it: 690 -> 755 us for the pair; packet norms behind the pairwise drift, W = 9, n = 4.6 M: 92 -> 97 us).
+// a call's one launch: its blocks' rows are all (two launches: the caller has counted them ahead)
+void rows_of_call(Params& P, uint32_t blocks) { if (P.total_rows == 0u) P.total_rows = blocks; }
+
 template <class... Formal, class... Actual>
 cudaError_t launch_after(bool early, void (*kern)(Formal...), dim3 grid, uint32_t threads, size_t smem, cudaStream_t s, const Actual&... args) {
   cudaLaunchAttribute at[1] = {};
@@ -120,7 +124,10 @@ cudaError_t launch_after(bool early, void (*kern)(Formal...), dim3 grid, uint32_
   cfg.stream = s;
   cfg.attrs = at;
   cfg.numAttrs = early ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kern, args...);
+  // (the arguments where they lie: cudaLaunchKernelEx copies them, 2 KB, once more)
+  static_assert((std::is_same<Formal, Actual>::value && ...), "a kernel's arguments as it declares them");
+  void* argv[] = {const_cast<void*>(static_cast<const void*>(&args))...};
+  return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(kern), argv);
 }
 
 // behind a call that failed: a ticketed launch may already be queued, and the counter must be zero again before the next call
@@ -155,8 +162,10 @@ void fill_common(lossy_ctx* ctx, uint64_t step, Params& P) {
   P.partials = ctx->partials;
   P.K = (uint32_t)ctx->K;
   P.reliable = ctx->reliable;
+#ifdef LOSSY_DEVCHECK
   P.check = ctx->status + 1;
   P.check_n = c.n - (ctx->check_shrink < c.n ? ctx->check_shrink : c.n);
+#endif
   if (c.n % c.packet_elems != 0) {   // the short last packet may have a launch of its own
     if (++ctx->calls == 0u) ctx->calls = 1u;
     P.gate = ctx->gate;
@@ -288,7 +297,7 @@ bool tma_geometry(const lossy_ctx* ctx, TmaGeom& G) {
 }
 
 template <class GT, class RT, int OPT, bool DRIFTK, int CW, int GS, int PRE, bool PACKED, bool SPLIT>
-int launch_tma(lossy_ctx* ctx, const Params& P, const TmaGeom& G, cudaStream_t s, uint32_t* blocks_out) {
+int launch_tma(lossy_ctx* ctx, Params& P, const TmaGeom& G, cudaStream_t s, uint32_t* blocks_out) {
   auto kern = lossy_fused_tma_kernel<GT, RT, OPT, DRIFTK, CW, GS, PRE, PACKED, SPLIT>;
   constexpr int kThreadsTma = TmaShape<CW>::kThreads;
   const uint32_t smem = kTmaSmemFixed + G.stages * G.stage_bytes + 2u * G.state_bytes + CW * kMaxW * (uint32_t)sizeof(double);
@@ -297,6 +306,7 @@ int launch_tma(lossy_ctx* ctx, const Params& P, const TmaGeom& G, cudaStream_t s
   if (blocks > G.num_tiles) blocks = G.num_tiles;
   *blocks_out = blocks;
   if (ctx->plan_only) return LOSSY_OK;
+  rows_of_call(P, blocks);
   static bool opted_in[kMaxDevices];   // per kernel instantiation and device: raise the dynamic shared memory limit once
   cudaError_t e;
   {
@@ -314,7 +324,7 @@ int launch_tma(lossy_ctx* ctx, const Params& P, const TmaGeom& G, cudaStream_t s
 }
 
 template <bool DRIFTK, int CW, int GS, int PRE, bool PACKED, bool SPLIT>
-int dispatch_tma(lossy_ctx* ctx, const Params& P, const TmaGeom& G, cudaStream_t s, uint32_t* blocks) {
+int dispatch_tma(lossy_ctx* ctx, Params& P, const TmaGeom& G, cudaStream_t s, uint32_t* blocks) {
   const bool gb = ctx->cfg.grad_dtype == LOSSY_BF16;
   const bool rb = ctx->cfg.replica_dtype == LOSSY_BF16;
   const bool adam = ctx->cfg.optimizer == LOSSY_ADAM;
@@ -327,7 +337,7 @@ int dispatch_tma(lossy_ctx* ctx, const Params& P, const TmaGeom& G, cudaStream_t
 }
 
 template <int CW, int GS, int PRE = 0, bool PACKED = false, bool SPLIT = false>
-int try_tma(lossy_ctx* ctx, const Params& P, bool drift, cudaStream_t s, uint32_t* blocks, bool* used) {
+int try_tma(lossy_ctx* ctx, Params& P, bool drift, cudaStream_t s, uint32_t* blocks, bool* used) {
   TmaGeom G = {};
   if (!tma_geometry<CW, GS, PACKED, SPLIT>(ctx, G)) return LOSSY_OK;
   *used = true;
@@ -440,13 +450,14 @@ bool gather_geometry(const lossy_ctx* ctx, bool rd, TmaGeom& G) {
 }
 
 template <class GT, class RT, int OPT, bool DRIFTK, int CW, bool RD, bool ANY>
-int launch_gather(lossy_ctx* ctx, const Params& P, const TmaGeom& G, cudaStream_t s, uint32_t* blocks_out) {
+int launch_gather(lossy_ctx* ctx, Params& P, const TmaGeom& G, cudaStream_t s, uint32_t* blocks_out) {
   auto kern = lossy_fused_gather_kernel<GT, RT, OPT, DRIFTK, CW, RD, ANY>;
   const uint32_t smem = kGatherSmemFixed<ANY> + G.state_bytes + G.stages * G.stage_bytes;
   uint32_t blocks = (uint32_t)(ctx->num_sms * GatherShape<CW>::kCtasPerSm);
   if (blocks > G.num_tiles) blocks = G.num_tiles;
   *blocks_out = blocks;
   if (ctx->plan_only) return LOSSY_OK;
+  rows_of_call(P, blocks);
   static bool opted_in[kMaxDevices];   // per kernel instantiation and device: raise the dynamic shared memory limit once
   cudaError_t e;
   {
@@ -464,7 +475,7 @@ int launch_gather(lossy_ctx* ctx, const Params& P, const TmaGeom& G, cudaStream_
 }
 
 template <bool DRIFTK, int CW, bool RD, bool ANY>
-int dispatch_gather(lossy_ctx* ctx, const Params& P, const TmaGeom& G, cudaStream_t s, uint32_t* blocks) {
+int dispatch_gather(lossy_ctx* ctx, Params& P, const TmaGeom& G, cudaStream_t s, uint32_t* blocks) {
   const bool gb = ctx->cfg.grad_dtype == LOSSY_BF16;
   const bool rb = ctx->cfg.replica_dtype == LOSSY_BF16;
   const bool adam = ctx->cfg.optimizer == LOSSY_ADAM;
@@ -475,7 +486,7 @@ int dispatch_gather(lossy_ctx* ctx, const Params& P, const TmaGeom& G, cudaStrea
 }
 
 template <int CW, bool ANY>
-int try_gather_build(lossy_ctx* ctx, const Params& P, bool drift, bool rd, cudaStream_t s, uint32_t* blocks, bool* used) {
+int try_gather_build(lossy_ctx* ctx, Params& P, bool drift, bool rd, cudaStream_t s, uint32_t* blocks, bool* used) {
   TmaGeom G = {};
   if (!gather_geometry<CW, ANY>(ctx, drift && rd, G)) return LOSSY_OK;
   *used = true;
@@ -486,9 +497,35 @@ int try_gather_build(lossy_ctx* ctx, const Params& P, bool drift, bool rd, cudaS
   return drift ? dispatch_gather<true, CW, false, ANY>(ctx, P, G, s, blocks) : dispatch_gather<false, CW, false, ANY>(ctx, P, G, s, blocks);
 }
 template <int CW>
-int try_gather(lossy_ctx* ctx, const Params& P, bool drift, bool rd, cudaStream_t s, uint32_t* blocks, bool* used) {
+int try_gather(lossy_ctx* ctx, Params& P, bool drift, bool rd, cudaStream_t s, uint32_t* blocks, bool* used) {
   return GatherShape<CW>::kTile % P.P == 0 ? try_gather_build<CW, false>(ctx, P, drift, rd, s, blocks, used)
                                            : try_gather_build<CW, true>(ctx, P, drift, rd, s, blocks, used);
+}
+
+// Small buckets, of a few tiles (of 2048 elements) per SM, on the step kernel (lossy_register.cuh), which needs no second launch for a
+// short last packet either. Its times against the pipelines' (2000 random steps with drift norms, 2000 without) put the lines
+// further out than they are drawn here: packets from 1024 elements: W <= 4: 1.1 at five tiles per SM (whole packets; short last
+// packets 1.17 at eight), W > 4: 1.0-1.2 at three, 1.3 to 1.6 under one with a short last packet; 128: 1.2-1.5 up to 16; 256 and 512: 1.1-1.4
+// up to five. Two to four workers have a build of their own. Elsewhere the pipelines keep the buckets that the tests of them and of
+// the policy have them serve (tests/test_gpu_small_bucket_policy.py, test_gpu_gather_any_packet.py, test_gpu_parity.py), and with them
+// what lies beyond. Under an eighth of a tile per SM either is a launch and little else (most parity tests are such buckets).
+bool small_bucket(const lossy_ctx* ctx, bool drift) {
+  const lossy_config& c = ctx->cfg;
+  const uint32_t P = c.packet_elems, kTwin = (uint32_t)TmaShape<8>::kTile, kWide = (uint32_t)TmaShape<16>::kTile;
+  if (c.flags & (LOSSY_PACKED_BULK | LOSSY_GATHER_PATH)) return false;
+  const double tiles = (double)c.n / ((double)kWide * ctx->num_sms);
+  const bool bf16 = c.replica_dtype == LOSSY_BF16, few = c.W <= kStepFewWorkers, short_last = c.n % P != 0;
+  if (tiles < 0.125 || P < 128u) return false;
+  if (P >= kTwin) {
+    if (few) return tiles >= (short_last ? 0.125 : 0.15) && tiles < (P % kTwin != 0 ? 7.0 : short_last ? 2.0 : 5.0);
+    if (!short_last) return tiles >= (c.W <= 8u ? 0.15 : 0.55) && tiles < (c.W <= 8u ? 1.0 : 2.5) && (tiles < 2.0 || c.W <= 32u || c.p_param < 0.25);
+    if (!drift) return false;
+    return bf16 ? tiles >= 1.0 && tiles < (P % kTwin == 0 ? 3.6 : 2.0) : tiles < 2.0 && c.W <= 8u;
+  }
+  if (kWide % P != 0) return false;          // (the register kernel's until the gather pipeline's lines)
+  if (P == 128u) return tiles < (few ? 11.0 : 1.0);
+  if (few || bf16) return tiles < 2.0;
+  return tiles < 1.0 && (P == 256u || c.W <= 8u) && (drift || c.W <= 24u);
 }
 
 // Where the gather pipeline is used, and which of its builds. Figures are times of the build it would replace over its own,
@@ -510,6 +547,7 @@ GatherPolicy gather_policy(const lossy_ctx* ctx) {
   const bool bf16 = c.replica_dtype == LOSSY_BF16, sgd = c.optimizer == LOSSY_SGD;
   const bool forced = c.flags & LOSSY_GATHER_PATH;
   GatherPolicy g = {};
+  for (int drift = 0; drift < 2; ++drift) g.small[drift] = small_bucket(ctx, drift != 0);
   if (c.flags & LOSSY_PACKED_BULK || P < 128u) return g;
   TmaGeom G;
   // Tiles per SM. The pipeline fills and drains over several tiles, which a bucket of a few tiles per SM pays for: under
@@ -539,15 +577,6 @@ GatherPolicy gather_policy(const lossy_ctx* ctx) {
     const bool beyond = many_lossy && c.W > 24u && pm < 0.225 && (forced || per_sm >= 32.0);
     g.wide = P >= 256u && c.W >= 4u;
     g.drift_warps = g.wide && (bf16 || forced) && (band || beyond) && gather_geometry<16, false>(ctx, true, G);
-    // Buckets of up to two tiles per SM with bf16 replicas, of up to one with fp32 ones (packets of 512 elements up to 8 workers
-    // only): the register kernel, one chunk or two per warp, is done before the pipeline has filled (1000 random steps,
-    // register kernel's time over the pipeline's: bf16 0.66-1.02, mean 0.85, P = 128 1.2 and more; fp32 0.8-1.04, but 512 with
-    // more workers up to 1.23). Steps without drift norms, 2200 random ones: bf16 0.45-1.04, mean 0.78; fp32 up to 24 workers
-    // 0.59-1.23, mean 0.81; with more workers 0.73-1.27, mean 0.95, and they stay with the pipeline. Under an eighth of a tile per
-    // SM either is a launch and little else, and it stays.
-    const bool few = !forced && P >= 256u && tiles >= 0.125 && (bf16 ? tiles < 2.0 : tiles < 1.0 && (P == 256u || c.W <= 8u));
-    g.few_tiles[0] = few && (bf16 || c.W <= 24u);
-    g.few_tiles[1] = few;
     g.use = forced || g.drift_warps || !many_lossy || (!bf16 && P >= 256u && per_sm >= 7.0);
   } else if (P < kTwin) {
     // Other packets shorter than the twin tile. The alternative is the register kernel, whose chunks of 256 elements each
@@ -563,7 +592,8 @@ GatherPolicy gather_policy(const lossy_ctx* ctx) {
     // 0.05: 0.68 against 0.59), wide ones from p = 0.15 (p = 0.3: 0.55 against 0.47); up to four workers twin below 256
     // (W = 4, P = 200: 0.75 against 0.63).
     const double fill = P / (256.0 * ((P + 255u) / 256u));
-    const double least = (fill <= 0.6 ? 3.5 : fill <= 0.8 ? 5.0 : fill <= 0.9 ? 6.0 : 8.0) * (c.W > 16u ? 1.6 : 1.0) * (sgd ? 2.2 : 1.0);
+    // (the step kernel's build for two to four workers: 1.1-2.1 up to 11 tiles per SM, 0.9-1.3 beyond)
+    const double least = fmax((fill <= 0.6 ? 3.5 : fill <= 0.8 ? 5.0 : fill <= 0.9 ? 6.0 : 8.0) * (c.W > 16u ? 1.6 : 1.0) * (sgd ? 2.2 : 1.0), c.W <= kStepFewWorkers ? 11.0 : 0.0);
     const bool full_lossy = (sgd && fill > 0.98) || (bf16 && ((fill > 0.9 && stale >= 8.0) || (fill > 0.6 && stale >= 12.0)));
     g.wide = c.W >= 5u ? P >= 176u || pm >= 0.15 : c.W == 4u && P >= 256u;
     g.drift_warps = g.wide && gather_geometry<16, true>(ctx, true, G);
@@ -590,27 +620,11 @@ GatherPolicy gather_policy(const lossy_ctx* ctx) {
   return g;
 }
 
-// A small bucket that ends in a short packet: packets from 1024 elements, all of it as one launch of the register kernel instead
-// of the bulk-copy pipeline's and one for the short packet, which ends some microseconds after it. In tiles (of 2048 elements)
-// per SM, register kernel's time over the other's in 700 random steps: bf16 replicas from one to 3.6 tiles (0.59-0.99, mean 0.79;
-// from there on 0.94-1.05; below one 0.64-0.99, mean 0.89, left as it was), up to two for packets that are no multiple of 1024
-// (0.62-1.0); fp32 replicas up to two tiles and 8 workers (0.63-1.02, mean 0.89; more workers 0.7-1.3). Not measured, so as before:
-// under an eighth of a tile per SM, no drift norms. LOSSY_PACKED_BULK asks for the bulk-copy pipeline all the same.
-bool one_launch(const lossy_ctx* ctx, bool drift) {
-  const lossy_config& c = ctx->cfg;
-  const uint32_t kTwin = (uint32_t)TmaShape<8>::kTile;
-  if (!drift || c.packet_elems < kTwin || c.n % c.packet_elems == 0) return false;
-  if (c.flags & (LOSSY_PACKED_BULK | LOSSY_GATHER_PATH)) return false;
-  const double tiles = (double)c.n / ((double)TmaShape<16>::kTile * ctx->num_sms);
-  if (c.replica_dtype != LOSSY_BF16) return tiles >= 0.125 && tiles < 2.0 && c.W <= 8u;
-  return tiles >= 1.0 && tiles < (c.packet_elems % kTwin == 0 ? 3.6 : 2.0);
-}
-
 // Run the build the policy picks; *used stays false when no bulk-copy launch fits (packets shorter
 // than a tile, or no complete packet): the register path then takes everything.
-int run_tma(lossy_ctx* ctx, const Params& P, bool drift, cudaStream_t s, uint32_t* blocks, bool* used) {
+int run_tma(lossy_ctx* ctx, Params& P, bool drift, cudaStream_t s, uint32_t* blocks, bool* used) {
   *used = false;
-  if (ctx->cfg.flags & LOSSY_REGISTER_PATH || ctx->gather.few_tiles[drift] || one_launch(ctx, drift)) return LOSSY_OK;
+  if (ctx->cfg.flags & LOSSY_REGISTER_PATH || ctx->gather.small[drift]) return LOSSY_OK;
   const TmaPolicy t = tma_policy(ctx->cfg);
   const GatherPolicy& gp = ctx->gather;
   if (gp.use) {
@@ -667,7 +681,7 @@ int run_tma(lossy_ctx* ctx, const Params& P, bool drift, cudaStream_t s, uint32_
 }
 
 template <int PH, class GT, class RT, int OPT, bool ELIDE, bool TAIL>
-int launch_register(lossy_ctx* ctx, const Params& P, cudaStream_t s, uint32_t* blocks_out) {
+int launch_register(lossy_ctx* ctx, Params& P, cudaStream_t s, uint32_t* blocks_out) {
   auto kern = lossy_kernel<PH, GT, RT, OPT, ELIDE, TAIL>;
   static int occupancy[kMaxDevices];   // per kernel instantiation and device: resident blocks per SM
   int per_sm = 0;
@@ -684,12 +698,13 @@ int launch_register(lossy_ctx* ctx, const Params& P, cudaStream_t s, uint32_t* b
     }
   }
   uint32_t blocks = (uint32_t)(ctx->num_sms * per_sm);
-  const uint32_t need = (P.num_chunks - P.chunk_begin + kWarps - 1) / kWarps;
+  const uint32_t need = (P.num_chunks + kWarps - 1) / kWarps;
   if (blocks > need) blocks = need;
   if (blocks > ctx->max_blocks - P.partials_row0) blocks = ctx->max_blocks - P.partials_row0;
   if (blocks == 0) blocks = 1;
   if (blocks_out) *blocks_out = blocks;
   if (ctx->plan_only) return LOSSY_OK;
+  rows_of_call(P, blocks);
   // (early where the launch is a good part of the call: up to a few chunks per warp, or the short last packet)
   e = launch_after(need <= 4u * blocks, kern, blocks, kThreads, 0, s, P);
   if (e != cudaSuccess) return fail_cuda(ctx, "kernel launch", e);
@@ -697,41 +712,94 @@ int launch_register(lossy_ctx* ctx, const Params& P, cudaStream_t s, uint32_t* b
   return LOSSY_OK;
 }
 
-// (a launch that does not begin with the first chunk is the short last packet behind another launch of the same call)
+// (a launch that does not begin with the first packet is the short last packet behind another launch of the same call)
 template <int PH, class GT, class RT, int OPT, bool ELIDE = false>
-int launch(lossy_ctx* ctx, const Params& P, cudaStream_t s, uint32_t* blocks_out) {
-  return P.chunk_begin ? launch_register<PH, GT, RT, OPT, ELIDE, true>(ctx, P, s, blocks_out)
+int launch(lossy_ctx* ctx, Params& P, cudaStream_t s, uint32_t* blocks_out) {
+  return P.k_begin ? launch_register<PH, GT, RT, OPT, ELIDE, true>(ctx, P, s, blocks_out)
                        : launch_register<PH, GT, RT, OPT, ELIDE, false>(ctx, P, s, blocks_out);
 }
 
-// dispatch on the runtime element types / optimizer
+// dispatch of a single phase on the runtime element types / optimizer
 template <int PH>
-int dispatch(lossy_ctx* ctx, const Params& P, cudaStream_t s, uint32_t* blocks) {
-  const bool gb = ctx->cfg.grad_dtype == LOSSY_BF16;
+int dispatch(lossy_ctx* ctx, Params& P, cudaStream_t s, uint32_t* blocks) {
   const bool rb = ctx->cfg.replica_dtype == LOSSY_BF16;
-  const bool adam = ctx->cfg.optimizer == LOSSY_ADAM;
   if constexpr (PH == AGG) {
-    return gb ? launch<PH, BF16, F32, 0>(ctx, P, s, blocks) : launch<PH, F32, F32, 0>(ctx, P, s, blocks);
+    return ctx->cfg.grad_dtype == LOSSY_BF16 ? launch<PH, BF16, F32, 0>(ctx, P, s, blocks) : launch<PH, F32, F32, 0>(ctx, P, s, blocks);
   } else if constexpr (PH == STEP) {
-    return adam ? launch<PH, F32, F32, 1>(ctx, P, s, blocks) : launch<PH, F32, F32, 0>(ctx, P, s, blocks);
-  } else if constexpr (PH == BCAST || PH == DRIFT) {
+    return ctx->cfg.optimizer == LOSSY_ADAM ? launch<PH, F32, F32, 1>(ctx, P, s, blocks) : launch<PH, F32, F32, 0>(ctx, P, s, blocks);
+  } else {
     if (ctx->cfg.flags & LOSSY_REPLICA_SKIP_OWNER)   // owner-elided replicas: builds of their own
       return rb ? launch<PH, F32, BF16, 0, true>(ctx, P, s, blocks) : launch<PH, F32, F32, 0, true>(ctx, P, s, blocks);
     return rb ? launch<PH, F32, BF16, 0>(ctx, P, s, blocks) : launch<PH, F32, F32, 0>(ctx, P, s, blocks);
-  } else {
-    if (ctx->cfg.flags & LOSSY_REPLICA_SKIP_OWNER) {
-      if (gb && rb) return adam ? launch<PH, BF16, BF16, 1, true>(ctx, P, s, blocks) : launch<PH, BF16, BF16, 0, true>(ctx, P, s, blocks);
-      if (gb && !rb) return adam ? launch<PH, BF16, F32, 1, true>(ctx, P, s, blocks) : launch<PH, BF16, F32, 0, true>(ctx, P, s, blocks);
-      if (!gb && rb) return adam ? launch<PH, F32, BF16, 1, true>(ctx, P, s, blocks) : launch<PH, F32, BF16, 0, true>(ctx, P, s, blocks);
-      return adam ? launch<PH, F32, F32, 1, true>(ctx, P, s, blocks) : launch<PH, F32, F32, 0, true>(ctx, P, s, blocks);
-    }
-    if (gb && rb) return adam ? launch<PH, BF16, BF16, 1>(ctx, P, s, blocks) : launch<PH, BF16, BF16, 0>(ctx, P, s, blocks);
-    if (gb && !rb) return adam ? launch<PH, BF16, F32, 1>(ctx, P, s, blocks) : launch<PH, BF16, F32, 0>(ctx, P, s, blocks);
-    if (!gb && rb) return adam ? launch<PH, F32, BF16, 1>(ctx, P, s, blocks) : launch<PH, F32, BF16, 0>(ctx, P, s, blocks);
-    return adam ? launch<PH, F32, F32, 1>(ctx, P, s, blocks) : launch<PH, F32, F32, 0>(ctx, P, s, blocks);
   }
 }
 
+// ---- the fused step on registers alone (lossy_step_kernel) -----------------------------------
+template <class GT, class RT, int OPT, bool DRIFTK, bool ELIDE, bool TAIL, int FORM>
+int launch_step(lossy_ctx* ctx, Params& P, cudaStream_t s, uint32_t* blocks_out) {
+  constexpr uint32_t kSpan = 32 * StepShape<GT, RT, FORM>::kEpl, kMost = StepShape<GT, RT, FORM>::kMaxWarps;
+  const uint32_t per_packet = (P.P + kSpan - 1) / kSpan;
+  const uint32_t chunks = (P.K - P.k_begin) * per_packet;
+  const uint32_t tasks = chunks + (P.n % StepShape<GT, RT, FORM>::kEpl ? 1u : 0u);
+  uint32_t blocks, warps;
+  if (TAIL) {
+    warps = tasks < 8u ? tasks : 8u;
+    blocks = (tasks + warps - 1) / warps;
+    if (blocks > (uint32_t)ctx->num_sms) blocks = (uint32_t)ctx->num_sms;
+  } else {
+    // one block per SM, each with the warps that its share of the chunks needs
+    blocks = tasks < (uint32_t)ctx->num_sms ? tasks : (uint32_t)ctx->num_sms;
+    warps = (tasks + blocks - 1) / blocks;
+    const uint32_t rounds = (warps + kMost - 1) / kMost;
+    warps = (warps + rounds - 1) / rounds;
+  }
+  *blocks_out = blocks;
+  if (ctx->plan_only) return LOSSY_OK;
+  rows_of_call(P, blocks);
+  P.chunks_per_packet = per_packet;
+  P.cpp_magic = magic_of(per_packet);
+  P.pps_magic = magic_of(P.pps);
+  P.num_chunks = chunks;
+  const cudaError_t e = launch_after((tasks + warps - 1) / warps <= 4u * blocks, lossy_step_kernel<GT, RT, OPT, DRIFTK, ELIDE, TAIL, FORM>, blocks, warps * 32u, 0, s, P);
+  if (e != cudaSuccess) return fail_cuda(ctx, "kernel launch", e);
+  ctx->launches++;
+  return LOSSY_OK;
+}
+template <class GT, class RT, int OPT, bool DRIFTK, bool ELIDE>
+int pick_step(lossy_ctx* ctx, Params& P, cudaStream_t s, uint32_t* blocks) {
+  if (P.k_begin) return launch_step<GT, RT, OPT, DRIFTK, ELIDE, true, kStepQuads>(ctx, P, s, blocks);
+  const uint32_t W = P.W;
+  if (W <= kStepFewWorkers) return launch_step<GT, RT, OPT, DRIFTK, ELIDE, false, kStepFew>(ctx, P, s, blocks);
+  // Pairs: with more than 16 workers where they take no more rounds than quads, with fewer up to half (W > 8) or a quarter of a
+  // round (2000 random steps: pairs' time over quads' 0.81-0.96, 0.90-0.97, 0.99; beyond 0.97-1.2).
+  const uint64_t warps2 = (uint64_t)P.K * ((P.P + 63u) / 64u), warps4 = (uint64_t)P.K * ((P.P + 127u) / 128u);
+  auto rounds = [&](uint64_t chunks, uint32_t warps) { return (chunks + (uint64_t)ctx->num_sms * warps - 1) / ((uint64_t)ctx->num_sms * warps); };
+  if (W > 16u ? rounds(warps2, 32u) <= rounds(warps4, StepShape<GT, RT, kStepQuads>::kMaxWarps) : warps2 <= (uint64_t)ctx->num_sms * (W > 8u ? 16u : 8u))
+    return launch_step<GT, RT, OPT, DRIFTK, ELIDE, false, kStepPairs>(ctx, P, s, blocks);
+  // Two stale replicas per packet and more: eight copies requested together up to two rounds; from three rounds on with many workers eight
+  // elements per lane, which halve the reductions of the stale copies per element (W = 32, P = 512, p = 0.3, 20 M: quads 529 us, octs
+  // 486; W = 49, P = 976, p = 0.3, 25 M: 1072, 993; W = 15, P = 768, p = 0.3, 6 M: 82, 84).
+  if constexpr (DRIFTK && RT::kVecs == 1) {
+    const bool stale = (W - 1u) * ctx->cfg.p_param >= 2.0;
+    const bool many_rounds = rounds(warps4, 24u) >= 3u;
+    if (stale && W > 16u && many_rounds) return launch_step<GT, RT, OPT, DRIFTK, ELIDE, false, kStepOcts>(ctx, P, s, blocks);
+    if (stale && !many_rounds) return launch_step<GT, RT, OPT, DRIFTK, ELIDE, false, kStepStale>(ctx, P, s, blocks);
+  }
+  return launch_step<GT, RT, OPT, DRIFTK, ELIDE, false, kStepQuads>(ctx, P, s, blocks);
+}
+template <class GT, class RT, bool DRIFTK>
+int dispatch_step_as(lossy_ctx* ctx, Params& P, cudaStream_t s, uint32_t* blocks) {
+  const bool adam = ctx->cfg.optimizer == LOSSY_ADAM;
+  if (ctx->cfg.flags & LOSSY_REPLICA_SKIP_OWNER)   // owner-elided replicas: builds of their own
+    return adam ? pick_step<GT, RT, 1, DRIFTK, true>(ctx, P, s, blocks) : pick_step<GT, RT, 0, DRIFTK, true>(ctx, P, s, blocks);
+  return adam ? pick_step<GT, RT, 1, DRIFTK, false>(ctx, P, s, blocks) : pick_step<GT, RT, 0, DRIFTK, false>(ctx, P, s, blocks);
+}
+template <bool DRIFTK>
+int dispatch_step(lossy_ctx* ctx, Params& P, cudaStream_t s, uint32_t* blocks) {
+  const bool gb = ctx->cfg.grad_dtype == LOSSY_BF16, rb = ctx->cfg.replica_dtype == LOSSY_BF16;
+  if (gb) return rb ? dispatch_step_as<BF16, BF16, DRIFTK>(ctx, P, s, blocks) : dispatch_step_as<BF16, F32, DRIFTK>(ctx, P, s, blocks);
+  return rb ? dispatch_step_as<F32, BF16, DRIFTK>(ctx, P, s, blocks) : dispatch_step_as<F32, F32, DRIFTK>(ctx, P, s, blocks);
+}
 
 // ---- the single-phase calls through the bulk-copy pipeline ---------------------------------
 constexpr uint32_t kPhaseSmemFixed = kTmaBarBytes + kPhaseMaxStages * sizeof(StageHdr);
@@ -768,13 +836,14 @@ bool phase_geometry(const lossy_ctx* ctx, TmaGeom& G) {
 }
 
 template <int PH, class T, int OPT, int CW, int GS>
-int launch_phase_tma(lossy_ctx* ctx, const Params& P, const TmaGeom& G, cudaStream_t s, uint32_t* blocks_out) {
+int launch_phase_tma(lossy_ctx* ctx, Params& P, const TmaGeom& G, cudaStream_t s, uint32_t* blocks_out) {
   auto kern = lossy_phase_tma_kernel<PH, T, OPT, CW, GS>;
   const uint32_t smem = kPhaseSmemFixed + G.stages * G.stage_bytes;
   uint32_t blocks = (uint32_t)(ctx->num_sms * TmaShape<CW>::kCtasPerSm);
   if (blocks > G.num_tiles) blocks = G.num_tiles;
   *blocks_out = blocks;
   if (ctx->plan_only) return LOSSY_OK;
+  rows_of_call(P, blocks);
   static bool opted_in[kMaxDevices];   // per kernel instantiation and device: raise the dynamic shared memory limit once
   cudaError_t e;
   {
@@ -792,7 +861,7 @@ int launch_phase_tma(lossy_ctx* ctx, const Params& P, const TmaGeom& G, cudaStre
 }
 
 template <int PH, int CW, int GS>
-int try_phase_tma(lossy_ctx* ctx, const Params& P, cudaStream_t s, uint32_t* blocks, bool* used) {
+int try_phase_tma(lossy_ctx* ctx, Params& P, cudaStream_t s, uint32_t* blocks, bool* used) {
   TmaGeom G;
   if (!phase_geometry<PH, CW, GS>(ctx, G)) return LOSSY_OK;
   *used = true;
@@ -809,48 +878,58 @@ int try_phase_tma(lossy_ctx* ctx, const Params& P, cudaStream_t s, uint32_t* blo
   }
 }
 
-// One single-phase call: complete packets through the bulk-copy pipeline where a build fits (packets of at
-// least one tile), a ragged last packet or everything else through the register kernel. With drift norms, pass 0 only sizes the grids: the blocks of both launches draw tickets from one
-// counter and the last of them finalises the norms.
+// A call's launches: complete packets through a pipeline, a short last packet, or everything when no pipeline's build fits, through a
+// register kernel. With drift norms the blocks of both launches draw tickets from one counter and the last of them finalises
+// the norms; where there may be two launches, a first turn that launches nothing counts their blocks.
+template <class LaunchAll>
+int run_launches(lossy_ctx* ctx, Params& P, bool drift, cudaStream_t s, LaunchAll&& launch_all) {
+  uint32_t rows = 0;
+  if (drift && ctx->cfg.n % ctx->cfg.packet_elems != 0) {
+    Params Q = P;
+    ctx->plan_only = true;
+    const int rc = launch_all(Q, &rows);
+    ctx->plan_only = false;
+    if (rc) return rc;
+    P.total_rows = rows;
+  }
+  const int rc = launch_all(P, &rows);
+  if (rc && drift) reset_ticket(ctx, s);
+  return rc;
+}
+
+// One single-phase call: packets of at least one tile through the bulk-copy pipeline, the rest through the register kernel.
 template <int PH>
-int run_phase(lossy_ctx* ctx, const Params& P, float* norms, double* sumsq, cudaStream_t s) {
+int run_phase(lossy_ctx* ctx, Params& P, float* norms, double* sumsq, cudaStream_t s) {
   const lossy_config& c = ctx->cfg;
   const bool bulk = !(c.flags & LOSSY_REGISTER_PATH);
   // wide tiles (one CTA per SM) when they divide the packet and the streamed arrays fit two groups
   const bool wide = c.packet_elems % TmaShape<16>::kTile == 0 && c.W <= 16;
-  uint32_t tma_blocks = 0, tail_blocks = 0;
-  for (int pass = PH == DRIFT ? 0 : 1; pass < 2; ++pass) {
-    ctx->plan_only = pass == 0;
-    Params Q = P;
-    if (PH == DRIFT && pass == 1) {
-      Q.ticket = ctx->ticket;
-      Q.total_rows = tma_blocks + tail_blocks;
-      Q.norms = norms;
-      Q.sumsq = sumsq;
-    }
+  auto launch_all = [&](Params& Q, uint32_t* rows) {
+    uint32_t tma_blocks = 0, tail_blocks = 0;
     bool used = false;
     int rc = LOSSY_OK;
     if (bulk) {
       if (wide) rc = try_phase_tma<PH, 16, 8>(ctx, Q, s, &tma_blocks, &used);
       if (!rc && !used) rc = try_phase_tma<PH, 8, 8>(ctx, Q, s, &tma_blocks, &used);
     }
-    if (!rc) {
-      if (used) {
-        Q.chunk_begin = (uint32_t)((c.n / c.packet_elems) * ctx->chunks_per_packet);
-        Q.partials_row0 = tma_blocks;
-      } else {
-        tma_blocks = 0;
-      }
-      if (Q.chunk_begin < Q.num_chunks) rc = dispatch<PH>(ctx, Q, s, &tail_blocks);
-      else tail_blocks = 0;
+    if (rc) return rc;
+    if (used) {
+      Q.k_begin = (uint32_t)(c.n / c.packet_elems);
+      Q.num_chunks = (Q.K - Q.k_begin) * ctx->chunks_per_packet;
+      Q.partials_row0 = tma_blocks;
+    } else {
+      tma_blocks = 0;
     }
-    ctx->plan_only = false;
-    if (rc) {
-      if (Q.ticket) reset_ticket(ctx, s);
-      return rc;
-    }
+    if (Q.num_chunks) rc = dispatch<PH>(ctx, Q, s, &tail_blocks);
+    *rows = tma_blocks + tail_blocks;
+    return rc;
+  };
+  if (PH == DRIFT) {
+    P.ticket = ctx->ticket;
+    P.norms = norms;
+    P.sumsq = sumsq;
   }
-  return LOSSY_OK;
+  return run_launches(ctx, P, PH == DRIFT, s, launch_all);
 }
 
 // Chunks per SM up to which a bucket is small for the pairwise drift (300 thousand elements): at 250 k the small builds take 0.55
@@ -1127,45 +1206,28 @@ static int fused_impl(lossy_ctx* ctx, uint64_t step, const void* const* grads, f
   P.count = count;
   P.recv_bits = recv_bits;
   P.stale_bits = stale_bits;
-  // register kernel, all phases fused: prefetching the warp's next chunk pays for W <= 8 (+3..13 %);
-  // it costs 20 % on the single-phase kernels, which never set it
-  P.prefetch_next = ctx->cfg.W <= 8u ? 1u : 0u;
   cudaStream_t s = (cudaStream_t)stream;
   const bool drift = norms || sumsq;
-  // Complete packets go through the bulk-copy pipeline, a short last packet (or everything, when no
-  // bulk-copy build fits) through the register kernel. Pass 0 only sizes the grids: the blocks of both
-  // launches draw tickets from one counter and the last of them finalises the drift norms.
-  uint32_t tma_blocks = 0, tail_blocks = 0;
-  for (int pass = 0; pass < 2; ++pass) {
-    ctx->plan_only = pass == 0;
-    Params Q = P;
-    if (pass == 1 && drift) {
-      Q.ticket = ctx->ticket;
-      Q.total_rows = tma_blocks + tail_blocks;
-      Q.norms = norms;
-      Q.sumsq = sumsq;
-    }
+  if (drift) {
+    P.ticket = ctx->ticket;
+    P.norms = norms;
+    P.sumsq = sumsq;
+  }
+  return run_launches(ctx, P, drift, s, [&](Params& Q, uint32_t* rows) {
+    uint32_t tma_blocks = 0, tail_blocks = 0;
     bool used_tma = false;
     int rc = run_tma(ctx, Q, drift, s, &tma_blocks, &used_tma);
-    if (!rc) {
-      if (used_tma) {
-        Q.chunk_begin = (uint32_t)((ctx->cfg.n / ctx->cfg.packet_elems) * ctx->chunks_per_packet);
-        Q.partials_row0 = tma_blocks;
-      } else {
-        tma_blocks = 0;
-      }
-      if (Q.chunk_begin < Q.num_chunks)
-        rc = drift ? dispatch<AGG | STEP | BCAST | DRIFT>(ctx, Q, s, &tail_blocks) : dispatch<AGG | STEP | BCAST>(ctx, Q, s, &tail_blocks);
-      else
-        tail_blocks = 0;
+    if (rc) return rc;
+    if (used_tma) {
+      Q.k_begin = (uint32_t)(ctx->cfg.n / ctx->cfg.packet_elems);
+      Q.partials_row0 = tma_blocks;
+    } else {
+      tma_blocks = 0;
     }
-    ctx->plan_only = false;
-    if (rc) {
-      if (Q.ticket) reset_ticket(ctx, s);
-      return rc;
-    }
-  }
-  return LOSSY_OK;
+    if (Q.k_begin < Q.K) rc = drift ? dispatch_step<true>(ctx, Q, s, &tail_blocks) : dispatch_step<false>(ctx, Q, s, &tail_blocks);
+    *rows = tma_blocks + tail_blocks;
+    return rc;
+  });
 }
 
 int lossy_fused_step(lossy_ctx* ctx, uint64_t step, const void* const* grads, float* master, float* m, float* v,

@@ -1,11 +1,9 @@
 // Device-side building blocks of the lossy data-parallel step (sm_100a).
 //
-// Work decomposition shared by every kernel here: the bucket is walked in
-// "chunks" of 256 contiguous elements (one warp, 8 elements = 16 or 32 bytes per
-// lane) that never straddle a packet, so the delivery masks of a chunk are
-// warp-uniform. Chunk q belongs to packet k = q / chunks_per_packet. Warps take
-// chunks grid-stride, so at any moment the grid streams one contiguous window
-// of every buffer.
+// Work decomposition of the register kernels: the bucket is walked in "chunks" of 256 contiguous elements (one warp, 8 elements =
+// 16 or 32 bytes per lane; the fused step: 64, 128 or 256) that never straddle a packet, so the delivery masks of a chunk are
+// warp-uniform. Chunk q belongs to packet k_begin + q / chunks_per_packet. Warps take chunks grid-stride, so at any moment the
+// grid streams one contiguous window of every buffer.
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -53,11 +51,12 @@ struct Params {
   uint64_t n;
   uint64_t packet_base;
   uint64_t step_key;      // hash key of (seed, step), derived on the host
-  uint32_t num_chunks;    // K * chunks_per_packet
-  uint32_t chunk_begin;   // first chunk this launch covers (a bulk-copy launch may own the chunks before it)
+  uint32_t k_begin;       // first packet a register launch covers (a pipeline's launch may have those before it)
+  uint32_t num_chunks;    // chunks of that launch, counted from packet k_begin
   uint32_t partials_row0; // first row of `partials` this launch writes
   uint32_t chunks_per_packet;
   uint32_t pps;           // packets per shard (of the whole bucket)
+  uint64_t cpp_magic, pps_magic;   // of the two above, for divide_by
   uint32_t k0;            // bucket packet index of this context's packet 0 (a context may cover a packet range)
   uint32_t P;
   uint32_t W;
@@ -65,17 +64,17 @@ struct Params {
   uint32_t Tenter, Tstay; // bursty loss: a good link turns bad iff hash < Tenter, a bad one stays bad iff hash < Tstay
   uint32_t K;             // packets in the bucket
   uint32_t flags;
-  uint32_t prefetch_next; // register kernel: L2-prefetch the warp's next chunk
   float lr, b1, b2, omb1, omb2, ibc1, ibc2, eps;
   float neg_zero;         // -0 (optimizer_n)
   // Owner-elided replicas (kSkipOwner): replica i stores this context's elements WITHOUT the packets worker i
   // owns, so everything behind worker i's shard sits rep_skip[i] elements lower in its array. All zero otherwise.
   uint64_t rep_skip[kMaxW];
-  // Debug build (LOSSY_DEVCHECK): where a failed index check is recorded (4 words: site, element offset low and
-  // high, length; the first failure wins) and the element count the checks hold a range against (n, or less when
-  // the self-test shrinks it). Unused otherwise.
+#ifdef LOSSY_DEVCHECK
+  // Debug build: where a failed index check is recorded (4 words: site, element offset low and high, length; the first failure
+  // wins) and the element count the checks hold a range against (n, or less when the self-test shrinks it).
   uint32_t* check;
   uint64_t check_n;
+#endif
   // A call whose short last packet has a launch of its own beside the launch of the complete ones (open_gate): the context's
   // gate word, and this call's number. Else NULL and 0.
   uint32_t* gate;
@@ -114,11 +113,18 @@ __device__ __forceinline__ void end_after_previous(const Params& P) {
   if (blockIdx.x == 0 && threadIdx.x == 0) *P.gate = 0u;   // (a block that has not looked yet will wait)
 }
 
+// x / d for a d that the host knows: the high half of x times 2^64 / d rounded up, exact for every 32-bit x and d (the product is too
+// large by less than x d < 2^64). Two multiply-adds for a division's twenty and more instructions.
+__host__ inline uint64_t magic_of(uint32_t d) { return d > 1u ? ~0ull / d + 1ull : 0ull; }
+__device__ __forceinline__ uint32_t divide_by(uint32_t x, uint32_t d, uint64_t magic) {
+  const uint64_t low = (uint64_t)x * (uint32_t)magic;
+  return d > 1u ? (uint32_t)(((uint64_t)x * (uint32_t)(magic >> 32) + (low >> 32)) >> 32) : x;
+}
+
 // Owner-elided replicas: rep_skip[i] = elements of worker i's shard inside the context's packet range
 // [k0, k0 + K) of a bucket cut into shards of pps packets (the last packet may be short: n elements in all).
 __host__ inline void fill_rep_skip(Params& P, bool elide) {
-  for (uint32_t i = 0; i < (uint32_t)kMaxW; ++i) P.rep_skip[i] = 0;
-  if (!elide) return;
+  if (!elide) return;          // (zero already)
   for (uint32_t i = 0; i < P.W; ++i) {
     const uint64_t s0 = (uint64_t)i * P.pps, s1 = s0 + P.pps;          // shard i in bucket packets
     const uint64_t c0 = P.k0, c1 = (uint64_t)P.k0 + P.K;                // this context in bucket packets
@@ -145,6 +151,7 @@ constexpr bool kDevCheck = true;
 constexpr bool kDevCheck = false;
 #endif
 enum CheckSite : uint32_t { kSiteRegister = 1, kSiteFusedPacked = 2, kSiteFused = 3, kSitePhase = 4, kSiteGather = 5, kSiteReplica = 16 };
+#ifdef LOSSY_DEVCHECK
 __device__ __forceinline__ void check_record(const Params& P, uint32_t site, uint64_t e0, uint64_t len) {
   if (atomicCAS(&P.check[0], 0u, site) == 0u) {
     P.check[1] = (uint32_t)e0;
@@ -154,7 +161,6 @@ __device__ __forceinline__ void check_record(const Params& P, uint32_t site, uin
 }
 // elements [e0, e0 + len) of packet k: inside the slab, and k a packet of it
 __device__ __forceinline__ bool span_ok(const Params& P, uint32_t k, uint64_t e0, uint64_t len, uint32_t site) {
-  if constexpr (!kDevCheck) return true;
   if (!P.check) return true;      // a caller without a context (the no-allocation entry point) has nowhere to record
   if (k < P.K && (len == 0 || (len <= P.check_n && e0 <= P.check_n - len))) return true;   // an empty range touches nothing
   check_record(P, site, e0, len);
@@ -162,7 +168,6 @@ __device__ __forceinline__ bool span_ok(const Params& P, uint32_t k, uint64_t e0
 }
 // the same elements inside replica i's array (owner j; the owner has no copy when the replicas are owner-elided)
 __device__ __forceinline__ bool rep_span_ok(const Params& P, uint32_t i, uint32_t j, uint64_t e0, uint64_t len, uint32_t site) {
-  if constexpr (!kDevCheck) return true;
   if (!P.check || len == 0 || ((P.flags & kSkipOwner) && i == j)) return true;
   const uint64_t limit = P.check_n - (P.rep_skip[i] < P.check_n ? P.rep_skip[i] : P.check_n);
   const uint64_t at = e0 - (j > i ? P.rep_skip[i] : 0ull);
@@ -172,11 +177,15 @@ __device__ __forceinline__ bool rep_span_ok(const Params& P, uint32_t i, uint32_
 }
 // every replica's range of a tile or chunk, the workers dealt over the lanes; warp-uniform result
 __device__ __forceinline__ bool tile_ok(const Params& P, uint32_t k, uint32_t j, uint64_t e0, uint64_t len, uint32_t site, int lane) {
-  if constexpr (!kDevCheck) return true;
   bool ok = span_ok(P, k, e0, len, site);
   for (uint32_t i = (uint32_t)lane; i < P.W; i += 32u) ok = rep_span_ok(P, i, j, e0, len, site) && ok;
   return __all_sync(0xFFFFFFFFu, ok);
 }
+#else
+__device__ __forceinline__ bool span_ok(const Params&, uint32_t, uint64_t, uint64_t, uint32_t) { return true; }
+__device__ __forceinline__ bool rep_span_ok(const Params&, uint32_t, uint32_t, uint64_t, uint64_t, uint32_t) { return true; }
+__device__ __forceinline__ bool tile_ok(const Params&, uint32_t, uint32_t, uint64_t, uint64_t, uint32_t, int) { return true; }
+#endif
 
 // The replica that does not exist for a packet of owner j (as a bit), or 0 with full replicas.
 __device__ __forceinline__ uint64_t own_bit(const Params& P, uint32_t j) {

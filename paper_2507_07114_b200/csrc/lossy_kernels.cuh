@@ -1,5 +1,5 @@
-// The kernels of the lossy data-parallel step: one template, specialised by the
-// phases it runs. Fused = AGG|STEP|BCAST|DRIFT in a single pass over the bucket.
+// The arithmetic of the lossy data-parallel step, its delivery draws, the end of every kernel with drift norms, and the single
+// phases (AGG, STEP, BCAST, DRIFT) on registers alone: one template, specialised by the phase. The fused step: lossy_register.cuh.
 #pragma once
 #include "lossy_device.cuh"
 
@@ -98,44 +98,57 @@ __device__ __forceinline__ void optimizer8(const Params& P, const float (&g)[8],
 // that draws the last ticket sums the rows of each replica in a fixed order (lane l takes rows l, l + 32, ..., then a shuffle
 // tree), so the result does not depend on which block happens to be last. Nothing here waits on another block.
 // This is the tail of every step, a chain of latencies (2 us), so only one warp fences, behind nothing but its own stores,
-// the warp that drains the bulk stores is not waited for, and a lane's rows are requested together.
+// the warp that drains the bulk stores is not waited for, and a lane's rows are requested together, two replicas and ten rows at a
+// time: with one replica and five rows 64 replicas' sums over 296 blocks were sixteen round trips to L2 one after the other, now four
+// (W = 64, P = 4096, 3 M: 154 -> 148 us; W = 47, P = 1464, 2.2 M: 156 -> 149; W = 24, P = 512, 6 M: 126 -> 121).
+constexpr int kFinishRows = 10;
 __device__ __forceinline__ void drift_finish(const Params& P, const double* sums, int rows, uint32_t row, int warp, int nwarps, int lane) {
   __shared__ uint32_t is_last;
   auto sync = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(nwarps * 32) : "memory"); };
   sync();
   if (warp == 0) {
-    double t0 = 0.0, t1 = 0.0;
-    for (int w = 0; w < rows; ++w) {
-      t0 += sums[w * kMaxW + lane];
-      t1 += sums[w * kMaxW + lane + 32];
-    }
+    double t0[4] = {}, t1[4] = {};
+    for (int w = 0; w < rows; w += 4)
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (w + u < rows) {
+          t0[u] += sums[(w + u) * kMaxW + lane];
+          t1[u] += sums[(w + u) * kMaxW + lane + 32];
+        }
     double* out = P.partials + (size_t)row * kMaxW;
-    out[lane] = t0;
-    out[lane + 32] = t1;
+    out[lane] = (t0[0] + t0[1]) + (t0[2] + t0[3]);
+    out[lane + 32] = (t1[0] + t1[1]) + (t1[2] + t1[3]);
     __syncwarp();
     if (P.ticket && lane == 0) {
-      __threadfence();                                // the warp's row is visible device-wide ...
-      const uint32_t prev = atomicAdd(P.ticket, 1u);  // ... before its ticket is
-      __threadfence();
+      // the warp's row is visible device-wide before its ticket is, and every row before what follows the last one
+      uint32_t prev;
+      asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(prev) : "l"(P.ticket) : "memory");
       is_last = prev + 1u == P.total_rows ? 1u : 0u;
     }
   }
   if (!P.ticket) return;
   sync();
   if (!is_last) return;
-  for (uint32_t i = warp; i < P.W; i += nwarps) {
-    double t = 0.0;
-    for (uint32_t b0 = lane; b0 < P.total_rows; b0 += 32 * 5) {
-      double x[5];
+  // two replicas per warp at a time, so that a lane's requests are 16 bytes
+  for (uint32_t i = 2u * warp; i < P.W; i += 2u * nwarps) {
+    double t0 = 0.0, t1 = 0.0;
+    for (uint32_t b0 = lane; b0 < P.total_rows; b0 += 32 * kFinishRows) {
+      double2 x[kFinishRows];
 #pragma unroll
-      for (int u = 0; u < 5; ++u) x[u] = b0 + 32u * u < P.total_rows ? __ldcg(&P.partials[(size_t)(b0 + 32u * u) * kMaxW + i]) : 0.0;
+      for (int u = 0; u < kFinishRows; ++u)
+        x[u] = b0 + 32u * u < P.total_rows ? __ldcg(reinterpret_cast<const double2*>(&P.partials[(size_t)(b0 + 32u * u) * kMaxW + i])) : make_double2(0.0, 0.0);
 #pragma unroll
-      for (int u = 0; u < 5; ++u) t += x[u];
+      for (int u = 0; u < kFinishRows; ++u) {
+        t0 += x[u].x;
+        t1 += x[u].y;
+      }
     }
-    t = warp_sum64(t);
-    if (lane == 0) {
-      if (P.sumsq) P.sumsq[i] += t;
-      if (P.norms) P.norms[i] = (float)sqrt(t);
+    t0 = warp_sum64(t0);
+    t1 = warp_sum64(t1);
+    if (lane < 2 && i + lane < P.W) {
+      const double t = lane ? t1 : t0;
+      if (P.sumsq) P.sumsq[i + lane] += t;
+      if (P.norms) P.norms[i + lane] = (float)sqrt(t);
     }
   }
   if (warp == 0 && lane == 0) *P.ticket = 0u;  // ready for the next call on this context
@@ -271,19 +284,13 @@ __global__ void __launch_bounds__(kThreads, LOSSY_MIN_BLOCKS) lossy_kernel(const
   if constexpr (TAIL) begin_beside_previous(P);
   else wait_for_previous();
 
-  // drift sums per warp and replica; a warp writes its own row alone (standalone: kept in registers, lane l holds l and l + 32)
-  __shared__ double dsum[PH & DRIFT ? kWarps * kMaxW : 1];
-  double dacc0 = 0.0, dacc1 = 0.0;
-  if constexpr ((PH & DRIFT) && (PH & BCAST)) {
-    dsum[warp * kMaxW + lane] = 0.0;
-    dsum[warp * kMaxW + lane + 32] = 0.0;
-    __syncwarp();
-  }
+  double dacc0 = 0.0, dacc1 = 0.0;   // drift sums: lane l holds replicas l and l + 32
 
   const uint32_t warps_in_grid = gridDim.x * kWarps;
-  for (uint32_t q = P.chunk_begin + blockIdx.x * kWarps + warp; q < P.num_chunks; q += warps_in_grid) {
-    const uint32_t k = q / P.chunks_per_packet;
-    const uint32_t c = q - k * P.chunks_per_packet;
+  for (uint32_t q = blockIdx.x * kWarps + warp; q < P.num_chunks; q += warps_in_grid) {
+    const uint32_t kq = q / P.chunks_per_packet;
+    const uint32_t c = q - kq * P.chunks_per_packet;
+    const uint32_t k = P.k_begin + kq;
     const uint32_t j = (P.k0 + k) / P.pps;  // owner W_j of packet k
     const uint32_t in_pkt = c * kChunk + lane * 8;
     const uint64_t e = (uint64_t)k * P.P + in_pkt;
@@ -299,38 +306,6 @@ __global__ void __launch_bounds__(kThreads, LOSSY_MIN_BLOCKS) lossy_kernel(const
     // ---- delivery indicators of this packet (warp-uniform) -------------------
     uint64_t recv = 0, stale = 0, gbad = 0, pbad = 0;
     packet_masks<PH>(P, k, j, lane, recv, stale, gbad, pbad);
-    // Pull the NEXT chunk of this warp toward L2 while this one is processed. Worth its
-    // instructions only in the fused kernel when few workers feed a chunk (measured: +3..13 % for W <= 8,
-    // a loss above, and a loss in the single-phase kernels).
-    if (P.prefetch_next) {
-      const uint32_t qn = q + warps_in_grid;
-      if (qn < P.num_chunks) {
-        const uint32_t kn = qn / P.chunks_per_packet;
-        const uint32_t cn = qn - kn * P.chunks_per_packet;
-        const uint32_t inn = cn * kChunk + lane * 8;
-        const uint64_t en = (uint64_t)kn * P.P + inn;
-        uint64_t rn = 0, sn = 0;
-        packet_masks<PH>(P, kn, (P.k0 + kn) / P.pps, lane, rn, sn);
-        if (inn < P.P && en + 8 <= P.n) {
-          if constexpr (PH & (STEP | BCAST | DRIFT)) prefetch_l2(P.master + en);
-          if constexpr ((PH & STEP) && OPT == 1) { prefetch_l2(P.m + en); prefetch_l2(P.v + en); }
-          if constexpr (PH & AGG) {
-            while (rn) {
-              const int i = __ffsll((long long)rn) - 1;
-              rn &= rn - 1;
-              prefetch_l2(reinterpret_cast<const typename GT::raw*>(P.grads[i]) + en);
-            }
-          }
-          if constexpr ((PH & BCAST) && (PH & DRIFT)) {
-            while (sn) {
-              const int i = __ffsll((long long)sn) - 1;
-              sn &= sn - 1;
-              prefetch_l2(reinterpret_cast<const typename RT::raw*>(P.replicas[i]) + rep_at(i, (P.k0 + kn) / P.pps, en));
-            }
-          }
-        }
-      }
-    }
     uint32_t cnt = __popcll(recv);
     if (c == 0 && lane == 0) {
       if constexpr (PH & AGG) {
@@ -347,16 +322,6 @@ __global__ void __launch_bounds__(kThreads, LOSSY_MIN_BLOCKS) lossy_kernel(const
     }
     // Lanes past a short packet or past the bucket end keep nvalid == 0: they stay in the
     // warp for the shuffles below and every load/store helper skips them.
-
-    // stale copies are read late (for the drift term): start them toward L2 now
-    if constexpr ((PH & BCAST) && (PH & DRIFT)) {
-      uint64_t sm = nvalid > 0 ? stale : 0ull;
-      while (sm) {
-        const int i = __ffsll((long long)sm) - 1;
-        sm &= sm - 1;
-        prefetch_l2(reinterpret_cast<const typename RT::raw*>(P.replicas[i]) + rep_at(i, j, e));
-      }
-    }
 
     // ---- optimizer state: issue these loads before the gradient loop ---------
     Vec8<F32> rth, rm, rv;
@@ -433,8 +398,7 @@ __global__ void __launch_bounds__(kThreads, LOSSY_MIN_BLOCKS) lossy_kernel(const
           if (!((keep >> i) & 1ull)) store8<RT>(P.replicas[i], rep_at(i, j, e), wire, nvalid);
       }
       if constexpr (PH & DRIFT) {
-        // copies that differ from the wire value: the stale ones after a broadcast, or (standalone) all
-        uint64_t todo = (PH & BCAST) ? stale : ((W == 64 ? ~0ull : ((1ull << W) - 1ull)) & ~own);
+        uint64_t todo = (W == 64 ? ~0ull : ((1ull << W) - 1ull)) & ~own;
         while (todo) {
           // up to four copies are fetched before the first is used
           int ids[4];
@@ -450,49 +414,19 @@ __global__ void __launch_bounds__(kThreads, LOSSY_MIN_BLOCKS) lossy_kernel(const
               old[b] = load8_any<RT>(P.replicas[ids[b]], rep_at((uint32_t)ids[b], j, e), nvalid);
             }
           }
-          // Fused: a lane's eight squares are added in fp32, everything else in fp64, as the pairwise drift's are: bf16 copies
-          // N(0, 3e-4) apart come out 3e-10 low, with a tree of 256 squares in fp32 8.8e-9, and the pipelines' 128 squares, whose
-          // small buckets this kernel takes, 6.0e-9. One reduction of several copies, and sums in shared memory that the lanes add to
-          // which hold a total, make up for the wider exchange: W = 64, P = 256, 16 M, p = 0.3: 792 -> 773 us; W = 16, P = 512, 0.6 M, p =
-          // 0.3: 16.3 -> 15.9; W = 20, P = 336, 0.2 M: 17.7 both; W = 44, P = 352, 1.6 M, fp32: 170.9 -> 174.5. The drift norms alone
-          // read all copies of every chunk and keep the fp32 tree (W = 24, P = 704, 2 M, the four phases: 101 us, with fp64 108).
-          auto squares = [&](int b) {      // of copy b's differences, this lane's eight elements
-            float diff[8], s = 0.0f;
-            minus8<RT>(old[b], xw, diff);
 #pragma unroll
-            for (int x = 0; x < 8; ++x) {
-              const float d = x < nvalid ? diff[x] : 0.0f;
-              s = __fadd_rn(s, __fmul_rn(d, d));
-            }
-            return s;
-          };
-          if constexpr (PH & BCAST) {
-            float sq[4];
+          for (int b = 0; b < 4; ++b) {
+            if (b < nb) {
+              float diff[8], s = 0.0f;
+              minus8<RT>(old[b], xw, diff);
 #pragma unroll
-            for (int b = 0; b < 4; ++b) sq[b] = b < nb ? squares(b) : 0.0f;
-            double tot;
-            int to = 0;                    // the copy whose total this lane adds: the first lane of each segment does
-            if (nb > 2) {
-              tot = warp_sum_multi64<4>(sq, lane);
-              to = lane >> 3;
-            } else if (nb == 2) {
-              const float two[2] = {sq[0], sq[1]};
-              tot = warp_sum_multi64<2>(two, lane);
-              to = lane >> 4;
-            } else {
-              tot = warp_sum64((double)sq[0]);
-            }
-            const int id = to < 2 ? (to ? ids[1] : ids[0]) : (to == 2 ? ids[2] : ids[3]);
-            if ((lane & (nb > 2 ? 7 : nb == 2 ? 15 : 31)) == 0 && to < nb) dsum[warp * kMaxW + id] += tot;
-            __syncwarp();                  // (another lane may add to this copy's sum next time)
-          } else {
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-              if (b < nb) {
-                const float tot = warp_sum(squares(b));
-                if ((ids[b] & 31) == lane) {
-                  if (ids[b] < 32) dacc0 += (double)tot; else dacc1 += (double)tot;
-                }
+              for (int x = 0; x < 8; ++x) {
+                const float d = x < nvalid ? diff[x] : 0.0f;
+                s = __fadd_rn(s, __fmul_rn(d, d));
+              }
+              const float tot = warp_sum(s);
+              if ((ids[b] & 31) == lane) {
+                if (ids[b] < 32) dacc0 += (double)tot; else dacc1 += (double)tot;
               }
             }
           }
@@ -503,10 +437,9 @@ __global__ void __launch_bounds__(kThreads, LOSSY_MIN_BLOCKS) lossy_kernel(const
 
   // ---- per-block drift partials, fixed order ------------------------------------
   if constexpr (PH & DRIFT) {
-    if constexpr (!(PH & BCAST)) {
-      dsum[warp * kMaxW + lane] = dacc0;
-      dsum[warp * kMaxW + lane + 32] = dacc1;
-    }
+    __shared__ double dsum[kWarps * kMaxW];   // per warp and replica
+    dsum[warp * kMaxW + lane] = dacc0;
+    dsum[warp * kMaxW + lane + 32] = dacc1;
     drift_finish(P, dsum, kWarps, P.partials_row0 + blockIdx.x, warp, kWarps, lane);
   }
   if constexpr (TAIL) end_after_previous(P);
