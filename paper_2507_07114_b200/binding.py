@@ -1,9 +1,9 @@
-"""Thin ctypes binding of the C ABI in include/lossy.h (argument marshalling only).
+"""Thin binding of the C ABI in include/lossy.h (argument marshalling only).
 
 Every function has the name of the C entry point it calls; tensors are passed as
-raw device pointers and the current torch CUDA stream as the stream argument. All
-arithmetic runs in the CUDA library. There is no fallback: if the shared library
-is missing, loading raises.
+raw device pointers and the current torch CUDA stream as the stream argument, by
+csrc/marshal.cpp where a step calls it, else by ctypes. All arithmetic runs in the
+CUDA library. There is no fallback: if a shared library is missing, loading raises.
 """
 from __future__ import annotations
 
@@ -47,6 +47,13 @@ class LossyError(RuntimeError):
 
 
 _lib = None
+_native = None         # _marshal.call
+# entry points whose arguments csrc/marshal.cpp marshals, and the kinds of the arguments (there); behind the context
+_NATIVE = {
+    "lossy_packet_sqnorms": "tps", "lossy_aggregate": "utppps", "lossy_step": "uppppps", "lossy_broadcast": "uptps", "drift_norms": "ptpps",
+    "drift_pairwise": "tps", "lossy_fused_step": "utppptpppppps", "lossy_aggregate_alg1": "utpppps", "lossy_fused_step_alg1": "utpppptpppppps",
+    "lossy_closed_loop_grads": "ppttts",
+}
 
 
 def default_library_path() -> str:
@@ -127,6 +134,15 @@ def load_library(path: str | None = None) -> C.CDLL:
     lib.lossy_selftest_shrink_checks.argtypes = [vp, u64]
     lib.lossy_describe_plan.restype = C.c_int
     lib.lossy_describe_plan.argtypes = [vp, C.c_int, C.c_char_p, C.c_size_t]
+    global _native
+    if _native is None:
+        try:
+            from . import _marshal
+        except ImportError as e:
+            raise FileNotFoundError(f"{os.path.join(os.path.dirname(__file__), '_marshal.so')} is missing or does not load ({e}): run "
+                                    "paper_2507_07114_b200.build.build()") from e
+        _native = _marshal.call
+    lib.at = {name: C.cast(getattr(lib, name), vp).value for name in _NATIVE}
     if path == default:
         _lib = lib
     return lib
@@ -140,9 +156,14 @@ def _dt(t: torch.dtype) -> int:
     raise TypeError(f"unsupported element type {t}")
 
 
-# Marshalling is a good part of a call on a small bucket, so it makes no objects that the call does not need: pointers go as
-# integers, a pointer table as the bytes of its entries, and the stream's handle is read without a Stream object around it
-# (3.2 -> 0.4 us; a table of 4: 0.8 -> 0.6 us, of 64: 8.8 -> 5.2 us; all of a fused step of four workers: 16 -> 12 us).
+# What a step calls goes through csrc/marshal.cpp. The rest: pointers as integers, a pointer table as the bytes of its entries, the
+# stream's handle without a Stream object around it.
+def _call(name, ctx, *args):
+    rc = _native(load_library().at[name], _NATIVE[name], ctx, *args)
+    if rc != LOSSY_OK:
+        _check(ctx, rc)
+
+
 def _p(t):
     return None if t is None else t.data_ptr()
 
@@ -195,29 +216,28 @@ def lossy_set_reliable(ctx, reliable):
 
 
 def lossy_packet_sqnorms(ctx, grads, out):
-    _check(ctx, load_library().lossy_packet_sqnorms(ctx, _table(grads), _p(out), _stream()))
+    _call("lossy_packet_sqnorms", ctx, grads, out)
 
 
 def lossy_aggregate(ctx, step, grads, ghat, count=None, recv_bits=None):
-    _check(ctx, load_library().lossy_aggregate(ctx, step, _table(grads), _p(ghat), _p(count), _p(recv_bits),
-                                               _stream()))
+    _call("lossy_aggregate", ctx, step, grads, ghat, count, recv_bits)
 
 
 def lossy_step(ctx, step, ghat, count, master, m=None, v=None):
-    _check(ctx, load_library().lossy_step(ctx, step, _p(ghat), _p(count), _p(master), _p(m), _p(v), _stream()))
+    _call("lossy_step", ctx, step, ghat, count, master, m, v)
 
 
 def lossy_broadcast(ctx, step, master, replicas, stale_bits=None):
-    _check(ctx, load_library().lossy_broadcast(ctx, step, _p(master), _table(replicas), _p(stale_bits), _stream()))
+    _call("lossy_broadcast", ctx, step, master, replicas, stale_bits)
 
 
 def drift_norms(ctx, master, replicas, norms=None, sumsq=None):
-    _check(ctx, load_library().drift_norms(ctx, _p(master), _table(replicas), _p(norms), _p(sumsq), _stream()))
+    _call("drift_norms", ctx, master, replicas, norms, sumsq)
 
 
 def drift_pairwise(ctx, replicas, d2):
     """d2: fp64 device tensor of W*W elements, added to (zero it first)."""
-    _check(ctx, load_library().drift_pairwise(ctx, _table(replicas), _p(d2), _stream()))
+    _call("drift_pairwise", ctx, replicas, d2)
 
 
 def drift_norms_static(*, W, n, packet_elems, replica_dtype, master, replicas, norms=None, sumsq=None, flags=0,
@@ -237,9 +257,7 @@ def drift_norms_static(*, W, n, packet_elems, replica_dtype, master, replicas, n
 
 def lossy_fused_step(ctx, step, grads, master, m, v, replicas, ghat=None, count=None, recv_bits=None,
                      stale_bits=None, norms=None, sumsq=None):
-    _check(ctx, load_library().lossy_fused_step(ctx, step, _table(grads), _p(master), _p(m), _p(v), _table(replicas),
-                                                _p(ghat), _p(count), _p(recv_bits), _p(stale_bits), _p(norms),
-                                                _p(sumsq), _stream()))
+    _call("lossy_fused_step", ctx, step, grads, master, m, v, replicas, ghat, count, recv_bits, stale_bits, norms, sumsq)
 
 
 class lossy_fused_step_prepared:
@@ -253,28 +271,26 @@ class lossy_fused_step_prepared:
                  norms=None, sumsq=None, ghat_prev=None, stream=None):
         lib = load_library()
         self._ctx, self._keep = ctx, (grads, master, m, v, replicas, ghat, count, recv_bits, stale_bits, norms, sumsq, ghat_prev)
-        self._fn = lib.lossy_fused_step if ghat_prev is None else lib.lossy_fused_step_alg1
-        head = (_table(grads),) + (() if ghat_prev is None else (_p(ghat_prev),))
-        self._args = head + (_p(master), _p(m), _p(v), _table(replicas), _p(ghat), _p(count), _p(recv_bits),
-                             _p(stale_bits), _p(norms), _p(sumsq))
-        self._stream = None if stream is None else stream.cuda_stream
+        self._fn = lib.at["lossy_fused_step" if ghat_prev is None else "lossy_fused_step_alg1"]
+        pointers = lambda *ts: tuple(_p(t) or 0 for t in ts)
+        head = (_table(grads),) + (() if ghat_prev is None else pointers(ghat_prev))
+        self._args = (head + pointers(master, m, v) + (_table(replicas),) + pointers(ghat, count, recv_bits, stale_bits, norms, sumsq)
+                      + (() if stream is None else (stream.cuda_stream,)))
+        self._kinds = "u" + "".join("b" if isinstance(a, bytes) else "u" for a in self._args) + ("s" if stream is None else "")
 
     def __call__(self, step):
-        rc = self._fn(self._ctx, step, *self._args, self._stream if self._stream is not None else _stream())
+        rc = _native(self._fn, self._kinds, self._ctx, step, *self._args)
         if rc != LOSSY_OK:
             _check(self._ctx, rc)
 
 
 def lossy_aggregate_alg1(ctx, step, grads, ghat_prev, ghat, count=None, recv_bits=None):
-    _check(ctx, load_library().lossy_aggregate_alg1(ctx, step, _table(grads), _p(ghat_prev), _p(ghat), _p(count),
-                                                    _p(recv_bits), _stream()))
+    _call("lossy_aggregate_alg1", ctx, step, grads, ghat_prev, ghat, count, recv_bits)
 
 
 def lossy_fused_step_alg1(ctx, step, grads, ghat_prev, master, m, v, replicas, ghat=None, count=None,
                           recv_bits=None, stale_bits=None, norms=None, sumsq=None):
-    _check(ctx, load_library().lossy_fused_step_alg1(ctx, step, _table(grads), _p(ghat_prev), _p(master), _p(m),
-                                                     _p(v), _table(replicas), _p(ghat), _p(count), _p(recv_bits),
-                                                     _p(stale_bits), _p(norms), _p(sumsq), _stream()))
+    _call("lossy_fused_step_alg1", ctx, step, grads, ghat_prev, master, m, v, replicas, ghat, count, recv_bits, stale_bits, norms, sumsq)
 
 
 def lossy_fused_step_host(ctx, step, host_grads, dev_grads, master, m, v, replicas, dev_norms, host_norms):
@@ -300,8 +316,7 @@ def lossy_mask_grid(ctx, step, src, dst, packet, out, is_param=False):
 
 
 def lossy_closed_loop_grads(ctx, curv, target, noise, replicas, grads_out):
-    _check(ctx, load_library().lossy_closed_loop_grads(ctx, _p(curv), _p(target), _table(noise), _table(replicas),
-                                                       _table(grads_out), _stream()))
+    _call("lossy_closed_loop_grads", ctx, curv, target, noise, replicas, grads_out)
 
 
 def lossy_device_status(ctx):

@@ -1,14 +1,17 @@
-"""Build the CUDA library in-tree with nvcc for sm_100a (no JIT cache, no torch extension)."""
+"""Build the CUDA library in-tree with nvcc for sm_100a, and the binding's marshalling module (no JIT cache)."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "liblossy_b200.so")
 CHECK_LIB_PATH = os.path.join(PKG_DIR, "liblossy_b200_check.so")   # the debug build: -DLOSSY_DEVCHECK (index checks in the kernels)
+MARSHAL_PATH = os.path.join(PKG_DIR, "_marshal.so")
+MARSHAL_SOURCE = os.path.join(CSRC, "marshal.cpp")
 SOURCES = ["lossy_api.cu", "lossy_noalloc.cu"]
 HEADERS = ["lossy_device.cuh", "lossy_kernels.cuh", "lossy_tma.cuh", "lossy_gather.cuh", "lossy_phase_tma.cuh", "lossy_register.cuh", "lossy_diag.cuh", os.path.join("..", "..", "include", "lossy.h")]
 
@@ -23,15 +26,30 @@ def _stale(lib: str) -> bool:
     if not os.path.exists(lib):
         return True
     t = os.path.getmtime(lib)
-    deps = [os.path.join(CSRC, s) for s in SOURCES + HEADERS] + [os.path.abspath(__file__)]
+    deps = ([MARSHAL_SOURCE] if lib == MARSHAL_PATH else [os.path.join(CSRC, s) for s in SOURCES + HEADERS]) + [os.path.abspath(__file__)]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _marshal_command(out: str) -> list:
+    """g++ on marshal.cpp, against the headers of the Python and the torch that run this."""
+    import torch
+
+    root = os.path.dirname(torch.__file__)
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    include = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+               sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
+    return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI,
+            *["-isystem" + d for d in include], MARSHAL_SOURCE, "-o", out, "-L" + os.path.join(root, "lib"),
+            "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch", "-ltorch_python"]
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile liblossy_b200.so and its debug twin liblossy_b200_check.so next to this file (the two nvcc runs side by
-    side); returns the path of the normal library."""
+    """Compile liblossy_b200.so, its debug twin liblossy_b200_check.so and the binding's _marshal.so next to this file (the
+    compilers side by side); returns the path of the normal library."""
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     jobs = []
+    if force or _stale(MARSHAL_PATH):
+        jobs.append((MARSHAL_PATH, subprocess.Popen(_marshal_command(MARSHAL_PATH + ".tmp"), stdout=subprocess.PIPE, stderr=subprocess.PIPE, text=True)))
     for lib, extra in ((LIB_PATH, []), (CHECK_LIB_PATH, ["-DLOSSY_DEVCHECK=1"])):
         if not force and not _stale(lib):
             continue
@@ -48,7 +66,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         else:
             os.replace(lib + ".tmp", lib)
     if failed:
-        raise RuntimeError("nvcc failed:\n" + "\n".join(failed))
+        raise RuntimeError("build failed:\n" + "\n".join(failed))
     return LIB_PATH
 
 
