@@ -21,16 +21,6 @@ struct SqnormArgs {
   uint32_t W, P, K;
 };
 constexpr int kSqLoads = 4;
-// load8_any for lanes of which many may lie past a short piece: those load nothing (and take no scalar path)
-template <class T>
-__device__ __forceinline__ Vec8<T> load8_some(const void* base, uint64_t e, int nvalid) {
-  if (nvalid > 0) return load8_any<T>(base, e, nvalid);
-  Vec8<T> r;
-#pragma unroll
-  for (int i = 0; i < T::kVecs; ++i) r.q[i] = make_uint4(0u, 0u, 0u, 0u);
-  return r;
-}
-
 template <class GT, bool MANY>
 static __global__ void __launch_bounds__(256) packet_sqnorms_kernel(const __grid_constant__ SqnormArgs A) {
   const int lane = threadIdx.x & 31;
@@ -55,7 +45,7 @@ static __global__ void __launch_bounds__(256) packet_sqnorms_kernel(const __grid
         const uint64_t k = (uint64_t)t * kSqLoads + u;
         const uint64_t e0 = k * A.P, e1 = e0 + A.P < A.n ? e0 + A.P : A.n, e = e0 + (uint64_t)lane * 8;
         nvalid[u] = e >= e1 ? 0 : e1 - e >= 8 ? 8 : (int)(e1 - e);
-        raw[u] = load8_some<GT>(grads, e, nvalid[u]);
+        raw[u] = load8_any<GT>(grads, e, nvalid[u]);
       }
       float s[kSqLoads];
 #pragma unroll
@@ -76,7 +66,7 @@ static __global__ void __launch_bounds__(256) packet_sqnorms_kernel(const __grid
         for (int u = 0; u < kSqLoads; ++u) {
           const uint64_t e = eb + (uint64_t)u * kChunk;
           nvalid[u] = e >= e1 ? 0 : e1 - e >= 8 ? 8 : (int)(e1 - e);
-          raw[u] = load8_some<GT>(grads, e, nvalid[u]);
+          raw[u] = load8_any<GT>(grads, e, nvalid[u]);
         }
 #pragma unroll
         for (int u = 0; u < kSqLoads; ++u) s = add(s, raw[u], nvalid[u]);
