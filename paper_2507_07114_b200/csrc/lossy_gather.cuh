@@ -27,6 +27,8 @@
 // of the copy rate) and the bulk-copy pipeline with part-empty tiles (P = 1472, W = 8, p = 0.1: 1.28 times as fast), in
 // buckets of several tiles per SM. Every wait is bounded as in the other pipelines. No cluster, no multicast.
 #pragma once
+#include <type_traits>
+
 #include "lossy_tma.cuh"
 
 namespace lossy {
@@ -351,9 +353,32 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
         if (phase >= P.P) { phase -= P.P; ++kfirst; }
       }
     };
+    // Bursty loss: lane sp holds the words of its sub-packet's links, loaded a tile ahead. Loaded where they are used they were a round trip
+    // to memory or two per pass of draws, and this warp the step's bottleneck (W = 12, P = 256, p = 0.01, 38 M: 585 -> 469 us; W = 5,
+    // P = 128, 20 M: 257 -> 219). A loop of its own: in one loop for both independent loss paid 1-5 %.
+    // The twin RD builds (two to four workers) keep one loop that loads them: with two W = 3, P = 128, p = 0.3, 23 M without bursts took 169 us
+    // for 161.
+    auto all_tiles = [&](auto known) {
+    constexpr int kLinks = decltype(known)::value;
+    constexpr bool BURSTY = kLinks == kLinksGiven;
+    [[maybe_unused]] uint64_t gin_next = 0, pin_next = 0;
+    [[maybe_unused]] auto links_of = [&](uint32_t k) {      // (k: this lane's sub-packet, maybe behind the tile's last one)
+      if (lane < kSub && k < P.K) {
+        gin_next = P.burst_in[k];
+        pin_next = P.burst_in[(size_t)P.K + k];
+      }
+    };
+    if constexpr (BURSTY) links_of((ANY ? kfirst : blockIdx.x * G.packets_per_tile) + (uint32_t)lane);
     for (uint32_t tile = blockIdx.x; tile < G.num_tiles; tile += gridDim.x, next_tile()) {
       if (!mbar_wait(mempty_bar(slot), par ^ 1u, abort_flag)) break;
       if constexpr (!ANY) kfirst = tile * G.packets_per_tile;
+      uint64_t gin_l = 0, pin_l = 0;
+      if constexpr (BURSTY) {
+        gin_l = gin_next;
+        pin_l = pin_next;
+        if (tile + gridDim.x < G.num_tiles)
+          links_of((ANY ? kfirst + k_step + (phase + phase_step >= P.P ? 1u : 0u) : kfirst + gridDim.x * G.packets_per_tile) + (uint32_t)lane);
+      }
       // (packets that divide the tile: from the packets' numbers, as here; e0 and len from the tile's number cost a step of
       // W = 4, P = 512, p = 0.05 3 %, one of P = 128 1-2 %)
       uint64_t e0;
@@ -403,7 +428,12 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
           const uint32_t sp_l = q0 + ((uint32_t)lane >> lgWp), i_l = (uint32_t)lane & (Wp - 1u);
           const uint32_t k_l = kfirst + (sp_l < npk ? sp_l : 0u);
           const uint32_t j_l = (P.k0 + k_l) / P.pps;
-          const BatchDraws d = batch_draws<AGG | BCAST>(P, k_l, j_l, i_l, sp_l < npk && i_l < W);
+          uint64_t gin = 0, pin = 0;
+          if constexpr (BURSTY) {
+            gin = __shfl_sync(0xFFFFFFFFu, gin_l, (int)(sp_l < npk ? sp_l : 0u));
+            pin = __shfl_sync(0xFFFFFFFFu, pin_l, (int)(sp_l < npk ? sp_l : 0u));
+          }
+          const BatchDraws d = batch_draws<AGG | BCAST, kLinks>(P, k_l, j_l, i_l, sp_l < npk && i_l < W, gin, pin);
           uint64_t st_l = 0;                                 // the stale set of this lane's own sub-packet
           for (uint32_t x = 0; x < Bp && q0 + x < npk; ++x) {
             uint64_t r, st, gbad, pbad;
@@ -418,7 +448,12 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
         for (uint32_t sp = 0; sp < npk; ++sp) {
           uint64_t r, st, gbad, pbad;
           const uint32_t j_sp = (P.k0 + kfirst + sp) / P.pps;
-          packet_masks<AGG | BCAST>(P, kfirst + sp, j_sp, lane, r, st, gbad, pbad);
+          uint64_t gin = 0, pin = 0;
+          if constexpr (BURSTY) {
+            gin = __shfl_sync(0xFFFFFFFFu, gin_l, (int)sp);
+            pin = __shfl_sync(0xFFFFFFFFu, pin_l, (int)sp);
+          }
+          packet_masks<AGG | BCAST, kLinks>(P, kfirst + sp, j_sp, lane, r, st, gbad, pbad, gin, pin);
           if (lane == 0) report(sp, j_sp, r, st, gbad, pbad);
           if (prefetch_on) {
             for (uint32_t i = lane; i < W; i += 32)
@@ -441,6 +476,10 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
       if (lane == 0) mbar_arrive(mfull_bar(slot));
       if (++slot == kGatherRing) { slot = 0; par ^= 1u; }
     }
+    };
+    if constexpr (RD && CW < 16) all_tiles(std::integral_constant<int, kLinksLook>{});
+    else if (P.burst_in) all_tiles(std::integral_constant<int, kLinksGiven>{});
+    else all_tiles(std::integral_constant<int, kLinksNone>{});
   } else if (warp > CW && warp <= CW + kNP) {
     // ================================ gather warps ================================
     const uint32_t pw = (uint32_t)(warp - CW - 1);          // which gather warp

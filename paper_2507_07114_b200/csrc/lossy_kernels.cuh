@@ -159,13 +159,16 @@ __device__ __forceinline__ void drift_finish(const Params& P, const double* sums
 // Independent loss: one threshold compare per link. Bursty loss (P.burst_in set): each link is a two-state
 // chain on the same hash value, bad_t = bad_{t-1} ? (u < Tstay) : (u < Tenter), lost iff bad; the new states
 // come back in gbad / pbad for the one caller that stores them.
-template <int PH>
+// LINKS says what is known of that: nothing (the words are loaded here where they are needed), or that the loss is bursty and gin and
+// pin are the words, or that it is independent.
+enum Links : int { kLinksLook = 0, kLinksGiven = 1, kLinksNone = 2 };
+template <int PH, int LINKS = kLinksLook>
 __device__ __forceinline__ void packet_masks(const Params& P, uint32_t k, uint32_t j, int lane, uint64_t& recv,
-                                             uint64_t& stale, uint64_t& gbad, uint64_t& pbad) {
+                                             uint64_t& stale, uint64_t& gbad, uint64_t& pbad, uint64_t gin_given = 0, uint64_t pin_given = 0) {
   const uint32_t W = P.W;
   const uint64_t pkey = packet_key_of(P.step_key, P.packet_base + k);
   const uint32_t i0 = lane, i1 = lane + 32;
-  const bool bursty = P.burst_in != nullptr;
+  const bool bursty = LINKS == kLinksGiven || (LINKS == kLinksLook && P.burst_in != nullptr);
   gbad = 0;
   pbad = 0;
   if constexpr (PH & AGG) {
@@ -173,7 +176,7 @@ __device__ __forceinline__ void packet_masks(const Params& P, uint32_t k, uint32
     // hash) keeps or drops the packet's whole aggregate; otherwise one draw per contributing worker.
     const bool alg1 = P.ghat_prev != nullptr;
     const uint32_t src0 = alg1 ? j : i0, src1 = alg1 ? j : i1;
-    const uint64_t gin = bursty ? P.burst_in[k] : 0ull;
+    const uint64_t gin = LINKS == kLinksGiven ? gin_given : bursty ? P.burst_in[k] : 0ull;
     const uint32_t u0 = pair_hash(pkey, src0, j);
     const bool was0 = (gin >> (alg1 ? 0u : i0)) & 1ull;
     bool lost0 = bursty ? (was0 ? u0 < P.Tstay : u0 < P.Tenter) : u0 < P.Tg;
@@ -198,7 +201,7 @@ __device__ __forceinline__ void packet_masks(const Params& P, uint32_t k, uint32
     }
   }
   if constexpr (PH & BCAST) {
-    const uint64_t pin = bursty ? P.burst_in[(size_t)P.K + k] : 0ull;
+    const uint64_t pin = LINKS == kLinksGiven ? pin_given : bursty ? P.burst_in[(size_t)P.K + k] : 0ull;
     const uint32_t u0 = pair_hash(pkey, j, i0);
     const bool was0 = (pin >> i0) & 1ull;
     const bool d0 = i0 < W && i0 != j && (bursty ? (was0 ? u0 < P.Tstay : u0 < P.Tenter) : u0 < P.Tp);
@@ -230,13 +233,13 @@ struct BatchDraws {
   uint32_t grad_lost;   // bit = gradient link in its lossy state (before the reliable channel)
   uint32_t bcast_lost;  // bit = replica missed the broadcast (before the reliable channel)
 };
-template <int PH>
-__device__ __forceinline__ BatchDraws batch_draws(const Params& P, uint32_t k, uint32_t j, uint32_t i, bool valid) {
+template <int PH, int LINKS = kLinksLook>
+__device__ __forceinline__ BatchDraws batch_draws(const Params& P, uint32_t k, uint32_t j, uint32_t i, bool valid, uint64_t gin = 0, uint64_t pin = 0) {
   const uint64_t pkey = packet_key_of(P.step_key, P.packet_base + k);
-  const bool bursty = P.burst_in != nullptr;
+  const bool bursty = LINKS == kLinksGiven || (LINKS == kLinksLook && P.burst_in != nullptr);
   BatchDraws d = {0u, 0u, 0u};
   if constexpr (PH & AGG) {
-    const bool was = bursty && ((P.burst_in[k] >> i) & 1ull);
+    const bool was = bursty && (((LINKS == kLinksGiven ? gin : P.burst_in[k]) >> i) & 1ull);
     const uint32_t u = pair_hash(pkey, i, j);
     bool lost = bursty ? (was ? u < P.Tstay : u < P.Tenter) : u < P.Tg;
     if ((P.flags & 1u) && i == j) lost = false;
@@ -244,7 +247,7 @@ __device__ __forceinline__ BatchDraws batch_draws(const Params& P, uint32_t k, u
     d.grad_lost = __ballot_sync(0xFFFFFFFFu, valid && lost);
   }
   if constexpr (PH & BCAST) {
-    const bool was = bursty && ((P.burst_in[(size_t)P.K + k] >> i) & 1ull);
+    const bool was = bursty && (((LINKS == kLinksGiven ? pin : P.burst_in[(size_t)P.K + k]) >> i) & 1ull);
     const uint32_t u = pair_hash(pkey, j, i);
     const bool lost = i != j && (bursty ? (was ? u < P.Tstay : u < P.Tenter) : u < P.Tp);
     d.bcast_lost = __ballot_sync(0xFFFFFFFFu, valid && lost);
