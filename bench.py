@@ -867,7 +867,7 @@ def main():
                          "traffic": traffic, "traffic_source": traffic_note,
                          "frac_of_traffic": (traffic / (avg_launch_ms * 1e-3) / 1e9 / peak) if traffic else None,
                          "peak_source": peak_src + " (MEASURED_PEAKS.json hbm_gbs)" if peak_src == "measured"
-                         else peak_src, "kernel": ("lossy_kernel<AGG|STEP|BCAST|DRIFT>" if plan.startswith("register") else "lossy_fused_tma_kernel")
+                         else peak_src, "kernel": ("lossy_step_kernel" if plan.startswith("register") else "lossy_fused_tma_kernel")
                          + " (drift norms finalised by its last block)", "build": plan,
                          "algorithmic_bytes_per_launch": B,
                          "avg_launch_ms": avg_launch_ms, "min_launch_ms": min(per_launch_ms)},

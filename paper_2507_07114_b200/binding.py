@@ -263,7 +263,7 @@ def lossy_fused_step(ctx, step, grads, master, m, v, replicas, ghat=None, count=
 class lossy_fused_step_prepared:
     """lossy_fused_step (or, with ghat_prev, lossy_fused_step_alg1) with its arguments marshalled once: the pointer
     tables and handles are built here, a call `prepared(step)` is one foreign call. For buckets so small that a
-    step is bound by launch overhead (a 40 MB bucket: 19 -> 12 us per step); the tensors are kept alive by this
+    step is bound by the host; the tensors are kept alive by this
     object and must not be reallocated while it is used. `stream`: a torch stream whose handle is read once, or
     None to read the current stream at every call."""
 

@@ -354,8 +354,9 @@ __global__ void __launch_bounds__(GatherShape<CW, RD>::kThreads, GatherShape<CW,
       }
     };
     // Bursty loss: lane sp holds the words of its sub-packet's links, loaded a tile ahead. Loaded where they are used they were a round trip
-    // to memory or two per pass of draws, and this warp the step's bottleneck (W = 12, P = 256, p = 0.01, 38 M: 585 -> 469 us; W = 5,
-    // P = 128, 20 M: 257 -> 219). A loop of its own: in one loop for both independent loss paid 1-5 %.
+    // to memory or two per pass of draws, and this warp the step's bottleneck (W = 12, P = 256, p = 0.01, 38 M: 586 -> 432 us; W = 5,
+    // P = 128, 20 M: 257 -> 212). A loop of its own: in one loop for both independent loss paid 1-5 %, in two it gains up to 12 % where
+    // this warp is the busiest (W = 10, P = 128, 20 M: 298 -> 264 us).
     // The twin RD builds (two to four workers) keep one loop that loads them: with two W = 3, P = 128, p = 0.3, 23 M without bursts took 169 us
     // for 161.
     auto all_tiles = [&](auto known) {
