@@ -108,9 +108,11 @@ int check_replicas(lossy_ctx* ctx, const void* const* tab) {
 // 9.4 us a step; with a short last packet on a launch of its own (n = 262 184): 20.0 -> 11.4.
 // early = false, an ordinary launch: for kernels that load through L1 and run long. A block that begins early gets what
 // shared memory the kernel ahead has left its SM, after a gather pipeline 28 KB of L1 (closed-loop gradients of 58 M elements
-// behind it: 690 -> 755 us for the pair; packet norms behind the pairwise drift, W = 9, n = 4.6 M: 92 -> 97 us). On small buckets they
-// begin early too (pairwise drift and packet norms, W = 6, 250 k: 16.0 -> 12.3 us; W = 9, 82 k: 14.6 -> 12.3; closed loop, W = 10, 96 k:
-// 16.4 -> 14.8; with a fourth block per SM W = 16, 1 M: 42.2 -> 40.5, but W = 8, 1.2 M, behind a gather pipeline: 34.7 -> 35.9).
+// behind it: 690 -> 755 us for the pair; packet norms behind the pairwise drift, W = 9, n = 4.6 M: 92 -> 97 us). On small buckets packet
+// norms and the closed loop's gradients begin early too (closed loop, W = 10, 96 k: 16.4 -> 14.8 us; with a fourth block per SM W = 16, 1 M:
+// 42.2 -> 40.5, but W = 8, 1.2 M, behind a gather pipeline: 34.7 -> 35.9). The pairwise drift does not: its set kernel loads through the
+// read-only path, which must not run beside the writes of a step ahead, and there is nothing to gain (850 small buckets, behind the memset
+// of the matrix that the call adds to: 0.97 to 1.00 of the ordinary launch's speed).
 // a call's one launch: its blocks' rows are all (two launches: the caller has counted them ahead)
 void rows_of_call(Params& P, uint32_t blocks) { if (P.total_rows == 0u) P.total_rows = blocks; }
 
@@ -963,7 +965,7 @@ cudaError_t launch_pairwise(lossy_ctx* ctx, PairwiseArgs<ELIDE>& A, cudaStream_t
   if (chunks < (uint64_t)ctx->num_sms * warps) warps = (uint32_t)((chunks + ctx->num_sms - 1) / ctx->num_sms);
   uint64_t blocks = (chunks + warps - 1) / warps;
   if (blocks > (uint64_t)ctx->num_sms) blocks = ctx->num_sms;
-  return launch_after(SMALL, kern, (uint32_t)blocks, warps * 32u, warps * wb, s, A);
+  return launch_after(false, kern, (uint32_t)blocks, warps * 32u, warps * wb, s, A);
 }
 
 }  // namespace
@@ -1284,7 +1286,7 @@ int drift_pairwise(lossy_ctx* ctx, const void* const* replicas, double* d2, void
     if (c.W >= 2u && c.W <= 8u && (small || (c.W <= 4u && !bf16))) {
       const uint64_t cap = (uint64_t)ctx->num_sms * 3u;
       const uint32_t blocks = (uint32_t)((chunks + 3) / 4 < cap ? (chunks + 3) / 4 : cap);
-      return launch_after(small, bf16 ? (c.W <= 4u ? drift_pairwise_few_kernel<BF16, E, 4> : drift_pairwise_few_kernel<BF16, E, 8>)
+      return launch_after(false, bf16 ? (c.W <= 4u ? drift_pairwise_few_kernel<BF16, E, 4> : drift_pairwise_few_kernel<BF16, E, 8>)
                                : (c.W <= 4u ? drift_pairwise_few_kernel<F32, E, 4> : drift_pairwise_few_kernel<F32, E, 8>), blocks, 128, 0, s, A);
     }
     auto pick = [&](auto set, auto small) {
