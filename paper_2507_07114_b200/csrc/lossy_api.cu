@@ -756,6 +756,12 @@ int launch_step(lossy_ctx* ctx, Params& P, cudaStream_t s, uint32_t* blocks_out)
     warps = (tasks + blocks - 1) / blocks;
     const uint32_t rounds = (warps + kMost - 1) / kMost;
     warps = (warps + rounds - 1) / rounds;
+    // The end of the drift norms takes two replicas per warp and turn, each turn a round trip to L2 or more: warps for four turns at W = 64
+    // and for one up to 16, also where there are no chunks for them. (3000 random steps of a thousand to 40 thousand elements, W = 2-4, 5-8, 9-16,
+    // 17-32, 33-64: without them 1.10, 1.28, 1.54, 1.76 and 2.1 times as long under 9 thousand elements, 1.0, 1.02, 1.1, 1.1 and 1.17 from 19
+    // thousand on; W = 50, 7 thousand: 27.3 -> 12.5 us. Four warps 14.2, 16 11.8.)
+    const uint32_t enough = P.W < 16u ? (P.W + 1u) / 2u : 8u;
+    if (DRIFTK && warps < enough) warps = enough;
   }
   *blocks_out = blocks;
   if (ctx->plan_only) return LOSSY_OK;
