@@ -108,11 +108,11 @@ int check_replicas(lossy_ctx* ctx, const void* const* tab) {
 // 9.4 us a step; with a short last packet on a launch of its own (n = 262 184): 20.0 -> 11.4.
 // early = false, an ordinary launch: for kernels that load through L1 and run long. A block that begins early gets what
 // shared memory the kernel ahead has left its SM, after a gather pipeline 28 KB of L1 (closed-loop gradients of 58 M elements
-// behind it: 690 -> 755 us for the pair; packet norms behind the pairwise drift, W = 9, n = 4.6 M: 92 -> 97 us). On small buckets packet
-// norms and the closed loop's gradients begin early too (closed loop, W = 10, 96 k: 16.4 -> 14.8 us; with a fourth block per SM W = 16, 1 M:
-// 42.2 -> 40.5, but W = 8, 1.2 M, behind a gather pipeline: 34.7 -> 35.9). The pairwise drift does not: its set kernel loads through the
-// read-only path, which must not run beside the writes of a step ahead, and there is nothing to gain (850 small buckets, behind the memset
-// of the matrix that the call adds to: 0.97 to 1.00 of the ordinary launch's speed).
+// behind it: 690 -> 755 us for the pair; packet norms behind the pairwise drift, W = 9, n = 4.6 M: 92 -> 97 us). On small buckets the
+// closed loop's gradients begin early too, and packet norms of very few blocks (closed loop, W = 10, 96 k: 16.4 -> 14.8 us; with a fourth
+// block per SM W = 16, 1 M: 42.2 -> 40.5, but W = 8, 1.2 M, behind a gather pipeline: 34.7 -> 35.9). The pairwise drift does not: its set
+// kernel loads through the read-only path, which must not run beside the writes of a step ahead, and there is nothing to gain (850 small
+// buckets, behind the memset of the matrix that the call adds to: 0.97 to 1.00 of the ordinary launch's speed).
 // a call's one launch: its blocks' rows are all (two launches: the caller has counted them ahead)
 void rows_of_call(Params& P, uint32_t blocks) { if (P.total_rows == 0u) P.total_rows = blocks; }
 
@@ -1083,8 +1083,11 @@ int lossy_packet_sqnorms(lossy_ctx* ctx, const void* const* grads, float* out, v
   const dim3 grid((uint32_t)blocks, A.W);
   cudaStream_t s = (cudaStream_t)stream;
   const bool gb = ctx->cfg.grad_dtype == LOSSY_BF16;
-  // (early where its blocks are resident at once)
-  const cudaError_t e = launch_after(blocks * A.W <= (uint64_t)ctx->num_sms * 4, gb ? (many ? packet_sqnorms_kernel<BF16, true> : packet_sqnorms_kernel<BF16, false>)
+  // Early only with a handful of blocks. Blocks that begin early all go to the SMs that the kernel ahead leaves first, eight to an SM, and
+  // read at those few SMs' rate: W = 6, P = 6736, 0.5 M elements, 60 blocks, behind the pairwise drift: 12.5 us as an ordinary launch, 25.1
+  // early. 900 random buckets, ordinary over early: up to 15 blocks 1.04 to 1.10 (packets of 4096 and more 0.86 to 1.1), 16 to 31
+  // 0.98 to 1.07 (0.68 at the least), 32 to 127 0.68 to 1.02, 128 and more 0.76 to 0.98.
+  const cudaError_t e = launch_after(blocks * A.W < 16u, gb ? (many ? packet_sqnorms_kernel<BF16, true> : packet_sqnorms_kernel<BF16, false>)
                                         : (many ? packet_sqnorms_kernel<F32, true> : packet_sqnorms_kernel<F32, false>), grid, 256, 0, s, A);
   if (e != cudaSuccess) return fail_cuda(ctx, "packet norm launch", e);
   ctx->launches++;

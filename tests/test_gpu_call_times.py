@@ -50,3 +50,21 @@ def test_a_step_of_few_chunks_is_no_slower_than_one_of_many(W, P):
     many, many_grads = make(W, 36_864, P, flags=L.LOSSY_REGISTER_PATH)
     a, b = graph_times(lambda: few.step_fused(1, few_grads, outputs=False), lambda: many.step_fused(1, many_grads, outputs=False))
     assert a <= 1.15 * b, (a, b)
+
+
+@pytest.mark.parametrize("W,n,P", [(6, 497_803, 6736), (2, 2_126_753, 8192)])
+def test_packet_norms_right_behind_a_kernel(W, n, P):
+    """A memset in front makes any kernel's launch an ordinary one. Blocks that begin while the pairwise drift still runs share the few SMs
+    that it leaves first: with up to 592 of them 25 us for 12.5, memset included."""
+    run, grads = make(W, n, P)
+    d2, out, word = torch.zeros(W * W, dtype=torch.float64, device="cuda"), torch.empty(W * -(-n // P), device="cuda"), torch.zeros(1, device="cuda")
+
+    def diagnostics(between):
+        d2.zero_()
+        L.drift_pairwise(run.ctx, run.replicas, d2)
+        if between:
+            word.zero_()
+        L.lossy_packet_sqnorms(run.ctx, grads, out)
+
+    a, b = graph_times(lambda: diagnostics(False), lambda: diagnostics(True))
+    assert a <= 1.15 * b, (a, b)
