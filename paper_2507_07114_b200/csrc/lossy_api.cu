@@ -109,9 +109,8 @@ int check_replicas(lossy_ctx* ctx, const void* const* tab) {
 // early = false, an ordinary launch: for kernels that load through L1 and run long. A block that begins early gets what
 // shared memory the kernel ahead has left its SM, after a gather pipeline 28 KB of L1 (closed-loop gradients of 58 M elements
 // behind it: 690 -> 755 us for the pair; packet norms behind the pairwise drift, W = 9, n = 4.6 M: 92 -> 97 us). On small buckets the
-// closed loop's gradients begin early too, and packet norms of very few blocks (closed loop, W = 10, 96 k: 16.4 -> 14.8 us; with a fourth
-// block per SM W = 16, 1 M: 42.2 -> 40.5, but W = 8, 1.2 M, behind a gather pipeline: 34.7 -> 35.9). The pairwise drift does not: its set
-// kernel loads through the read-only path, which must not run beside the writes of a step ahead, and there is nothing to gain (850 small
+// closed loop's gradients begin early too, and packet norms of very few blocks (closed loop, W = 10, 96 k: 16.4 -> 14.8 us; lines
+// at the calls). The pairwise drift does not: its set kernel loads through the read-only path, which must not run beside the writes of a step ahead, and there is nothing to gain (850 small
 // buckets, behind the memset of the matrix that the call adds to: 0.97 to 1.00 of the ordinary launch's speed).
 // a call's one launch: its blocks' rows are all (two launches: the caller has counted them ahead)
 void rows_of_call(Params& P, uint32_t blocks) { if (P.total_rows == 0u) P.total_rows = blocks; }
@@ -1339,8 +1338,11 @@ int lossy_closed_loop_grads(lossy_ctx* ctx, const float* curv, const float* targ
   if (blocks > cap) blocks = cap;
   const bool gb = ctx->cfg.grad_dtype == LOSSY_BF16, rb = ctx->cfg.replica_dtype == LOSSY_BF16;
   cudaStream_t s = (cudaStream_t)stream;
-  // (early up to three blocks per SM)
-  const cudaError_t e = launch_after(nvec <= 256u * (uint64_t)ctx->num_sms * 3, gb ? (rb ? closed_loop_grads_kernel<BF16, BF16> : closed_loop_grads_kernel<BF16, F32>)
+  // Early up to 64 blocks, and with two or three workers up to three blocks per SM. Beyond, the blocks crowd the SMs that come free first, as
+  // the packet norms' do. 2000 random buckets, ordinary over early: up to 64 blocks 1.01 to 1.06; from there on W = 2-3 1.02 to 1.03, W = 4-7
+  // 1.00 to 1.02 (0.84 at the least), W = 8-15 0.98 to 0.995 (0.82), W = 16-31 0.96 to 0.99 (0.80), more 0.98 (0.79: W = 59, 0.3 M, fp32,
+  // with the step behind it: 95.4 us, early 120.5).
+  const cudaError_t e = launch_after(blocks <= 64u || (A.W <= 3u && blocks <= (uint64_t)ctx->num_sms * 3), gb ? (rb ? closed_loop_grads_kernel<BF16, BF16> : closed_loop_grads_kernel<BF16, F32>)
                                         : (rb ? closed_loop_grads_kernel<F32, BF16> : closed_loop_grads_kernel<F32, F32>), (uint32_t)blocks, 256, 0, s, A);
   if (e != cudaSuccess) return fail_cuda(ctx, "closed-loop gradient launch", e);
   ctx->launches++;
