@@ -708,8 +708,13 @@ int launch_register(lossy_ctx* ctx, Params& P, cudaStream_t s, uint32_t* blocks_
   if (blocks_out) *blocks_out = blocks;
   if (ctx->plan_only) return LOSSY_OK;
   rows_of_call(P, blocks);
-  // (early where the launch is a good part of the call: up to a few chunks per warp, or the short last packet)
-  e = launch_after(need <= 4u * blocks, kern, blocks, kThreads, 0, s, P);
+  // Early where the launch is a good part of the call: up to a few chunks per warp, or the short last packet; a broadcast up to 64 blocks.
+  // Its blocks need so few registers that they crowd the SMs that come free first, as the packet norms' do. (780 random buckets of
+  // packets under 1024 elements, the four phases, early up to 64 blocks over early up to a few chunks per warp: 1.00 to 1.02 under 130
+  // thousand elements, 1.02 to 1.10 up to 4 M; W = 41, P = 512, 374 k, fp32 replicas: 73 -> 63 us; W = 63, P = 256, 737 k: 203 -> 157.
+  // The other phases so as well: no gain, 0.96 at 130 thousand.)
+  const bool crowds = PH == BCAST && !TAIL && blocks > 64u;
+  e = launch_after(need <= 4u * blocks && !crowds, kern, blocks, kThreads, 0, s, P);
   if (e != cudaSuccess) return fail_cuda(ctx, "kernel launch", e);
   ctx->launches++;
   return LOSSY_OK;

@@ -85,3 +85,22 @@ def test_closed_loop_gradients_right_behind_a_step(W, n, P):
 
     a, b = graph_times(lambda: step(False), lambda: step(True))
     assert a <= 1.08 * b, (a, b)
+
+
+@pytest.mark.parametrize("W,n,P", [(41, 374_272, 512), (63, 737_394, 256)])
+def test_a_broadcast_right_behind_the_optimizer(W, n, P):
+    """The same for the broadcast, of packets that no pipeline takes: with 183 blocks and 361 begun early the four phases took 73 us for 63
+    and 203 for 157."""
+    run, grads = make(W, n, P, 0.0 if P == 512 else 0.01, "bf16", "f32")
+    word = torch.zeros(1, device="cuda")
+
+    def step(between):
+        L.lossy_aggregate(run.ctx, 1, grads, run.ghat)
+        L.lossy_step(run.ctx, 1, run.ghat, None, run.master, run.m, run.v)
+        if between:
+            word.zero_()
+        L.lossy_broadcast(run.ctx, 1, run.master, run.replicas)
+        L.drift_norms(run.ctx, run.master, run.replicas, run.norms)
+
+    a, b = graph_times(lambda: step(False), lambda: step(True))
+    assert a <= 1.05 * b, (a, b)
