@@ -256,13 +256,18 @@ __device__ __forceinline__ Vec8<T> load8_tail(const void* base, uint64_t e, int 
   }
   return r;
 }
+// Accesses of a lane with nvalid of its eight elements. `tail`: the bucket's end may fall into this lane or another one of its warp (best
+// the same for the whole warp), whose elements are then taken one by one. Where it does not, a lane behind a short packet's end skips the access
+// (the four single phases, W = 38, P = 128, 33 M: 3138 -> 2452 us; W = 6, P = 736, 20 M: 322 -> 302); where it does, such a lane runs along
+// beside that one: a third way through every access made broadcasts of buckets that end inside eight elements a third longer (W = 60,
+// 75 k: 6.8 -> 9.0 us).
 template <class T>
-__device__ __forceinline__ void store8(void* base, uint64_t e, const Vec8<T>& v, int nvalid) {
+__device__ __forceinline__ void store8(void* base, uint64_t e, const Vec8<T>& v, int nvalid, bool tail) {
   typename T::raw* p = reinterpret_cast<typename T::raw*>(base) + e;
   if (nvalid == 8) {
 #pragma unroll
     for (int i = 0; i < T::kVecs; ++i) st_stream(reinterpret_cast<uint4*>(p) + i, v.q[i]);
-  } else if (nvalid > 0) {
+  } else if (tail) {
     const uint32_t* w = reinterpret_cast<const uint32_t*>(&v.q[0]);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
@@ -274,11 +279,9 @@ __device__ __forceinline__ void store8(void* base, uint64_t e, const Vec8<T>& v,
   }
 }
 template <class T>
-__device__ __forceinline__ Vec8<T> load8_any(const void* base, uint64_t e, int nvalid) {
+__device__ __forceinline__ Vec8<T> load8_any(const void* base, uint64_t e, int nvalid, bool tail) {
   if (nvalid == 8) return load8<T>(base, e);
-  if (nvalid > 0) return load8_tail<T>(base, e, nvalid);
-  // a lane behind a short packet's end: nothing, and not element by element (the four single phases, W = 38, P = 128, 33 M: 3138 -> 2452
-  // us; W = 6, P = 736, 20 M: 322 -> 302)
+  if (tail) return load8_tail<T>(base, e, nvalid);
   Vec8<T> r;
 #pragma unroll
   for (int i = 0; i < T::kVecs; ++i) r.q[i] = make_uint4(0u, 0u, 0u, 0u);

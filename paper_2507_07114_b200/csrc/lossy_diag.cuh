@@ -45,7 +45,7 @@ static __global__ void __launch_bounds__(256) packet_sqnorms_kernel(const __grid
         const uint64_t k = (uint64_t)t * kSqLoads + u;
         const uint64_t e0 = k * A.P, e1 = e0 + A.P < A.n ? e0 + A.P : A.n, e = e0 + (uint64_t)lane * 8;
         nvalid[u] = e >= e1 ? 0 : e1 - e >= 8 ? 8 : (int)(e1 - e);
-        raw[u] = load8_any<GT>(grads, e, nvalid[u]);
+        raw[u] = load8_any<GT>(grads, e, nvalid[u], nvalid[u] > 0);
       }
       float s[kSqLoads];
 #pragma unroll
@@ -66,7 +66,7 @@ static __global__ void __launch_bounds__(256) packet_sqnorms_kernel(const __grid
         for (int u = 0; u < kSqLoads; ++u) {
           const uint64_t e = eb + (uint64_t)u * kChunk;
           nvalid[u] = e >= e1 ? 0 : e1 - e >= 8 ? 8 : (int)(e1 - e);
-          raw[u] = load8_any<GT>(grads, e, nvalid[u]);
+          raw[u] = load8_any<GT>(grads, e, nvalid[u], nvalid[u] > 0);
         }
 #pragma unroll
         for (int u = 0; u < kSqLoads; ++u) s = add(s, raw[u], nvalid[u]);

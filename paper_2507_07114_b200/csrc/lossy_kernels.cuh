@@ -299,6 +299,7 @@ __global__ void __launch_bounds__(kThreads, LOSSY_MIN_BLOCKS) lossy_kernel(const
     const uint64_t e = (uint64_t)k * P.P + in_pkt;
     int nvalid = 0;
     if (in_pkt < P.P && e < P.n) nvalid = (P.n - e >= 8) ? 8 : (int)(P.n - e);
+    const bool tail = __any_sync(0xFFFFFFFFu, (nvalid & 7) != 0);   // the bucket ends inside a lane of this chunk
     if constexpr (kDevCheck) {   // debug build: the chunk's range, in the slab and in every replica
       const uint64_t c0 = (uint64_t)k * P.P + (uint64_t)c * kChunk;
       const uint64_t in_packet = P.P - c * kChunk < (uint32_t)kChunk ? P.P - c * kChunk : (uint32_t)kChunk;   // a chunk ends with its packet
@@ -328,10 +329,10 @@ __global__ void __launch_bounds__(kThreads, LOSSY_MIN_BLOCKS) lossy_kernel(const
 
     // ---- optimizer state: issue these loads before the gradient loop ---------
     Vec8<F32> rth, rm, rv;
-    if constexpr (PH & (STEP | BCAST | DRIFT)) rth = load8_any<F32>(P.master, e, nvalid);
+    if constexpr (PH & (STEP | BCAST | DRIFT)) rth = load8_any<F32>(P.master, e, nvalid, tail);
     if constexpr ((PH & STEP) && OPT == 1) {
-      rm = load8_any<F32>(P.m, e, nvalid);
-      rv = load8_any<F32>(P.v, e, nvalid);
+      rm = load8_any<F32>(P.m, e, nvalid, tail);
+      rv = load8_any<F32>(P.v, e, nvalid, tail);
     }
 
     // ---- (2) unbiased aggregate: masked sum in ascending worker order / count --
@@ -345,7 +346,7 @@ __global__ void __launch_bounds__(kThreads, LOSSY_MIN_BLOCKS) lossy_kernel(const
         Vec8<GT> raw[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u)
-          if ((bits >> u) & 1u) raw[u] = load8_any<GT>(P.grads[g0 + u], e, nvalid);
+          if ((bits >> u) & 1u) raw[u] = load8_any<GT>(P.grads[g0 + u], e, nvalid, tail);
 #pragma unroll
         for (int u = 0; u < 8; ++u)
           if ((bits >> u) & 1u) add8<GT>(raw[u], g);
@@ -354,18 +355,18 @@ __global__ void __launch_bounds__(kThreads, LOSSY_MIN_BLOCKS) lossy_kernel(const
       if (P.ghat_prev) {
         // Algorithm 1: a dropped packet falls back to the saved aggregate, a surviving one is saved
         if (cnt == 0) {
-          const Vec8<F32> pv = load8_any<F32>(P.ghat_prev, e, nvalid);
+          const Vec8<F32> pv = load8_any<F32>(P.ghat_prev, e, nvalid, tail);
           widen<F32>(pv, g);
         } else {
-          store8<F32>(P.ghat_prev, e, narrow<F32>(g), nvalid);
+          store8<F32>(P.ghat_prev, e, narrow<F32>(g), nvalid, tail);
         }
       }
       if (P.ghat) {
         Vec8<F32> o = narrow<F32>(g);
-        store8<F32>(P.ghat, e, o, nvalid);
+        store8<F32>(P.ghat, e, o, nvalid, tail);
       }
     } else if constexpr (PH & STEP) {
-      Vec8<F32> r = load8_any<F32>(P.ghat, e, nvalid);
+      Vec8<F32> r = load8_any<F32>(P.ghat, e, nvalid, tail);
       widen<F32>(r, g);
       cnt = (P.flags & 2u) ? (uint32_t)P.count_in[k] : 1u;
     }
@@ -381,10 +382,10 @@ __global__ void __launch_bounds__(kThreads, LOSSY_MIN_BLOCKS) lossy_kernel(const
           widen<F32>(rv, v);
         }
         optimizer8<OPT>(P, g, th, m, v);
-        store8<F32>(P.master, e, narrow<F32>(th), nvalid);
+        store8<F32>(P.master, e, narrow<F32>(th), nvalid, tail);
         if constexpr (OPT == 1) {
-          store8<F32>(P.m, e, narrow<F32>(m), nvalid);
-          store8<F32>(P.v, e, narrow<F32>(v), nvalid);
+          store8<F32>(P.m, e, narrow<F32>(m), nvalid, tail);
+          store8<F32>(P.v, e, narrow<F32>(v), nvalid, tail);
         }
       }
     }
@@ -398,7 +399,7 @@ __global__ void __launch_bounds__(kThreads, LOSSY_MIN_BLOCKS) lossy_kernel(const
       if constexpr (PH & BCAST) {
         const uint64_t keep = stale | own;
         for (uint32_t i = 0; i < W; ++i)
-          if (!((keep >> i) & 1ull)) store8<RT>(P.replicas[i], rep_at(i, j, e), wire, nvalid);
+          if (!((keep >> i) & 1ull)) store8<RT>(P.replicas[i], rep_at(i, j, e), wire, nvalid, tail);
       }
       if constexpr (PH & DRIFT) {
         uint64_t todo = (W == 64 ? ~0ull : ((1ull << W) - 1ull)) & ~own;
@@ -414,7 +415,7 @@ __global__ void __launch_bounds__(kThreads, LOSSY_MIN_BLOCKS) lossy_kernel(const
               ids[b] = __ffsll((long long)todo) - 1;
               todo &= todo - 1;
               nb = b + 1;
-              old[b] = load8_any<RT>(P.replicas[ids[b]], rep_at((uint32_t)ids[b], j, e), nvalid);
+              old[b] = load8_any<RT>(P.replicas[ids[b]], rep_at((uint32_t)ids[b], j, e), nvalid, tail);
             }
           }
 #pragma unroll
@@ -486,16 +487,16 @@ static __global__ void __launch_bounds__(256) closed_loop_grads_kernel(const __g
     const uint64_t e = vi * 8;
     const int nvalid = A.n - e >= 8 ? 8 : (int)(A.n - e);
     float a[8], xs[8];
-    widen<F32>(load8_any<F32>(A.curv, e, nvalid), a);
-    widen<F32>(load8_any<F32>(A.target, e, nvalid), xs);
+    widen<F32>(load8_any<F32>(A.curv, e, nvalid, true), a);
+    widen<F32>(load8_any<F32>(A.target, e, nvalid, true), xs);
     for (uint32_t i0 = 0; i0 < A.W; i0 += 4) {
       Vec8<RT> rep[4];
       Vec8<GT> nz[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u)
         if (i0 + u < A.W) {
-          rep[u] = load8_any<RT>(A.replicas[i0 + u], e, nvalid);
-          nz[u] = load8_any<GT>(A.noise[i0 + u], e, nvalid);
+          rep[u] = load8_any<RT>(A.replicas[i0 + u], e, nvalid, true);
+          nz[u] = load8_any<GT>(A.noise[i0 + u], e, nvalid, true);
         }
 #pragma unroll
       for (int u = 0; u < 4; ++u)
@@ -505,7 +506,7 @@ static __global__ void __launch_bounds__(256) closed_loop_grads_kernel(const __g
 #pragma unroll
           for (int x = 0; x < 8; ++x) g[x] = __fmul_rn(a[x], g[x]);
           add8<GT>(nz[u], g);
-          store8<GT>(A.grads[i0 + u], e, narrow<GT>(g), nvalid);
+          store8<GT>(A.grads[i0 + u], e, narrow<GT>(g), nvalid, true);
         }
     }
   }

@@ -104,3 +104,12 @@ def test_a_broadcast_right_behind_the_optimizer(W, n, P):
 
     a, b = graph_times(lambda: step(False), lambda: step(True))
     assert a <= 1.05 * b, (a, b)
+
+
+@pytest.mark.parametrize("W,n,P", [(60, 74_933, 512)])
+def test_a_bucket_that_ends_inside_eight_elements(W, n, P):
+    """The lane that the end falls into loads and stores its few elements one by one, for every replica; the lanes behind it ran beside it
+    before they skipped every access, and then behind it: broadcast of W = 60 9.0 us, 5.4 of the whole packets, 6.8 as it was."""
+    (ragged, _), (whole, _) = make(W, n, P), make(W, -(-n // P) * P, P)
+    a, b = graph_times(*(lambda x=x: L.lossy_broadcast(x.ctx, 1, x.master, x.replicas, x.stale) for x in (ragged, whole)))
+    assert a <= 1.45 * b, (a, b)
