@@ -512,6 +512,14 @@ int try_gather(lossy_ctx* ctx, Params& P, bool drift, bool rd, cudaStream_t s, u
 // up to five. Two to four workers have a build of their own. Elsewhere the pipelines keep the buckets that the tests of them and of
 // the policy have them serve (tests/test_gpu_small_bucket_policy.py, test_gpu_gather_any_packet.py, test_gpu_parity.py), and with them
 // what lies beyond. Under an eighth of a tile per SM either is a launch and little else (most parity tests are such buckets).
+// Four workers, whole packets that are no multiple of 1024 elements, bf16 replicas, Adam and little loss: the lines for up to four workers
+// lie nearer, at 5.75 tiles per SM instead of 7 (packets from 1024 elements) and 6.75 instead of 11. Pipelines' time over the step kernel's
+// beyond them: p up to 0.05 0.98 (0.91 at the least) and 0.99 (0.86), p from 0.1 1.05 and 1.04; fp32 replicas 1.04-1.09 and 1.06, SGD
+// 1.15 and 1.18, owner-elided replicas 1.14 and 1.10, a short last packet 1.2-1.3 (700 random steps).
+bool four_light(const lossy_config& c) {
+  return c.W == kStepFewWorkers && c.n % c.packet_elems == 0 && c.replica_dtype == LOSSY_BF16 && c.optimizer == LOSSY_ADAM &&
+         !(c.flags & LOSSY_REPLICA_SKIP_OWNER) && fmax(c.p_grad, c.p_param) < 0.075;
+}
 bool small_bucket(const lossy_ctx* ctx, bool drift) {
   const lossy_config& c = ctx->cfg;
   const uint32_t P = c.packet_elems, kTwin = (uint32_t)TmaShape<8>::kTile, kWide = (uint32_t)TmaShape<16>::kTile;
@@ -520,7 +528,7 @@ bool small_bucket(const lossy_ctx* ctx, bool drift) {
   const bool bf16 = c.replica_dtype == LOSSY_BF16, few = c.W <= kStepFewWorkers, short_last = c.n % P != 0;
   if (tiles < 0.125 || P < 128u) return false;
   if (P >= kTwin) {
-    if (few) return tiles >= (short_last ? 0.125 : 0.15) && tiles < (P % kTwin != 0 ? 7.0 : short_last ? 2.0 : 5.0);
+    if (few) return tiles >= (short_last ? 0.125 : 0.15) && tiles < (P % kTwin != 0 ? (four_light(c) ? 5.75 : 7.0) : short_last ? 2.0 : 5.0);
     if (!short_last) return tiles >= (c.W <= 8u ? 0.15 : 0.55) && tiles < (c.W <= 8u ? 1.0 : 2.5) && (tiles < 2.0 || c.W <= 32u || c.p_param < 0.25);
     if (!drift) return false;
     return bf16 ? tiles >= 1.0 && tiles < (P % kTwin == 0 ? 3.6 : 2.0) : tiles < 2.0 && c.W <= 8u;
@@ -596,7 +604,7 @@ GatherPolicy gather_policy(const lossy_ctx* ctx) {
     // (W = 4, P = 200: 0.75 against 0.63).
     const double fill = P / (256.0 * ((P + 255u) / 256u));
     // (the step kernel's build for two to four workers: 1.1-2.1 up to 11 tiles per SM, 0.9-1.3 beyond)
-    const double least = fmax((fill <= 0.6 ? 3.5 : fill <= 0.8 ? 5.0 : fill <= 0.9 ? 6.0 : 8.0) * (c.W > 16u ? 1.6 : 1.0) * (sgd ? 2.2 : 1.0), c.W <= kStepFewWorkers ? 11.0 : 0.0);
+    const double least = fmax((fill <= 0.6 ? 3.5 : fill <= 0.8 ? 5.0 : fill <= 0.9 ? 6.0 : 8.0) * (c.W > 16u ? 1.6 : 1.0) * (sgd ? 2.2 : 1.0), c.W > kStepFewWorkers ? 0.0 : four_light(c) ? 6.75 : 11.0);
     const bool full_lossy = (sgd && fill > 0.98) || (bf16 && ((fill > 0.9 && stale >= 8.0) || (fill > 0.6 && stale >= 12.0)));
     g.wide = c.W >= 5u ? P >= 176u || pm >= 0.15 : c.W == 4u && P >= 256u;
     g.drift_warps = g.wide && gather_geometry<16, true>(ctx, true, G);
