@@ -159,9 +159,19 @@ def _dt(t: torch.dtype) -> int:
 # What a step calls goes through csrc/marshal.cpp. The rest: pointers as integers, a pointer table as the bytes of its entries, the
 # stream's handle without a Stream object around it.
 def _call(name, ctx, *args):
-    rc = _native(load_library().at[name], _NATIVE[name], ctx, *args)
+    lib = load_library()
+    try:
+        rc = _native(lib.at[name], _NATIVE[name], ctx, *args)
+    except (TypeError, OverflowError):
+        rc = _by_ctypes(getattr(lib, name), _NATIVE[name], ctx, args)
     if rc != LOSSY_OK:
         _check(ctx, rc)
+
+
+def _by_ctypes(fn, kinds, ctx, args):
+    """Arguments that marshal.cpp leaves to ctypes: converted as those of the other calls are, taken or refused by fn's signature."""
+    args = iter(args)
+    return fn(ctx, *(_stream() if k == "s" else {"t": _table, "p": _p}.get(k, lambda a: a)(next(args)) for k in kinds))
 
 
 def _p(t):
@@ -271,7 +281,8 @@ class lossy_fused_step_prepared:
                  norms=None, sumsq=None, ghat_prev=None, stream=None):
         lib = load_library()
         self._ctx, self._keep = ctx, (grads, master, m, v, replicas, ghat, count, recv_bits, stale_bits, norms, sumsq, ghat_prev)
-        self._fn = lib.at["lossy_fused_step" if ghat_prev is None else "lossy_fused_step_alg1"]
+        name = "lossy_fused_step" if ghat_prev is None else "lossy_fused_step_alg1"
+        self._fn, self._ctypes_fn = lib.at[name], getattr(lib, name)
         pointers = lambda *ts: tuple(_p(t) or 0 for t in ts)
         head = (_table(grads),) + (() if ghat_prev is None else pointers(ghat_prev))
         self._args = (head + pointers(master, m, v) + (_table(replicas),) + pointers(ghat, count, recv_bits, stale_bits, norms, sumsq)
@@ -279,7 +290,10 @@ class lossy_fused_step_prepared:
         self._kinds = "u" + "".join("b" if isinstance(a, bytes) else "u" for a in self._args) + ("s" if stream is None else "")
 
     def __call__(self, step):
-        rc = _native(self._fn, self._kinds, self._ctx, step, *self._args)
+        try:
+            rc = _native(self._fn, self._kinds, self._ctx, step, *self._args)
+        except (TypeError, OverflowError):      # (its table and pointers are bytes and integers already, which ctypes takes as they are)
+            rc = self._ctypes_fn(self._ctx, step, *self._args, *((_stream(),) if self._kinds[-1] == "s" else ()))
         if rc != LOSSY_OK:
             _check(self._ctx, rc)
 

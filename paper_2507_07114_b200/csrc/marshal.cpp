@@ -1,6 +1,8 @@
 // The binding's calls into the library: tensors to pointers, lists of them to pointer tables, the current stream, the call.
 // A step of a small bucket takes the GPU five microseconds; as Python and ctypes work its arguments took four (four workers)
 // to eight (26) on the host, so that the host was what such a step waited for. Nothing is kept from one call for the next.
+// What an argument is taken as is what ctypes takes it as. The arguments of a usual program are taken here; any other (a ctypes integer, a
+// pointer object, ...) is a TypeError or OverflowError, nothing has been called then, and the binding leaves it to ctypes.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
@@ -18,6 +20,7 @@ namespace {
 constexpr int kMaxArgs = 16, kMaxTables = 4, kTable = 64;
 PyObject* g_data_ptr;   // "data_ptr"
 PyObject* g_value;      // "value"
+PyObject* g_pointer;    // ctypes.c_void_p
 
 bool whole(PyObject* o, uint64_t* out) {   // modulo 2^64, as a C argument of that width takes an integer
   if (!PyLong_Check(o)) {
@@ -40,9 +43,9 @@ bool address(PyObject* o, bool plain, uint64_t* out) {
   }
   PyObject* r = PyObject_CallMethodNoArgs(o, g_data_ptr);
   if (!r) return false;
-  const bool ok = whole(r, out);
+  *out = PyLong_Check(r) ? PyLong_AsUnsignedLongLong(r) : (PyErr_SetString(PyExc_TypeError, "data_ptr() is no integer"), 0);
   Py_DECREF(r);
-  return ok;
+  return !PyErr_Occurred();
 }
 
 bool handle(PyObject* o, uint64_t* out) {   // a ctypes.c_void_p, an integer or None
@@ -51,6 +54,10 @@ bool handle(PyObject* o, uint64_t* out) {   // a ctypes.c_void_p, an integer or 
     return true;
   }
   if (PyLong_Check(o)) return whole(o, out);
+  if (!PyObject_TypeCheck(o, reinterpret_cast<PyTypeObject*>(g_pointer))) {
+    PyErr_Format(PyExc_TypeError, "a c_void_p, an integer or None is wanted, not %.100s", Py_TYPE(o)->tp_name);
+    return false;
+  }
   PyObject* v = PyObject_GetAttr(o, g_value);
   if (!v) return false;
   const bool ok = v == Py_None ? (*out = 0, true) : whole(v, out);
@@ -77,6 +84,7 @@ struct Table {
 };
 
 bool table(PyObject* o, bool plain, Table& t, uint64_t* out) {
+  if (PyObject_Size(o) < 0) return false;      // (what is walked once has no length, and is no table)
   PyObject* seq = PySequence_Fast(o, "a sequence of tensors is wanted");
   if (!seq) return false;
   const Py_ssize_t n = PySequence_Fast_GET_SIZE(seq);
@@ -89,10 +97,10 @@ bool table(PyObject* o, bool plain, Table& t, uint64_t* out) {
     t.few.fill(0);      // (a table that is too short ends in null pointers)
   }
   for (Py_ssize_t i = 0; ok && i < n && i < PySequence_Fast_GET_SIZE(seq); ++i) {   // (an entry's own answer may change the list)
-    PyObject* o = PySequence_Fast_GET_ITEM(seq, i);
-    Py_INCREF(o);
-    ok = address(o, plain, &p[i]);
-    Py_DECREF(o);
+    PyObject* entry = PySequence_Fast_GET_ITEM(seq, i);
+    Py_INCREF(entry);
+    ok = address(entry, plain, &p[i]);
+    Py_DECREF(entry);
   }
   Py_DECREF(seq);
   *out = reinterpret_cast<uint64_t>(p);
@@ -165,6 +173,9 @@ PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "_marshal", nullptr, -1, g_method
 PyMODINIT_FUNC PyInit__marshal() {
   g_data_ptr = PyUnicode_InternFromString("data_ptr");
   g_value = PyUnicode_InternFromString("value");
-  if (!g_data_ptr || !g_value) return nullptr;
+  PyObject* ctypes = PyImport_ImportModule("ctypes");
+  g_pointer = ctypes ? PyObject_GetAttrString(ctypes, "c_void_p") : nullptr;
+  Py_XDECREF(ctypes);
+  if (!g_data_ptr || !g_value || !g_pointer) return nullptr;
   return PyModule_Create(&g_module);
 }
