@@ -8,6 +8,7 @@ CUDA library. There is no fallback: if a shared library is missing, loading rais
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
 import struct
 
@@ -47,7 +48,7 @@ class LossyError(RuntimeError):
 
 
 _lib = None
-_native = None         # _marshal.call
+_native = None         # call of the marshalling module
 # entry points whose arguments csrc/marshal.cpp marshals, and the kinds of the arguments (there); behind the context
 _NATIVE = {
     "lossy_packet_sqnorms": "tps", "lossy_aggregate": "utppps", "lossy_step": "uppppps", "lossy_broadcast": "uptps", "drift_norms": "ptpps",
@@ -136,12 +137,14 @@ def load_library(path: str | None = None) -> C.CDLL:
     lib.lossy_describe_plan.argtypes = [vp, C.c_int, C.c_char_p, C.c_size_t]
     global _native
     if _native is None:
+        marshal = _build.marshal_path()
         try:
-            from . import _marshal
+            spec = importlib.util.spec_from_file_location(__package__ + "._marshal", marshal)
+            module = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(module)
         except ImportError as e:
-            raise FileNotFoundError(f"{os.path.join(os.path.dirname(__file__), '_marshal.so')} is missing or does not load ({e}): run "
-                                    "paper_2507_07114_b200.build.build()") from e
-        _native = _marshal.call
+            raise FileNotFoundError(f"{marshal} is missing or does not load ({e}): run paper_2507_07114_b200.build.build()") from e
+        _native = module.call
     lib.at = {name: C.cast(getattr(lib, name), vp).value for name in _NATIVE}
     if path == default:
         _lib = lib

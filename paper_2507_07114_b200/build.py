@@ -10,7 +10,6 @@ PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "liblossy_b200.so")
 CHECK_LIB_PATH = os.path.join(PKG_DIR, "liblossy_b200_check.so")   # the debug build: -DLOSSY_DEVCHECK (index checks in the kernels)
-MARSHAL_PATH = os.path.join(PKG_DIR, "_marshal.so")
 MARSHAL_SOURCE = os.path.join(CSRC, "marshal.cpp")
 SOURCES = ["lossy_api.cu", "lossy_noalloc.cu"]
 HEADERS = ["lossy_device.cuh", "lossy_kernels.cuh", "lossy_tma.cuh", "lossy_gather.cuh", "lossy_phase_tma.cuh", "lossy_register.cuh", "lossy_diag.cuh", os.path.join("..", "..", "include", "lossy.h")]
@@ -22,11 +21,19 @@ NVCC_FLAGS = [
 ]
 
 
+def marshal_path() -> str:
+    """The binding's marshalling module. It uses the C++ interfaces of one Python and one torch, which its name holds: with others another
+    file is wanted, missing until it is built."""
+    import torch
+
+    return os.path.join(PKG_DIR, f"_marshal-{sysconfig.get_config_var('SOABI')}-torch-{torch.__version__}.so")
+
+
 def _stale(lib: str) -> bool:
     if not os.path.exists(lib):
         return True
     t = os.path.getmtime(lib)
-    deps = ([MARSHAL_SOURCE] if lib == MARSHAL_PATH else [os.path.join(CSRC, s) for s in SOURCES + HEADERS]) + [os.path.abspath(__file__)]
+    deps = ([MARSHAL_SOURCE] if os.path.basename(lib).startswith("_marshal") else [os.path.join(CSRC, s) for s in SOURCES + HEADERS]) + [os.path.abspath(__file__)]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
@@ -44,12 +51,13 @@ def _marshal_command(out: str) -> list:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile liblossy_b200.so, its debug twin liblossy_b200_check.so and the binding's _marshal.so next to this file (the
-    compilers side by side); returns the path of the normal library."""
+    """Compile liblossy_b200.so, its debug twin liblossy_b200_check.so and the binding's marshalling module next to this file
+    (the compilers side by side); returns the path of the normal library."""
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     jobs = []
-    if force or _stale(MARSHAL_PATH):
-        jobs.append((MARSHAL_PATH, subprocess.Popen(_marshal_command(MARSHAL_PATH + ".tmp"), stdout=subprocess.PIPE, stderr=subprocess.PIPE, text=True)))
+    marshal = marshal_path()
+    if force or _stale(marshal):
+        jobs.append((marshal, subprocess.Popen(_marshal_command(marshal + ".tmp"), stdout=subprocess.PIPE, stderr=subprocess.PIPE, text=True)))
     for lib, extra in ((LIB_PATH, []), (CHECK_LIB_PATH, ["-DLOSSY_DEVCHECK=1"])):
         if not force and not _stale(lib):
             continue
