@@ -97,6 +97,7 @@ enum {
 };
 
 #define LOSSY_MAX_WORKERS 64u
+#define LOSSY_PLAN_BUILD 0x100   /* lossy_describe_plan, added to with_drift: name the register kernel's build too */
 
 typedef struct {
   uint32_t W;            /* workers = shards = replicas, 1..64 (the paper's N)           */
@@ -482,8 +483,11 @@ uint64_t lossy_kernel_launches(const lossy_ctx* ctx);
 
 /* lossy_describe_plan — which kernel build lossy_fused_step would launch for the complete packets of
  * this context, as text for logs and benchmarks: "bulk-copy wide|twin group=4|8 stale=late|early|staged
- * [packed] [split] stages=N", or "register kernel" when no bulk-copy build fits (a ragged last packet goes
- * to the register kernel in either case). with_drift != 0 asks for the call that also returns drift norms.
+ * [packed] [split] stages=N", "gather wide|twin packets/tile=N stages=N [drift-warps]", or "register kernel" when
+ * the bucket is small or no pipeline's build fits (a ragged last packet goes to the register kernel in any case).
+ * with_drift != 0 asks for the call that also returns drift norms. With LOSSY_PLAN_BUILD added the register kernel is
+ * "register kernel pairs|quads|few|stale|octs warps=N rounds=N": the build, a block's warps and the chunks that
+ * each of them takes at most.
  * Host only: launches nothing and allocates nothing. Writes at most size bytes including the terminator
  * (truncating); buf is a host buffer owned by the caller. LOSSY_EINVAL for a NULL argument or size 0.
  * The paper has no counterpart: the build choice is this library's measured launch policy. */

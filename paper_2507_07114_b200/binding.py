@@ -21,6 +21,7 @@ LOSSY_F32, LOSSY_BF16 = 0, 1
 LOSSY_SGD, LOSSY_ADAM = 0, 1
 LOSSY_SELF_LOSSLESS, LOSSY_ZERO_SKIP, LOSSY_REGISTER_PATH, LOSSY_REPLICA_SKIP_OWNER, LOSSY_PACKED_BULK = 1, 2, 4, 8, 16
 LOSSY_GATHER_PATH = 32
+LOSSY_PLAN_BUILD = 0x100
 
 EXPORTS = [
     "lossy_init", "lossy_destroy", "lossy_set_lr", "lossy_set_bursty", "lossy_set_reliable", "lossy_packet_sqnorms", "lossy_aggregate", "lossy_step", "lossy_broadcast",
@@ -373,8 +374,9 @@ def lossy_kernel_launches(ctx) -> int:
     return load_library().lossy_kernel_launches(ctx)
 
 
-def lossy_describe_plan(ctx, with_drift: bool = True) -> str:
-    """Text naming the kernel build lossy_fused_step would launch for this context's complete packets."""
+def lossy_describe_plan(ctx, with_drift: bool = True, build: bool = False) -> str:
+    """Text naming the kernel build lossy_fused_step would launch for this context's complete packets. build: of the register kernel
+    its build, a block's warps and their rounds too."""
     buf = C.create_string_buffer(128)
-    _check(ctx, load_library().lossy_describe_plan(ctx, int(with_drift), buf, len(buf)))
+    _check(ctx, load_library().lossy_describe_plan(ctx, int(bool(with_drift)) | (LOSSY_PLAN_BUILD if build else 0), buf, len(buf)))
     return buf.value.decode()

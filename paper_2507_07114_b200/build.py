@@ -12,7 +12,7 @@ LIB_PATH = os.path.join(PKG_DIR, "liblossy_b200.so")
 CHECK_LIB_PATH = os.path.join(PKG_DIR, "liblossy_b200_check.so")   # the debug build: -DLOSSY_DEVCHECK (index checks in the kernels)
 MARSHAL_SOURCE = os.path.join(CSRC, "marshal.cpp")
 SOURCES = ["lossy_api.cu", "lossy_noalloc.cu"]
-HEADERS = ["lossy_device.cuh", "lossy_kernels.cuh", "lossy_tma.cuh", "lossy_gather.cuh", "lossy_phase_tma.cuh", "lossy_register.cuh", "lossy_diag.cuh", os.path.join("..", "..", "include", "lossy.h")]
+HEADERS = ["lossy_divide.h", "lossy_device.cuh", "lossy_kernels.cuh", "lossy_tma.cuh", "lossy_gather.cuh", "lossy_phase_tma.cuh", "lossy_register.cuh", "lossy_diag.cuh", os.path.join("..", "..", "include", "lossy.h")]
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",

@@ -776,6 +776,10 @@ int launch_step(lossy_ctx* ctx, Params& P, cudaStream_t s, uint32_t* blocks_out)
     if (DRIFTK && warps < enough) warps = enough;
   }
   *blocks_out = blocks;
+  if (ctx->plan) {
+    static const char* const kForms[] = {"pairs", "quads", "few", "stale", "octs"};
+    snprintf(ctx->plan, ctx->plan_size, "register kernel %s warps=%u rounds=%u", kForms[FORM], warps, (tasks + blocks * warps - 1u) / (blocks * warps));
+  }
   if (ctx->plan_only) return LOSSY_OK;
   rows_of_call(P, blocks);
   P.chunks_per_packet = per_packet;
@@ -1491,7 +1495,9 @@ int lossy_describe_plan(lossy_ctx* ctx, int with_drift, char* buf, size_t size) 
   ctx->plan = buf;
   ctx->plan_size = size;
   ctx->plan_only = true;             // sizes grids, launches nothing
-  const int rc = run_tma(ctx, P, with_drift != 0, nullptr, &blocks, &used);
+  const bool drift = (with_drift & ~LOSSY_PLAN_BUILD) != 0;
+  int rc = run_tma(ctx, P, drift, nullptr, &blocks, &used);
+  if (!rc && !used && (with_drift & LOSSY_PLAN_BUILD)) rc = drift ? dispatch_step<true>(ctx, P, nullptr, &blocks) : dispatch_step<false>(ctx, P, nullptr, &blocks);
   ctx->plan_only = false;
   ctx->plan = nullptr;
   return rc;

@@ -9,6 +9,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "lossy_divide.h"
+
 namespace lossy {
 
 constexpr int kMaxW = 64;
@@ -111,14 +113,6 @@ __device__ __forceinline__ void begin_beside_previous(const Params& P) {
 __device__ __forceinline__ void end_after_previous(const Params& P) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (blockIdx.x == 0 && threadIdx.x == 0) *P.gate = 0u;   // (a block that has not looked yet will wait)
-}
-
-// x / d for a d that the host knows: the high half of x times 2^64 / d rounded up, exact for every 32-bit x and d (the product is too
-// large by less than x d < 2^64). Two multiply-adds for a division's twenty and more instructions.
-__host__ inline uint64_t magic_of(uint32_t d) { return d > 1u ? ~0ull / d + 1ull : 0ull; }
-__device__ __forceinline__ uint32_t divide_by(uint32_t x, uint32_t d, uint64_t magic) {
-  const uint64_t low = (uint64_t)x * (uint32_t)magic;
-  return d > 1u ? (uint32_t)(((uint64_t)x * (uint32_t)(magic >> 32) + (low >> 32)) >> 32) : x;
 }
 
 // Owner-elided replicas: rep_skip[i] = elements of worker i's shard inside the context's packet range

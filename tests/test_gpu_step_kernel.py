@@ -1,7 +1,5 @@
 """The fused step's register kernel in each of its builds, at the edges of its chunks, rounds and tasks, against the pipelines bit for
-bit (whose parity with the oracle has tests of its own); and its arithmetic of divisions by multiplication, on the CPU."""
-import random
-
+bit (whose parity with the oracle has tests of its own)."""
 import pytest
 import torch
 
@@ -11,31 +9,33 @@ from parity_util import GpuRun, assert_rel, assert_same, run_parity, to_np
 
 SMS = 148
 REG, ELIDE, PACKED, GATHER = L.LOSSY_REGISTER_PATH, L.LOSSY_REPLICA_SKIP_OWNER, L.LOSSY_PACKED_BULK, L.LOSSY_GATHER_PATH
-# W, n, P, p, gradients, replicas, optimizer, further flags. A bucket that ends inside a lane has a task more than chunks.
+# W, n, P, p, gradients, replicas, optimizer, further flags, and the build, a block's warps and their rounds (148 SMs). A bucket that ends
+# inside a lane has a task more than chunks.
 CASES = [
-    (4, SMS * 32 * 128, 1024, 0.1, "f32", "f32", "sgd", 0),                # up to four workers: one full round,
-    (2, SMS * 32 * 128 + 3, 1024, 0.3, "bf16", "bf16", "adam", 0),         # and three elements more, which are a second one
-    (3, 136 * 900 + 1, 136, 0.2, "bf16", "f32", "adam", ELIDE),            # chunks that the packet does not fill
-    (9, 2048 * 40 + 1, 2048, 0.3, "bf16", "bf16", "adam", 0),              # two elements per lane: a lone last one
-    (64, 1024 * 60 + 1023, 1024, 0.3, "f32", "f32", "sgd", 0),             # 64 workers, nineteen stale copies: batches of four
-    (33, 512 * 100, 512, 0.2, "bf16", "bf16", "adam", ELIDE),
-    (17, SMS * 32 * 64, 256, 0.1, "bf16", "f32", "adam", 0),               # the last bucket of one round
-    (8, SMS * 24 * 128, 256, 0.05, "bf16", "bf16", "adam", 0),             # four per lane: one full round,
-    (8, SMS * 24 * 128 + 2, 256, 0.05, "f32", "bf16", "adam", 0),          # and two elements more
-    (16, 736 * 500 + 5, 736, 0.1, "f32", "f32", "sgd", ELIDE),
-    (12, 1024 * 400 + 1022, 1024, 0.3, "bf16", "bf16", "adam", 0),         # eight stale copies at a time
-    (20, 128 * 9000 + 7, 128, 0.3, "bf16", "bf16", "adam", 0),             # eight per lane, half of the lanes, seven behind the last
-    (40, 1024 * 1000, 1024, 0.3, "f32", "bf16", "sgd", ELIDE),
+    (4, SMS * 32 * 128, 1024, 0.1, "f32", "f32", "sgd", 0, "few warps=32 rounds=1"),           # up to four workers: one full round,
+    (2, SMS * 32 * 128 + 3, 1024, 0.3, "bf16", "bf16", "adam", 0, "few warps=17 rounds=2"),    # and three elements more, which are a second one
+    (3, 136 * 900 + 1, 136, 0.2, "bf16", "f32", "adam", ELIDE, "few warps=13 rounds=1"),       # chunks that the packet does not fill
+    (9, 2048 * 40 + 1, 2048, 0.3, "bf16", "bf16", "adam", 0, "pairs warps=9 rounds=1"),        # two elements per lane: a lone last one
+    (64, 1024 * 60 + 1023, 1024, 0.3, "f32", "f32", "sgd", 0, "pairs warps=8 rounds=1"),       # 64 workers, nineteen stale copies: batches of four
+    (33, 512 * 100, 512, 0.2, "bf16", "bf16", "adam", ELIDE, "pairs warps=8 rounds=1"),        # fewer chunks than the norms have warps for
+    (17, SMS * 32 * 64, 256, 0.1, "bf16", "f32", "adam", 0, "pairs warps=32 rounds=1"),        # the last bucket of one round
+    (8, SMS * 24 * 128, 256, 0.05, "bf16", "bf16", "adam", 0, "quads warps=24 rounds=1"),      # four per lane: one full round,
+    (8, SMS * 24 * 128 + 2, 256, 0.05, "f32", "bf16", "adam", 0, "quads warps=13 rounds=2"),   # and two elements more
+    (16, 736 * 500 + 5, 736, 0.1, "f32", "f32", "sgd", ELIDE, "quads warps=11 rounds=2"),
+    (12, 1024 * 400 + 1022, 1024, 0.3, "bf16", "bf16", "adam", 0, "stale warps=22 rounds=1"),  # eight stale copies at a time
+    (20, 128 * 9000 + 7, 128, 0.3, "bf16", "bf16", "adam", 0, "octs warps=16 rounds=4"),       # eight per lane, half of the lanes, seven behind the last
+    (40, 1024 * 1000, 1024, 0.3, "f32", "bf16", "sgd", ELIDE, "octs warps=10 rounds=3"),
 ]
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("case", CASES, ids=["W%d-n%d-P%d-p%g-%s-%s-%s-%d" % c for c in CASES])
+@pytest.mark.parametrize("case", CASES, ids=["W%d-n%d-P%d-p%g-%s-%s-%s-%d" % c[:8] for c in CASES])
 def test_builds_against_the_pipelines(case):
-    W, n, P, p, g, r, opt, flags = case
+    W, n, P, p, g, r, opt, flags, build = case
     w = workload.Workload("step", W, n, P, p, opt, 3e-4, g, r, 2, seed=n % 89)
     a, b = GpuRun(w, flags=flags | REG), GpuRun(w, flags=flags | (PACKED if P >= 1024 else GATHER))
-    assert L.lossy_describe_plan(a.ctx).startswith("register") and not L.lossy_describe_plan(b.ctx).startswith("register")
+    assert L.lossy_describe_plan(a.ctx, build=True) == "register kernel " + build
+    assert L.lossy_describe_plan(a.ctx) == "register kernel" and not L.lossy_describe_plan(b.ctx, build=True).startswith("register")
     for t in (1, 2):
         grads = [workload.grad_slab(w, t, i, 0, n, "cuda") for i in range(W)]
         a.step_fused(t, grads)
@@ -57,16 +57,3 @@ def test_builds_against_the_pipelines(case):
 def test_tiny_buckets_against_the_oracle(W, n, P):
     run_parity(workload.Workload("step_tiny", W, n, P, 0.3, "adam", 3e-4, "bf16", "f32", 3, seed=5), 3, flags=REG)
 
-
-def test_division_by_multiplication():
-    """floor(x m / 2^64) with m = 2^64 / d rounded up, in the two products that the kernel takes, is x / d for 32-bit x and d."""
-    rng = random.Random(3)
-    ds = [2, 3, 7, 64, 641, 2 ** 16 - 1, 2 ** 16 + 1, 2 ** 31, 2 ** 32 - 1] + [rng.randrange(2, 2 ** 32) for _ in range(2000)]
-    for d in ds:
-        m = (2 ** 64 - 1) // d + 1
-        for x in (0, 1, d - 1, d, 2 ** 32 - 1, (2 ** 32 - 1) // d * d, max((2 ** 32 - 1) // d * d - 1, 0), rng.randrange(2 ** 32)):
-            if x >= 2 ** 32:
-                continue
-            low = x * (m & 0xFFFFFFFF)
-            assert ((x * (m >> 32) + (low >> 32)) >> 32) == x // d, (x, d)
-            assert x * (m >> 32) + (low >> 32) < 2 ** 64
