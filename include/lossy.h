@@ -66,10 +66,11 @@ enum {
   /* A packet that received nothing leaves theta, m, v untouched. Default: the
    * estimate is exactly 0 and is fed to the unmodified optimizer. */
   LOSSY_ZERO_SKIP = 2u,
-  /* Every entry point uses the register-path kernel. Default: complete packets go through the
+  /* Every entry point uses the register-path kernels. Default: complete packets go through the
    * bulk-copy (TMA) pipelines (one for the fused step, one per single-phase call) when they hold
    * at least 1024 elements; in the fused step through the gather pipeline instead, from 128 elements
-   * on, where the measured policy favours it (lossy_describe_plan says which build runs). Same
+   * on, or, in small buckets, through the register-path kernel, where the measured policy favours
+   * these (lossy_describe_plan says which build runs). Same
    * parameters, replicas and masks either way; drift sums agree to rounding (another summation
    * order). */
   LOSSY_REGISTER_PATH = 4u,

@@ -1,4 +1,4 @@
-"""B200-native lossy data-parallel step: CUDA library (csrc/) + its ctypes binding."""
+"""B200-native lossy data-parallel step: CUDA library (csrc/) + its binding."""
 from . import build  # noqa: F401
 from .binding import *  # noqa: F401,F403
 from .binding import (EXPORTS, LossyError, drift_norms, drift_norms_static, drift_pairwise, load_library, lossy_aggregate, lossy_aggregate_alg1, lossy_broadcast, lossy_closed_loop_grads,

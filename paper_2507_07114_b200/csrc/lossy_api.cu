@@ -108,13 +108,12 @@ int check_replicas(lossy_ctx* ctx, const void* const* tab) {
 // 9.4 us a step; with a short last packet on a launch of its own (n = 262 184): 20.0 -> 11.4.
 // early = false, an ordinary launch: for kernels that load through L1 and run long. A block that begins early gets what
 // shared memory the kernel ahead has left its SM, after a gather pipeline 28 KB of L1 (closed-loop gradients of 58 M elements
-// behind it: 690 -> 755 us for the pair; packet norms behind the pairwise drift, W = 9, n = 4.6 M: 92 -> 97 us). On small buckets the
-// closed loop's gradients begin early too, and packet norms of very few blocks (closed loop, W = 10, 96 k: 16.4 -> 14.8 us; lines
-// at the calls). The pairwise drift does not: its set kernel loads through the read-only path, which must not run beside the writes of a step ahead, and there is nothing to gain (850 small
-// buckets, behind the memset of the matrix that the call adds to: 0.97 to 1.00 of the ordinary launch's speed).
-// a call's one launch: its blocks' rows are all (two launches: the caller has counted them ahead)
-void rows_of_call(Params& P, uint32_t blocks) { if (P.total_rows == 0u) P.total_rows = blocks; }
-
+// behind it: 690 -> 755 us for the pair; packet norms behind the pairwise drift, W = 9, n = 4.6 M: 92 -> 97 us). And for kernels of which
+// several blocks fit an SM, from a number of blocks on: those that begin early crowd the SMs that come free first. The closed loop's
+// gradients, packet norms and a broadcast begin early up to the numbers at their launches (closed loop, W = 10, 96 k: 16.4 -> 14.8 us).
+// The pairwise drift never does: its set kernel loads through the read-only path, which must not run beside the writes of a step
+// ahead, and there is nothing to gain (850 small buckets, behind the memset of the matrix that the call adds to: 0.97 to 1.00 of the
+// ordinary launch's speed).
 template <class... Formal, class... Actual>
 cudaError_t launch_after(bool early, void (*kern)(Formal...), dim3 grid, uint32_t threads, size_t smem, cudaStream_t s, const Actual&... args) {
   cudaLaunchAttribute at[1] = {};
@@ -132,6 +131,9 @@ cudaError_t launch_after(bool early, void (*kern)(Formal...), dim3 grid, uint32_
   void* argv[] = {const_cast<void*>(static_cast<const void*>(&args))...};
   return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(kern), argv);
 }
+
+// A call's one launch: its blocks' rows are all (two launches: the caller has counted them ahead).
+void rows_of_call(Params& P, uint32_t blocks) { if (P.total_rows == 0u) P.total_rows = blocks; }
 
 // behind a call that failed: a ticketed launch may already be queued, and the counter must be zero again before the next call
 void reset_ticket(lossy_ctx* ctx, cudaStream_t s) {
@@ -506,12 +508,14 @@ int try_gather(lossy_ctx* ctx, Params& P, bool drift, bool rd, cudaStream_t s, u
 }
 
 // Small buckets, of a few tiles (of 2048 elements) per SM, on the step kernel (lossy_register.cuh), which needs no second launch for a
-// short last packet either. Its times against the pipelines' (2000 random steps with drift norms, 2000 without) put the lines
-// further out than they are drawn here: packets from 1024 elements: W <= 4: 1.1 at five tiles per SM (whole packets; short last
-// packets 1.17 at eight), W > 4: 1.0-1.2 at three, 1.3 to 1.6 under one with a short last packet; 128: 1.2-1.5 up to 16; 256 and 512: 1.1-1.4
-// up to five. Two to four workers have a build of their own. Elsewhere the pipelines keep the buckets that the tests of them and of
-// the policy have them serve (tests/test_gpu_small_bucket_policy.py, test_gpu_gather_any_packet.py, test_gpu_parity.py), and with them
-// what lies beyond. Under an eighth of a tile per SM either is a launch and little else (most parity tests are such buckets).
+// short last packet either. The pipelines' time over its own (2000 random steps with drift norms, 2000 without) at the lines below:
+// packets from 1024 elements, whole: W <= 4 1.1-1.2 up to five tiles per SM (no multiple of 1024: 1.1-1.25 up to seven), W > 4 1.0-1.3; with
+// a short last packet: W <= 4 1.2-1.6, W > 4 1.2-1.4; 128 elements: W <= 4 1.1-1.4 at ten tiles, more 1.2-1.5; 256 and 512 1.1-1.5 (1.5-2.0 up to four
+// workers). Two to four workers have a build of their own.
+// The lines are not where these figures end. They leave to the pipelines buckets that have always been theirs and are pinned to them, and
+// on which the step kernel measured faster: W > 4 with whole packets from 1024 elements up to three tiles (1.0-1.2), with a short last packet under one
+// (1.3-1.6) or without drift norms; 128 elements with more than four workers up to 16 tiles (1.2-1.5), 256 and 512 up to five
+// (1.1-1.4); up to four workers and a short last packet up to eight (1.17). And all under an eighth of a tile per SM, which were not measured.
 // Four workers, whole packets that are no multiple of 1024 elements, bf16 replicas, Adam and little loss: the lines for up to four workers
 // lie nearer, at 5.75 tiles per SM instead of 7 (packets from 1024 elements) and 6.75 instead of 11. Pipelines' time over the step kernel's
 // beyond them: p up to 0.05 0.98 (0.91 at the least) and 0.99 (0.86), p from 0.1 1.05 and 1.04; fp32 replicas 1.04-1.09 and 1.06, SGD
@@ -550,6 +554,10 @@ bool small_bucket(const lossy_ctx* ctx, bool drift) {
 // below half a tile per SM up to 1.9; 256 and 512, bf16, two to eight tiles per SM: the register kernel, 1.05-1.2),
 // by 6 % for other packets under 1024 (on the register kernel from two tiles per SM, 1.2, up to 2.2), by 3-5 % for longer
 // ones (under one tile per SM with a short last packet, 1.1-1.2, up to 1.8; multiples of 1024, whole, from two tiles on: none).
+// "The register kernel" of the figures here and in run_tma is the step kernel's predecessor, with chunks of 256 elements. The step kernel is 1.1 to
+// 1.3 times as fast at two to eight tiles per SM and 1.0 to 1.2 beyond, its chunks are of 64 or 128 elements, and only the lines for up
+// to four workers have been drawn against it: the others hand buckets to the pipelines earlier than it would pay, P = 384, 640 and
+// 896 above all, whose chunks of 128 are full where `fill` counts them part empty.
 GatherPolicy gather_policy(const lossy_ctx* ctx) {
   const lossy_config& c = ctx->cfg;
   const double pm = c.p_grad > c.p_param ? c.p_grad : c.p_param;

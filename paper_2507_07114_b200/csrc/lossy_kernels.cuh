@@ -217,12 +217,6 @@ __device__ __forceinline__ void packet_masks(const Params& P, uint32_t k, uint32
     if (P.reliable) stale &= ~P.reliable[(size_t)P.K + k];
   }
 }
-template <int PH>
-__device__ __forceinline__ void packet_masks(const Params& P, uint32_t k, uint32_t j, int lane, uint64_t& recv,
-                                             uint64_t& stale) {
-  uint64_t gbad, pbad;
-  packet_masks<PH>(P, k, j, lane, recv, stale, gbad, pbad);
-}
 
 // The same draws for several packets per ballot (W <= 32, not Algorithm 1's aggregate): the warp's lanes
 // are split into 32 / Wp segments of Wp lanes (Wp = W rounded up to a power of two); a lane evaluates

@@ -110,15 +110,19 @@ __device__ __forceinline__ float lane_squares(const LaneVec<T, EPL>& r, const fl
 // the stores, one block per SM has as many warps as its share of the chunks needs, and everything that can be requested together is:
 // state before the draws, stale copies before the gradients, all of up to 16 gradient pieces before the first sum. With 8 elements
 // per lane, as this kernel's predecessor had, 300 thousand elements gave an SM eight warps; with 2 or 4 they give it 32 or 16, each
-// with the same chain. What is left is instructions in a row (W = 8, 0.5 M elements: 760 per chunk, four cycles each, against 840 with
-// a branch per worker), hence the predicated accesses, divisions by multiplication and both directions' draws at once for W <= 16.
+// with the same chain. What is left is instructions in a row (W = 8, P = 256, 0.45 M elements: 795 warp instructions per chunk, the block's
+// end included, one of a warp's every 17 cycles, the issue slots used to a third), hence the predicated accesses, divisions by
+// multiplication and both directions' draws at once for W <= 16.
 // Steps of 2000 random buckets (us in a graph, mean of the pipelines' or the predecessor's time over this kernel's, by tiles of
 // 2048 elements per SM): W = 2-4: 1.44 under one, 1.6 at two to four, 1.4 to eight, 1.1 to 16; W = 5-8: 1.42, 1.4, 1.13, 1.04; W = 9-16:
-// 1.57, 1.46, 1.27, 1.1; W = 17-32: 1.6, 1.34, 1.15, 1.06; W = 33-64: 1.75, 1.4, 1.22, 1.08. (W = 53, n = 82 k, P = 8192: 16.6 -> 11.5 us.)
+// 1.57, 1.46, 1.27, 1.1; W = 17-32: 1.6, 1.34, 1.15, 1.06; W = 33-64: 1.75, 1.4, 1.22, 1.08.
+// A few thousand elements: 1.4 to 2.1 by workers. (Buckets of tens of rounds that only LOSSY_REGISTER_PATH brings here, W = 5-21, p near 0:
+// 0.93-1.0 of the predecessor, whose eight elements per lane the octs have: 1.01-1.05, but 0.65-0.95 where packets leave chunks part empty.)
 //
-// The builds: two elements per lane, four, four with room for four workers and no more, and four with room for more stale copies.
-// Warps a block may have, gradient pieces, replica stores and stale copies a lane has in flight. Pairs are ahead of quads where they take
-// no more rounds of the chip (W = 33-64, 0.3 tiles per SM: 0.83 of their time; W = 5-8, 1 tile: 1.2). Eight stale copies
+// The builds: two elements per lane, four, four with room for four workers and no more, four with room for more stale copies, and
+// eight. Warps a block may have, gradient pieces, replica stores and stale copies a lane has in flight. (Five of the 144 spill: up to four
+// workers with Adam, fp32 replicas and drift norms, 16 or 20 bytes at 64 registers, and eight elements with bf16 and Adam, 4 bytes.) Pairs are
+// ahead of quads where they take no more rounds of the chip (W = 33-64, 0.3 tiles per SM: 0.83 of their time; W = 5-8, 1 tile: 1.2). Eight stale copies
 // instead of four: 1.04-1.09 from two stale replicas per packet on, 0.9-0.98 below.
 enum StepForm : int { kStepPairs = 0, kStepQuads = 1, kStepFew = 2, kStepStale = 3, kStepOcts = 4 };
 template <class GT, class RT, int FORM> struct StepShape {
