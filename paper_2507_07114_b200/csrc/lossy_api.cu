@@ -516,6 +516,10 @@ int try_gather(lossy_ctx* ctx, Params& P, bool drift, bool rd, cudaStream_t s, u
 // on which the step kernel measured faster: W > 4 with whole packets from 1024 elements up to three tiles (1.0-1.2), with a short last packet under one
 // (1.3-1.6) or without drift norms; 128 elements with more than four workers up to 16 tiles (1.2-1.5), 256 and 512 up to five
 // (1.1-1.4); up to four workers and a short last packet up to eight (1.17). And all under an eighth of a tile per SM, which were not measured.
+// All of this is one stream. A block of the step kernel takes most of an SM, so steps of several streams hardly share one: four
+// streams that each step a bucket of its own (2500 such buckets, all streams' time per step, what they ran on before over the step kernel):
+// W <= 8 1.1-2.4, packets under 1024 elements 1.2-2.4, W = 9-16 with longer ones 1.2 under a tile, 1.0 and 0.95 under two and four, W > 16 with
+// longer ones 0.78-0.9 (0.58 at the least; one stream 1.27-1.45).
 // Four workers, whole packets that are no multiple of 1024 elements, bf16 replicas, Adam and little loss: the lines for up to four workers
 // lie nearer, at 5.75 tiles per SM instead of 7 (packets from 1024 elements) and 6.75 instead of 11. Pipelines' time over the step kernel's
 // beyond them: p up to 0.05 0.98 (0.91 at the least) and 0.99 (0.86), p from 0.1 1.05 and 1.04; fp32 replicas 1.04-1.09 and 1.06, SGD
